@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <map>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 namespace dsrg {
@@ -18,13 +19,17 @@ namespace {
 // exact window: digits are balanced, |d| <= 64, so a level sum over one
 // window has at most 8 pairs x 480 products of |d d'| <= 2^12,
 // 8 x 480 x 4096 < 2^24, and is exact in FP32
-constexpr int OZ_BM = 128, OZ_BK = 16, OZ_NBUF = 4, OZ_WIN = 30;
+constexpr int OZ_BM = 128, OZ_BK = 16, OZ_MAXBUF = 8, OZ_WIN = 30;
 // fewest stages per k split
 constexpr int OZ_SPLIT_MIN = 8;
 // row tiles per rasterisation group
 constexpr int OZ_GROUP = 8;
 constexpr int OZ_THREADS = 256;  // 8 warps: lane quadrant (warp % 4) x column half (warp / 4)
-constexpr int OZ_CTA_THREADS = OZ_THREADS + 32;  // and a ninth warp that issues the bulk copies
+constexpr int OZ_CTA_THREADS = OZ_THREADS + 128;  // and a warpgroup with one warp for the bulk copies and one for the MMAs
+// registers per thread: the block is launched with 384 x 168 (a quarter of
+// them on each sub-partition) and the warpgroups take 208 + 208 + 88 = 3 x 168
+constexpr int OZ_REGS = 168, OZ_REGS_SUM = 208, OZ_REGS_ISSUE = 88;
+static_assert(2 * OZ_REGS_SUM + OZ_REGS_ISSUE == 3 * OZ_REGS, "register split");
 constexpr int OZ_TILE_ELEMS = OZ_BM * OZ_BK;  // A stage tile of one slice: 2048 bf16 = 4 KiB
 constexpr int OZ_TILE_BYTES = OZ_TILE_ELEMS * 2;
 // exponents are stored as 2048 + frexp exponent of the row / column maximum (0: all zero)
@@ -93,6 +98,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t phase, long lo
   }
 }
 
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
@@ -104,6 +113,12 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
                    smem_u32(dst)),
                "l"(src), "r"(bytes), "r"(smem_u32(bar))
                : "memory");
+}
+
+// *p += v without a load of *p into the SM (one addition per element and
+// launch, so the result does not depend on any order)
+__device__ __forceinline__ void red_add(double* p, double v) {
+  asm volatile("red.global.add.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
 }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -118,43 +133,46 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
       : "memory");
 }
 
+// true on one lane of the (converged) warp
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.b32 %0, 1, 0, p;\n}" : "=r"(p));
+  return p != 0;
+}
+
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
 }
 
-#define OZ_R32(a)                                                                                                   \
-  "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]), "=r"(a[8]),      \
-      "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]), "=r"(a[14]), "=r"(a[15]), "=r"(a[16]),        \
-      "=r"(a[17]), "=r"(a[18]), "=r"(a[19]), "=r"(a[20]), "=r"(a[21]), "=r"(a[22]), "=r"(a[23]), "=r"(a[24]),       \
-      "=r"(a[25]), "=r"(a[26]), "=r"(a[27]), "=r"(a[28]), "=r"(a[29]), "=r"(a[30]), "=r"(a[31])
-#define OZ_W32(a)                                                                                                   \
-  "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]), "r"(a[7]), "r"(a[8]), "r"(a[9]),    \
-      "r"(a[10]), "r"(a[11]), "r"(a[12]), "r"(a[13]), "r"(a[14]), "r"(a[15]), "r"(a[16]), "r"(a[17]), "r"(a[18]),   \
-      "r"(a[19]), "r"(a[20]), "r"(a[21]), "r"(a[22]), "r"(a[23]), "r"(a[24]), "r"(a[25]), "r"(a[26]), "r"(a[27]),   \
-      "r"(a[28]), "r"(a[29]), "r"(a[30]), "r"(a[31])
-#define OZ_P32                                                                                                      \
-  "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, " \
-  "%24, %25, %26, %27, %28, %29, %30, %31}"
-#define OZ_Q32                                                                                                      \
-  "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, "     \
-  "%24, %25, %26, %27, %28, %29, %30, %31, %32}"
-
-// 32 consecutive TMEM columns of this thread's lane
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 " OZ_P32 ", [%32];" : OZ_R32(r) : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], " OZ_Q32 ";" ::"r"(taddr), OZ_W32(r) : "memory");
+// 16 consecutive TMEM columns of this thread's lane
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
+      "[%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+__device__ __forceinline__ long long c_offset32(unsigned lin, int nd, const FastDiv* f, const long long* st) {
+  long long o = 0;
+  for (int d = nd - 1; d >= 0; --d) {
+    const unsigned q = fast_div(lin, f[d]);
+    o += (long long)(lin - q * f[d].d) * st[d];
+    lin = q;
+  }
+  return o;
+}
 
 struct OzArgs {
-  const __nv_bfloat16* As;  // [S][MT][KT] tiles
-  const __nv_bfloat16* Bs;  // [S][NT][KT] tiles
+  const __nv_bfloat16* As;  // [MT][KT][S] tiles
+  const __nv_bfloat16* Bs;  // [NT][KT][S] tiles
   const int* ea;            // [MT*128]
-  const int* fb;            // [NT*128]
+  const int* fb;            // [NT*BN]
+  const unsigned* sq;       // [2] largest sum of squared digits of 16 k, A and B
   int S, MT, NT, KT;
   long long M, N;
   double alpha;
@@ -162,14 +180,17 @@ struct OzArgs {
   // C offsets: row m -> decoded with (nM, eM, cM), column n -> (nN, eN, cN)
   int nM, nN;
   int eM[4], eN[4];
+  FastDiv fM[4], fN[4];  // divisors of eM, eN
   long long cM[4], cN[4];
   int rowfast;  // C's row index has the smaller stride (epilogue writes along rows)
   int* status;
   long long wait_cycles;  // budget of each bounded wait (clock cycles)
-  // split over k tiles: CTA z covers [z*ktper, (z+1)*ktper) and writes its
+  // split over k tiles: split z covers [z*ktper, (z+1)*ktper) and writes its
   // scaled partial tile to part[z][MT*128][NT*BN] instead of C
   int splits, ktper;
   double* part;
+  long long tiles;  // MT * NT * splits
+  int nbuf;         // stage buffers
 };
 
 __device__ __forceinline__ long long c_offset(long long lin, int nd, const int* ext, const long long* st) {
@@ -180,44 +201,6 @@ __device__ __forceinline__ long long c_offset(long long lin, int nd, const int* 
     lin = q;
   }
   return o;
-}
-
-// paired FP32 arithmetic on two floats held in one 64-bit register
-__device__ __forceinline__ uint64_t f2_pack(uint32_t a, uint32_t b) {
-  uint64_t d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(a), "r"(b));
-  return d;
-}
-__device__ __forceinline__ void f2_unpack(uint64_t v, uint32_t& a, uint32_t& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=r"(a), "=r"(b) : "l"(v));
-}
-__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-
-// (double)f * 2^k assembled from the bit pattern of the float f (sign,
-// re-biased exponent, mantissa) with integer instructions; zero gives zero and
-// subnormal, non-finite or out-of-range cases take the library path.
-__device__ __forceinline__ double f32_to_f64_scaled(uint32_t u, int k) {
-  if ((u << 1) == 0) return 0.0;
-  const uint32_t ex = (u >> 23) & 0xFFu;
-  const int e = (int)ex - 127 + 1023 + k;
-  if (ex == 0 || ex == 255 || e <= 0 || e >= 2047) return ldexp((double)__uint_as_float(u), k);
-  const unsigned long long bits = ((unsigned long long)(u >> 31) << 63) | ((unsigned long long)e << 52) |
-                                  ((unsigned long long)(u & 0x7FFFFFu) << 29);
-  return __longlong_as_double((long long)bits);
 }
 
 // barrier 1 over the 8 warps of the tile (the copy warp does not take part);
@@ -233,80 +216,158 @@ __device__ __forceinline__ bool tile_sync_and(bool pred) {
   return r != 0;
 }
 
-// Thread 0: every digit pair (t, u), t + u <= S + 1, of one stage into the
-// accumulator of level t + u.  For a fixed A slice t the levels
-// t + 1 .. S + 1 are adjacent in TMEM and the B slices 1 .. S + 1 - t adjacent
-// in shared memory, so one MMA of N = BN (S + 1 - t) columns (pieces of at
-// most 256) covers them and reads A_t once.  The first stage of a window
-// overwrites: the t = 1 MMAs cover every level.  descA0 / descB0 describe
-// the first A / B tile of buffer 0; boff is the buffer's byte offset (the
-// descriptors differ only in the start-address field, bytes / 16).
-template <int BN, int S>
-__device__ __forceinline__ void oz_issue_stage(uint32_t tm, uint64_t descA0, uint64_t descB0, uint32_t boff,
-                                               bool fresh) {
+// Digit pairs (t, u), t + u <= S + 1, of one stage into the accumulators of
+// their levels t + u (one thread), for the A slices t = LO .. HI.  For a fixed
+// t the levels t + 1 .. S + 1 are adjacent in TMEM and the B slices
+// 1 .. S + 1 - t adjacent in shared memory, so one MMA of N = BN (S + 1 - t)
+// columns (pieces of at most 256) covers them and reads A_t once.  FRESH (the
+// first stage of a window): t = 1, whose MMAs cover every level, comes first
+// and overwrites.  Otherwise the slices run downwards, so that a stage ends
+// with its widest MMAs.  dA / dB describe the first A / B tile of the stage's
+// buffer (the descriptors differ only in the start-address field, bytes / 16).
+template <int BN, int S, int LO, int HI, bool FRESH>
+__device__ __forceinline__ void oz_issue(uint32_t tm, uint64_t dA, uint64_t dB) {
   constexpr int B_TILE_BYTES = BN * OZ_BK * 2;
   constexpr int UMAX = 256 / BN;
-  const uint64_t dA = descA0 + (boff >> 4), dB = descB0 + (boff >> 4);
 #pragma unroll
-  for (int t = 1; t <= S; ++t) {
+  for (int i = LO; i <= HI; ++i) {
+    const int t = FRESH ? i : HI - (i - LO);
 #pragma unroll
     for (int u0 = 1; u0 <= S + 1 - t; u0 += UMAX) {
       const int nu = (S + 1 - t) - u0 + 1 < UMAX ? (S + 1 - t) - u0 + 1 : UMAX;
       mma_bf16(tm + (uint32_t)((t + u0 - 2) * BN), dA + (uint64_t)(((t - 1) * OZ_TILE_BYTES) >> 4),
-               dB + (uint64_t)(((u0 - 1) * B_TILE_BYTES) >> 4), oz_idesc(nu * BN), (fresh && t == 1) ? 0u : 1u);
+               dB + (uint64_t)(((u0 - 1) * B_TILE_BYTES) >> 4), oz_idesc(nu * BN), FRESH && t == 1 ? 0u : 1u);
     }
   }
 }
 
-// One CTA: a 128 x BN tile of C.  Warps 0-7: warp w reads TMEM lanes
-// 32 (w % 4) .. and column half w / 4; its thread 0 issues the MMAs.  Warp 8
-// (lane 0) issues the bulk copies.  The k range is walked in stages of 16;
-// four shared-memory buffers rotate: the copy warp refills a buffer as soon
-// as the MMAs of the stage that used it have completed, so copies run up to
-// three stages ahead of the tensor cores, and the MMA thread only waits for
-// data.  Every level c = t + u has its own TMEM accumulator (S levels x BN
-// columns); after every OZ_WIN stages (an exact window) warps 0-7 fold the
-// level sums, scaled by 2^(-7c), into float-float (hi, lo) running sums held
-// in registers.
-template <int BN>
+// tile `lin` of the work list -> (k split z, row tile, column tile).  Grouped
+// rasterisation: consecutive tiles walk the columns of a group of OZ_GROUP row
+// tiles, so the CTAs running together share their digit tiles in L2.
+__device__ __forceinline__ void oz_tile(const OzArgs& a, long long lin, int& z, int& mt, int& nt) {
+  const long long per_z = (long long)a.MT * a.NT;
+  z = (int)(lin / per_z);
+  const long long l = lin - z * per_z;
+  const long long per = (long long)OZ_GROUP * a.NT;
+  const int first = (int)(l / per) * OZ_GROUP;
+  const int gm = a.MT - first < OZ_GROUP ? a.MT - first : OZ_GROUP;
+  const int within = (int)(l - (l / per) * per);
+  mt = first + within % gm;
+  nt = within / gm;
+}
+
+// (top 2^SH + bot) 2^k as a double, assembled with integer instructions and
+// rounded to nearest (bits beyond the 64th are dropped): the FP64 pipe has two
+// lanes a clock, and a conversion or an addition per element would bind it.
+template <int SH>
+__device__ __forceinline__ double oz_value(long long top, long long bot, int k) {
+  // 128-bit two's complement hi:lo = (top << SH) + bot
+  unsigned long long lo = (unsigned long long)top << SH;
+  long long hi = top >> (SH ? 64 - SH : 63);
+  const unsigned long long l2 = lo + (unsigned long long)bot;
+  hi += (bot >> 63) + (l2 < lo ? 1 : 0);
+  lo = l2;
+  const bool neg = hi < 0;
+  if (neg) {
+    lo = 0ULL - lo;
+    hi = ~hi + (lo == 0 ? 1 : 0);
+  }
+  int e = k;
+  unsigned long long m = lo;
+  if (hi) {
+    const int n = __clzll(hi);  // hi >= 0 here, n >= 1
+    m = ((unsigned long long)hi << n) | (lo >> (64 - n));
+    e += 64 - n;
+  } else {
+    if (!lo) return 0.0;
+    const int n = __clzll((long long)lo);
+    m = lo << n;
+    e -= n;
+  }
+  // m in [2^63, 2^64): value m 2^e
+  const unsigned long long r = (m >> 11) + ((m >> 10) & 1ULL);  // in [2^52, 2^53]
+  const int ex = e + 63 + 1023;
+  if (ex <= 0 || ex >= 2046) {  // subnormal or out of range: scaled in exact steps but the last
+    double v = (double)(neg ? -(long long)r : (long long)r);
+    for (int s = e + 11; s != 0;) {
+      const int t = s > 1000 ? 1000 : s < -1000 ? -1000 : s;
+      v *= __longlong_as_double((long long)(t + 1023) << 52);
+      s -= t;
+    }
+    return v;
+  }
+  const unsigned long long bits = ((unsigned long long)(ex - 1) << 52) + r;  // the leading bit of r adds one to ex - 1
+  return __longlong_as_double((long long)(bits | (neg ? 1ULL << 63 : 0ULL)));
+}
+
+// Bounded wait that also gives up once another role of the CTA has.
+__device__ __forceinline__ bool oz_wait(uint64_t* bar, uint32_t phase, long long budget, volatile int* stop) {
+  if (mbar_test(bar, phase)) return true;
+  const long long t0 = clock64();
+  while (true) {
+    if (clock64() - t0 > budget || *stop) {
+      *stop = 1;
+      return false;
+    }
+    if (mbar_try(bar, phase)) return true;
+  }
+}
+
+constexpr int OZ_EPC = 8;                  // columns per warp staged at a time in the epilogue
+constexpr int OZ_STAGE_LD = OZ_EPC + 1;    // padded against bank conflicts
+constexpr int OZ_STAGE_BYTES = (OZ_THREADS / 32) * 32 * OZ_STAGE_LD * 8;
+
+// Stages per exact window: the level sums over the window must stay within
+// 2^24.  With m the largest sum of squared digits (all slices) over any row's
+// 16 k of an operand (oz_digits measures it), a level sum over one stage, and
+// any part of it, is at most sqrt(mA mB) by Cauchy and Schwarz, once over k
+// and once over the digit pairs of the level.  Digits of real data are spread
+// over [-64, 64], about a third of the square of the largest, so windows are
+// about 2.5 times as long as the OZ_WIN stages that hold for any digits.
+__device__ __forceinline__ int oz_window(const OzArgs& a) {
+  const float p = sqrtf((float)a.sq[0]) * sqrtf((float)a.sq[1]);
+  const float w = 16777216.0f * 0.9999f / fmaxf(p, 1.0f);
+  const int n = (int)fminf(w, 1048576.0f);
+  return n > OZ_WIN ? n : OZ_WIN;
+}
+
+// Persistent CTAs: each walks the 128 x BN tiles of C (and k splits)
+// blockIdx.x, blockIdx.x + gridDim.x, ...  Three roles run concurrently:
+//  * warp 8 (lane 0) issues two bulk copies per 16-k stage (the S digit tiles
+//    of A and of B are contiguous) into a ring of nbuf buffers;
+//  * warp 9 (lane 0) issues the stage's MMAs as soon as its data are there;
+//  * warps 0-7 (warp w: TMEM lanes 32 (w % 4) .., column half w / 4) take the
+//    level sums of every exact window (oz_window) out of TMEM into two 64-bit
+//    integers per element, then write the tile while the next tile's MMAs run.
+// Every level c = t + u has its own TMEM accumulator (S levels x BN columns);
+// a window's level sums are exact integers below 2^24 in FP32, so the integer
+// sums are exact: top = levels 2 .. CT + 1 in units of 2^(-7 (CT + 1)), bot =
+// the rest in units of 2^(-7 (S + 1)).
+// Bound: the tensor pipe.  One CTA per tile with the fold in float-float and
+// 2 S copies per stage took 24.3 / 26.6 ms at 8192^3 (6 / 7 slices): 25 ms
+// of it were the copies alone (14 copies of 2-4 KB a stage), 21 ms the MMAs
+// alone (a shared issue thread).  Now 11.0 / 14.4 ms, 2090 / 2140 TFLOP/s
+// executed (above the measured bf16 burst rate of a library GEMM); 4096^3 at 8
+// slices 4.2 -> 2.4 ms.  11236 x 256 x 36 (2.3 tiles a CTA, 3 stages each): 50 us,
+// bound by the latency of a tile's set-up, sums and write.
+template <int BN, int S>
 __global__ void __launch_bounds__(OZ_CTA_THREADS, 1) k_ozaki_mma(const OzArgs a) {
-  constexpr uint32_t TMEM_COLS = 512;  // S <= 8 level accumulators of BN <= 64 columns
+  constexpr uint32_t TMEM_COLS = 512;
   constexpr int B_TILE_BYTES = BN * OZ_BK * 2;
-  // columns per warp in the fold and epilogue: two column halves for BN >= 64;
-  // for BN = 32 the second half of the warps sits out
-  constexpr int HALF = BN >= 64 ? BN / 2 : BN;
-  constexpr int NCH = HALF / 32;
-  static_assert(8 * BN <= (int)TMEM_COLS, "TMEM columns");
+  constexpr int STAGE_BYTES = S * (OZ_TILE_BYTES + B_TILE_BYTES);
+  constexpr int HALF = BN / 2;               // columns per warp
+  constexpr int CH = 16, NCH = HALF / CH;    // TMEM columns per load
+  constexpr int CT = (S + 1) / 2, SH = 7 * (S - CT);  // levels in top; unit of top over that of bot
+  static_assert(S * BN <= (int)TMEM_COLS && HALF % CH == 0, "tile");
   extern __shared__ unsigned char oz_smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)oz_smem_raw + 1023) & ~(uintptr_t)1023);
-  __shared__ uint64_t bar_load[OZ_NBUF], bar_mma[OZ_NBUF], bar_win;
+  __shared__ uint64_t bar_full[OZ_MAXBUF], bar_free[OZ_MAXBUF], bar_acc, bar_read, bar_drain;
   __shared__ uint32_t tmem_base;
   __shared__ long long colC[BN], rowC[OZ_BM];
-  __shared__ int colE[BN];
-  __shared__ int issued[OZ_NBUF];  // copies issued per buffer (copy warp), read at the end
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const bool copier = warp == OZ_THREADS / 32;
-  const int quad = warp & 3, half = (warp >> 2) & 1;  // TMEM lanes 32*quad.., columns half*HALF..
-  const int row = quad * 32 + (tid & 31);
-  // grouped rasterisation: consecutive CTAs walk the column tiles of a group
-  // of OZ_GROUP row tiles, so the CTAs running together share their A and B
-  // digit tiles in L2
-  int mt, nt;
-  {
-    const int lin = blockIdx.y * a.MT + blockIdx.x;
-    const int per = OZ_GROUP * a.NT;
-    const int first = (lin / per) * OZ_GROUP;
-    const int gm = a.MT - first < OZ_GROUP ? a.MT - first : OZ_GROUP;
-    const int within = lin - (lin / per) * per;
-    mt = first + within % gm;
-    nt = within / gm;
-  }
-  const int z = blockIdx.z;
-  const int kt0 = a.splits > 1 ? z * a.ktper : 0;
-  const int kt1 = a.splits > 1 ? (kt0 + a.ktper < a.KT ? kt0 + a.ktper : a.KT) : a.KT;
-  const int S = a.S;
-  const size_t stage_bytes = (size_t)S * (OZ_TILE_BYTES + B_TILE_BYTES);
-  const int ns = kt1 - kt0;
+  __shared__ int colE[BN], rowE[OZ_BM];
+  __shared__ volatile int stop;  // a bounded wait ran out
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nbuf = a.nbuf;
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
@@ -315,208 +376,208 @@ __global__ void __launch_bounds__(OZ_CTA_THREADS, 1) k_ozaki_mma(const OzArgs a)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
-    for (int i = 0; i < OZ_NBUF; ++i) {
-      mbar_init(&bar_load[i], 1);
-      mbar_init(&bar_mma[i], 1);
-      issued[i] = 0;
+    for (int i = 0; i < nbuf; ++i) {
+      mbar_init(&bar_full[i], 1);
+      mbar_init(&bar_free[i], 1);
     }
-    mbar_init(&bar_win, 1);
+    mbar_init(&bar_acc, 1);
+    mbar_init(&bar_read, OZ_THREADS / 32);
+    mbar_init(&bar_drain, 1);
+    stop = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  for (int t = tid; t < BN; t += OZ_CTA_THREADS) {
-    long long n = (long long)nt * BN + t;
-    colC[t] = n < a.N ? c_offset(n, a.nN, a.eN, a.cN) : -1;
-    colE[t] = a.fb[(long long)nt * BN + t] - (int)OZ_EBIAS;
-  }
-  for (int t = tid; t < OZ_BM; t += OZ_CTA_THREADS) {
-    long long m = (long long)mt * OZ_BM + t;
-    rowC[t] = m < a.M ? c_offset(m, a.nM, a.eM, a.cM) : -1;
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tm = tmem_base;
-  // matrix descriptors of the first A and B digit tiles of buffer 0; the
-  // others differ only in the start-address field (byte offset / 16)
-  const uint64_t descA0 = sdesc(smem_u32(smem));
-  const uint64_t descB0 = sdesc(smem_u32(smem + (size_t)S * OZ_TILE_BYTES));
 
-  // ---- copy warp: stage k (relative to kt0) into buffer k % OZ_NBUF, once
-  // the MMAs of stage k - OZ_NBUF (the buffer's last use) have completed
-  if (copier) {
-    if ((tid & 31) == 0) {
-      uint32_t ph_mma[OZ_NBUF] = {};
-      for (int k = 0; k < ns; ++k) {
-        const int b = k % OZ_NBUF, kt = kt0 + k;
-        if (k >= OZ_NBUF) {
-          if (!mbar_wait(&bar_mma[b], ph_mma[b], a.wait_cycles)) break;  // the MMA thread stopped
-          ph_mma[b] ^= 1;
+  if (warp >= OZ_THREADS / 32) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(OZ_REGS_ISSUE));
+    if (warp == OZ_THREADS / 32 && lane == 0) {
+      // ---- copies
+      int b = 0;
+      uint32_t lap = 0;  // times the ring has been walked
+      bool ok = true;
+      for (long long lin = blockIdx.x; ok && lin < a.tiles; lin += gridDim.x) {
+        int z, mt, nt;
+        oz_tile(a, lin, z, mt, nt);
+        const int kt0 = z * a.ktper, kt1 = kt0 + a.ktper < a.KT ? kt0 + a.ktper : a.KT;
+        const __nv_bfloat16* pa = a.As + ((size_t)mt * a.KT + kt0) * (S * OZ_TILE_ELEMS);
+        const __nv_bfloat16* pb = a.Bs + ((size_t)nt * a.KT + kt0) * (S * BN * OZ_BK);
+        for (int kt = kt0; kt < kt1; ++kt, pa += S * OZ_TILE_ELEMS, pb += S * BN * OZ_BK) {
+          // the MMAs of the buffer's last use have completed
+          if (lap > 0 && !oz_wait(&bar_free[b], (lap - 1) & 1, a.wait_cycles, &stop)) {
+            ok = false;
+            break;
+          }
+          unsigned char* base = smem + (size_t)b * STAGE_BYTES;
+          mbar_expect_tx(&bar_full[b], (uint32_t)STAGE_BYTES);
+          bulk_g2s(base, pa, S * OZ_TILE_BYTES, &bar_full[b]);
+          bulk_g2s(base + S * OZ_TILE_BYTES, pb, S * B_TILE_BYTES, &bar_full[b]);
+          if (++b == nbuf) {
+            b = 0;
+            ++lap;
+          }
         }
-        unsigned char* base = smem + (size_t)b * stage_bytes;
-        mbar_expect_tx(&bar_load[b], (uint32_t)(S * (OZ_TILE_BYTES + B_TILE_BYTES)));
-        for (int s2 = 0; s2 < S; ++s2) {
-          bulk_g2s(base + (size_t)s2 * OZ_TILE_BYTES, a.As + ((size_t)(s2 * a.MT + mt) * a.KT + kt) * OZ_TILE_ELEMS,
-                   OZ_TILE_BYTES, &bar_load[b]);
-          bulk_g2s(base + (size_t)S * OZ_TILE_BYTES + (size_t)s2 * B_TILE_BYTES,
-                   a.Bs + ((size_t)(s2 * a.NT + nt) * a.KT + kt) * (BN * OZ_BK), B_TILE_BYTES, &bar_load[b]);
-        }
-        issued[b] += 1;
+      }
+      // before the shared memory is released every copy issued has landed
+      // (with the fixed default budget; immediate unless a wait ran out)
+      for (int i = 0; i < nbuf; ++i) {
+        const uint32_t n = lap + (i < b ? 1u : 0u);  // copies issued into buffer i
+        if (n > 0) mbar_wait(&bar_full[i], (n - 1) & 1, OZ_WAIT_CYCLES);
       }
     }
-  }
-
-  // ---- warps 0-7: MMAs (thread 0), folds, epilogue
-  const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
-  const uint32_t col0 = (uint32_t)(half * HALF);
-  const bool active = !copier && (BN >= 64 || half == 0);
-  uint32_t rhi[NCH][32], rlo[NCH][32];
-#pragma unroll
-  for (int j = 0; j < NCH; ++j)
-#pragma unroll
-    for (int q = 0; q < 32; ++q) rhi[j][q] = rlo[j][q] = 0u;
-  bool ok = true;
-  int consumed[OZ_NBUF] = {};                  // thread 0: loads waited for per buffer
-  uint32_t ph_load[OZ_NBUF] = {}, ph_win = 0;  // thread 0 / every tile thread
-  bool win_pending = false;                    // thread 0
-  if (!copier) {
-    for (int k = 0; k < ns; ++k) {
-      const int b = k % OZ_NBUF;
-      const bool fresh = (k % OZ_WIN) == 0;
-      const bool wend = (k % OZ_WIN) == OZ_WIN - 1 || k == ns - 1;
-      if (tid == 0) {
-        if (ok) {
-          if (mbar_wait(&bar_load[b], ph_load[b], a.wait_cycles)) {
-            ph_load[b] ^= 1;
-            consumed[b] += 1;
-          } else {
+    if (warp == OZ_THREADS / 32 + 1) {
+      // ---- MMAs (the whole warp walks the stages, one elected lane issues)
+      const uint64_t descA0 = sdesc(smem_u32(smem)), descB0 = sdesc(smem_u32(smem + S * OZ_TILE_BYTES));
+      const int window = oz_window(a);
+      int b = 0;                     // buffer of the next stage
+      uint32_t ph = 0, win = 0;      // its phase; windows issued
+      uint64_t dA = descA0, dB = descB0;
+      bool there = false;            // its data are known to be there
+      // one stage.  The tensor queue holds only a few MMAs, so the next
+      // stage's barrier is tested between this stage's, and the stage ends
+      // with wide ones: bookkeeping behind narrow ones left the pipe idle
+      // (8192^3: 13.4 -> 11.8 ms at 6 slices, 15.9 -> 14.9 ms at 7)
+      auto stage = [&](auto fresh) {
+        constexpr bool FRESH = decltype(fresh)::value;
+        constexpr int MID = S > 2 ? 2 : S;  // A slices 1 .. MID are the wide half
+        if (!there && !__all_sync(0xffffffffu, oz_wait(&bar_full[b], ph, a.wait_cycles, &stop))) return false;
+        uint64_t* const free = &bar_free[b];
+        const uint64_t cA = dA, cB = dB;
+        if (++b == nbuf) {
+          b = 0;
+          ph ^= 1;
+        }
+        dA = descA0 + (uint64_t)((uint32_t)(b * STAGE_BYTES) >> 4);
+        dB = descB0 + (uint64_t)((uint32_t)(b * STAGE_BYTES) >> 4);
+        if (elect_one()) {
+          if (FRESH) oz_issue<BN, S, 1, MID, FRESH>(tm, cA, cB);
+          else oz_issue<BN, S, MID + 1, S, FRESH>(tm, cA, cB);
+        }
+        const bool next = mbar_test(&bar_full[b], ph);
+        if (elect_one()) {
+          if (FRESH) oz_issue<BN, S, MID + 1, S, FRESH>(tm, cA, cB);
+          else oz_issue<BN, S, 1, MID, FRESH>(tm, cA, cB);
+          mma_commit(free);  // the buffer is free once these complete
+        }
+        there = __all_sync(0xffffffffu, next);
+        return true;
+      };
+      bool ok = true;
+      for (long long lin = blockIdx.x; ok && lin < a.tiles; lin += gridDim.x) {
+        const int z = (int)(lin / ((long long)a.MT * a.NT));
+        const int kt0 = z * a.ktper;
+        int left = (kt0 + a.ktper < a.KT ? kt0 + a.ktper : a.KT) - kt0;
+        while (ok && left > 0) {
+          // the last window's level sums have been read
+          if (win > 0 && !__all_sync(0xffffffffu, oz_wait(&bar_read, (win - 1) & 1, a.wait_cycles, &stop))) {
             ok = false;
+            break;
           }
-        }
-        if (ok) {
           tc_fence_after();
-          switch (S) {
-            case 1: oz_issue_stage<BN, 1>(tm, descA0, descB0, (uint32_t)(b * stage_bytes), fresh); break;
-            case 2: oz_issue_stage<BN, 2>(tm, descA0, descB0, (uint32_t)(b * stage_bytes), fresh); break;
-            case 3: oz_issue_stage<BN, 3>(tm, descA0, descB0, (uint32_t)(b * stage_bytes), fresh); break;
-            case 4: oz_issue_stage<BN, 4>(tm, descA0, descB0, (uint32_t)(b * stage_bytes), fresh); break;
-            case 5: oz_issue_stage<BN, 5>(tm, descA0, descB0, (uint32_t)(b * stage_bytes), fresh); break;
-            case 6: oz_issue_stage<BN, 6>(tm, descA0, descB0, (uint32_t)(b * stage_bytes), fresh); break;
-            case 7: oz_issue_stage<BN, 7>(tm, descA0, descB0, (uint32_t)(b * stage_bytes), fresh); break;
-            default: oz_issue_stage<BN, 8>(tm, descA0, descB0, (uint32_t)(b * stage_bytes), fresh); break;
-          }
-          mma_commit(&bar_mma[b]);  // the buffer is free once these complete
-        }
-        if (wend) {  // completes once every MMA issued so far has completed
-          mma_commit(&bar_win);
-          win_pending = true;
+          const int n = left < window ? left : window;
+          left -= n;
+          ok = stage(std::true_type{});
+          for (int i = 1; ok && i < n; ++i) ok = stage(std::false_type{});
+          if (ok && elect_one()) mma_commit(&bar_acc);  // completes once every MMA issued so far has
+          ++win;
         }
       }
-      if (!wend) continue;
-      const bool w = mbar_wait(&bar_win, ph_win, a.wait_cycles);
-      if (w) ph_win ^= 1;
-      if (tid == 0 && w) win_pending = false;
-      ok = tile_sync_and(ok && w);
-      tc_fence_after();
-      if (!ok) break;
-      // fold the window: (hi, lo) += acc_c * 2^(-7c), two-sum in paired FP32
-      if (active) {
-        for (int c = 2; c <= S + 1; ++c) {
-          const float scale = exp2f(-7.0f * (float)c);
-          const uint64_t sc2 = f2_pack(__float_as_uint(scale), __float_as_uint(scale));
+      // every MMA issued has completed before TMEM is released
+      __syncwarp();
+      if (elect_one()) mma_commit(&bar_drain);
+      mbar_wait(&bar_drain, 0, OZ_WAIT_CYCLES);
+    }
+    __syncwarp();
+  } else {
+    // ---- level sums and C
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(OZ_REGS_SUM));
+    const int quad = warp & 3, half = warp >> 2;
+    const int row = quad * 32 + lane;
+    const uint32_t taddr = tm + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * HALF);
+    double* stg = reinterpret_cast<double*>(smem + (size_t)nbuf * STAGE_BYTES) + warp * 32 * OZ_STAGE_LD;
+    uint32_t win = 0;
+    const int window = oz_window(a);
+    for (long long lin = blockIdx.x; lin < a.tiles; lin += gridDim.x) {
+      int z, mt, nt;
+      oz_tile(a, lin, z, mt, nt);
+      const int kt0 = z * a.ktper;
+      const int ns = (kt0 + a.ktper < a.KT ? kt0 + a.ktper : a.KT) - kt0;
+      const int nwin = (ns + window - 1) / window;
+      tile_sync();  // the last tile's tables are no longer read
+      if (tid < BN) {
+        const long long n = (long long)nt * BN + tid;
+        if (a.splits > 1) colC[tid] = n;
+        else colC[tid] = n < a.N ? c_offset32((unsigned)n, a.nN, a.fN, a.cN) : -1;
+        colE[tid] = a.fb[n] - (int)OZ_EBIAS;
+      } else if (tid >= OZ_THREADS - OZ_BM) {
+        const int t = tid - (OZ_THREADS - OZ_BM);
+        const long long m = (long long)mt * OZ_BM + t;
+        if (a.splits > 1) rowC[t] = ((long long)z * a.MT * OZ_BM + m) * ((long long)a.NT * BN);
+        else rowC[t] = m < a.M ? c_offset32((unsigned)m, a.nM, a.fM, a.cM) : -1;
+        rowE[t] = a.ea[m] - (int)OZ_EBIAS;
+      }
+      long long top[NCH][CH], bot[NCH][CH];
+#pragma unroll
+      for (int j = 0; j < NCH; ++j)
+#pragma unroll
+        for (int q = 0; q < CH; ++q) top[j][q] = bot[j][q] = 0;
+      bool ok = true;
+      for (int w = 0; w < nwin; ++w, ++win) {
+        // one thread polls, the others sleep at the barrier: polling by all
+        // eight warps slowed the MMA warp's issue
+        if (tid == 0) ok = oz_wait(&bar_acc, win & 1, a.wait_cycles, &stop);
+        ok = tile_sync_and(ok);
+        if (!ok) break;
+        tc_fence_after();
+#pragma unroll
+        for (int c = 0; c < S; ++c) {
 #pragma unroll
           for (int j = 0; j < NCH; ++j) {
-            uint32_t acc[32];
-            tmem_ld32(tm + lane_off + (uint32_t)((c - 2) * BN) + col0 + 32 * j, acc);
+            uint32_t acc[CH];
+            tmem_ld16(taddr + (uint32_t)(c * BN + j * CH), acc);
             tmem_wait_ld();
 #pragma unroll
-            for (int q = 0; q < 32; q += 2) {
-              const uint64_t x = f2_mul(f2_pack(acc[q], acc[q + 1]), sc2);
-              const uint64_t h = f2_pack(rhi[j][q], rhi[j][q + 1]);
-              const uint64_t s_ = f2_add(h, x);
-              const uint64_t bp = f2_sub(s_, h);
-              const uint64_t err = f2_add(f2_sub(h, f2_sub(s_, bp)), f2_sub(x, bp));
-              uint64_t l = f2_add(f2_pack(rlo[j][q], rlo[j][q + 1]), err);
-              const uint64_t s2 = f2_add(s_, l);
-              l = f2_sub(l, f2_sub(s2, s_));
-              f2_unpack(s2, rhi[j][q], rhi[j][q + 1]);
-              f2_unpack(l, rlo[j][q], rlo[j][q + 1]);
+            for (int q = 0; q < CH; ++q) {
+              const int v = __float2int_rn(__uint_as_float(acc[q]));
+              if (c < CT) top[j][q] += (long long)v * (1 << (7 * (CT - 1 - c)));
+              else bot[j][q] += (long long)v * (1 << (7 * (S - 1 - c)));
             }
           }
         }
+        // the accumulators are read; the next window may overwrite them
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bar_read);
       }
-      // the accumulators are read; the next window may overwrite them
-      tc_fence_before();
-      tile_sync();
-      tc_fence_after();
-    }
-  }
-  // every warp: the copy warp's count of issued copies is visible after this
-  __syncthreads();
-  // after a timed-out wait: wait once more (the fixed default budget) for
-  // copies issued but not consumed and for every MMA issued, before the
-  // shared memory and TMEM are released
-  if (!ok && tid == 0) {
-    for (int i = 0; i < OZ_NBUF; ++i)
-      if (issued[i] > consumed[i]) mbar_wait(&bar_load[i], ph_load[i], OZ_WAIT_CYCLES);
-    if (win_pending) mbar_wait(&bar_win, ph_win, OZ_WAIT_CYCLES);
-  }
-  // epilogue: the scaled tile 2^(ea[m] + fb[n]) (hi + lo) goes to shared
-  // memory (the stage buffers are free once the last MMA has completed and
-  // every copy was consumed; rows padded by one double against bank
-  // conflicts), then consecutive threads write consecutive columns of C
-  // (alpha times, accumulated) or of the split-k partial part[z]
-  constexpr int LDT = BN + 1;
-  double* stile = reinterpret_cast<double*>(smem);
-  if (ok && active) {
-    const int em = a.ea[(long long)mt * OZ_BM + row] - (int)OZ_EBIAS;
+      if (!tile_sync_and(ok)) break;  // and the tables are written
+      // 2^(ea[m] + fb[n] + 2 - 7 (S + 1)) (top 2^SH + bot), OZ_EPC columns at
+      // a time through this warp's staging rows, so that consecutive lanes
+      // touch consecutive elements of C (or of the split-k partial)
+      const int em = rowE[row] + 2 - 7 * (S + 1);
 #pragma unroll
-    for (int j = 0; j < NCH; ++j) {
-      const int cc = (int)col0 + 32 * j;
+      for (int j = 0; j < NCH; ++j) {
 #pragma unroll
-      for (int q = 0; q < 32; ++q) {
-        const int k = em + colE[cc + q] + 2;  // x = 2^(e + 1) sum_t d_t 2^(-7t) on both sides
-        stile[row * LDT + cc + q] = f32_to_f64_scaled(rhi[j][q], k) + f32_to_f64_scaled(rlo[j][q], k);
-      }
-    }
-  }
-  __syncthreads();
-  if (ok && !copier) {
-    if (a.splits > 1) {
-      const long long ldp = (long long)a.NT * BN;
-      double* pz = a.part + ((long long)z * a.MT * OZ_BM + (long long)mt * OZ_BM) * ldp + (long long)nt * BN;
-      for (int i = tid; i < OZ_BM * BN; i += OZ_THREADS) {
-        const int r = i / BN, c = i - r * BN;
-        const bool live = (long long)mt * OZ_BM + r < a.M && colC[c] >= 0;
-        pz[(long long)r * ldp + c] = live ? stile[r * LDT + c] : 0.0;
-      }
-    } else {
-      // eight read-modify-writes per thread with all loads issued first;
-      // consecutive threads on C's contiguous index (rows when rowfast)
-      constexpr int U = 8;
-      static_assert((OZ_BM * BN) % (U * OZ_THREADS) == 0, "epilogue tiling");
-      for (int base = 0; base < OZ_BM * BN; base += U * OZ_THREADS) {
-        long long off[U];
-        double cv[U], tv[U];
+        for (int g = 0; g < CH / OZ_EPC; ++g) {
+          const int c0 = half * HALF + j * CH + g * OZ_EPC;
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int i = base + u * OZ_THREADS + tid;
-          int r, c;
-          if (a.rowfast) {
-            c = i / OZ_BM;
-            r = i - c * OZ_BM;
-          } else {
-            r = i / BN;
-            c = i - r * BN;
+          for (int q = 0; q < OZ_EPC; ++q)
+            stg[lane * OZ_STAGE_LD + q] =
+                oz_value<SH>(top[j][g * OZ_EPC + q], bot[j][g * OZ_EPC + q], em + colE[c0 + q]);
+          __syncwarp();
+          double* const out = a.splits > 1 ? a.part : a.C;
+#pragma unroll
+          for (int u = 0; u < OZ_EPC; ++u) {
+            const int i = u * 32 + lane;
+            const int r = a.rowfast ? lane : i / OZ_EPC, c = a.rowfast ? u : i % OZ_EPC;
+            const long long oc = colC[c0 + c], orow = rowC[quad * 32 + r];
+            const double t = stg[r * OZ_STAGE_LD + c];
+            if (a.splits > 1) out[orow + oc] = t;
+            else if (oc >= 0 && orow >= 0) red_add(out + orow + oc, a.alpha * t);
           }
-          const long long oc = colC[c], orow = rowC[r];
-          off[u] = oc >= 0 && orow >= 0 ? orow + oc : -1;
-          tv[u] = stile[r * LDT + c];
+          __syncwarp();
         }
-#pragma unroll
-        for (int u = 0; u < U; ++u) cv[u] = off[u] >= 0 ? a.C[off[u]] : 0.0;
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (off[u] >= 0) a.C[off[u]] = cv[u] + a.alpha * tv[u];
       }
     }
   }
@@ -524,7 +585,7 @@ __global__ void __launch_bounds__(OZ_CTA_THREADS, 1) k_ozaki_mma(const OzArgs a)
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm), "r"(TMEM_COLS)
                               : "memory");
-  if (!ok && tid == 0) atomicExch(a.status ? a.status : &g_oz_status, 1);
+  if (stop && tid == 0) atomicExch(a.status ? a.status : &g_oz_status, 1);
 }
 
 // C[m, n] += alpha * sum_z part[z][m][n] (z in order)
@@ -688,6 +749,7 @@ struct PackPass {
   int kfast[2];
   FastDiv fQ[2], fR[2];
   unsigned W[2];
+  unsigned* sq;  // [2] (pass 2)
 };
 
 // Each CTA walks one contiguous range of work items, 256 at a time, and each
@@ -743,9 +805,9 @@ __global__ void __launch_bounds__(PACK_T) k_ozaki_rowexp(const PackPass pp) {
 // V = sum_t d_t 128^(S - t) with |d_t| <= 64, so x = 2^(e + 1) sum_t d_t 2^(-7t);
 // the digits are extracted from the lowest up with balanced remainders and
 // stored as bf16 (exact: |d| <= 64).  One call: group q of row r, S 16-byte
-// stores (one per slice tile).
+// stores (one per slice tile); returns the sum of the squared digits.
 template <int S>
-__device__ __forceinline__ void digits_item(const OzPack& p, const unsigned* eu, __nv_bfloat16* dst, unsigned r,
+__device__ __forceinline__ int digits_item(const OzPack& p, const unsigned* eu, __nv_bfloat16* dst, unsigned r,
                                             unsigned q) {
   const long long tile_elems = (long long)p.TR * OZ_BK;
   constexpr int F = 7 * S - 1;
@@ -795,6 +857,7 @@ __device__ __forceinline__ void digits_item(const OzPack& p, const unsigned* eu,
     }
     dg[0][j] = hi;  // |hi| <= 64 here
   }
+  int sq = 0;
   const unsigned tr = r / p.TR, rr = r - tr * p.TR;  // TR is 32, 64 or 128
   const int tk = (int)(q >> 1), chunk = (int)(q & 1);   // two 8-element chunks per 16-k row
   const long long within = (long long)rr * OZ_BK + ((chunk ^ ((rr >> 2) & 1)) << 3);
@@ -804,12 +867,14 @@ __device__ __forceinline__ void digits_item(const OzPack& p, const unsigned* eu,
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
       // |d| <= 64: exact in float and in bf16, so the conversion is exact
+      sq += dg[t - 1][2 * h] * dg[t - 1][2 * h] + dg[t - 1][2 * h + 1] * dg[t - 1][2 * h + 1];
       const __nv_bfloat162 b2 = __floats2bfloat162_rn((float)dg[t - 1][2 * h], (float)dg[t - 1][2 * h + 1]);
       w[h] = *reinterpret_cast<const uint32_t*>(&b2);
     }
-    const long long tile = ((long long)(t - 1) * p.T + tr) * p.KT + tk;
+    const long long tile = ((long long)tr * p.KT + tk) * S + (t - 1);  // the S tiles of a stage are adjacent
     *reinterpret_cast<uint4*>(dst + tile * tile_elems + within) = make_uint4(w[0], w[1], w[2], w[3]);
   }
+  return sq;
 }
 
 // A 16-k row of a digit tile is 32 bytes, one DRAM sector, filled by its two
@@ -830,16 +895,32 @@ __global__ void __launch_bounds__(PACK_T) k_ozaki_digits(const PackPass pp) {
   const FastDiv fQ = pp.fQ[o], fR = pp.fR[o];
   const unsigned W = pp.W[o];
   const unsigned stride = gridDim.x * PACK_T;
-  for (unsigned i = blockIdx.x * PACK_T + threadIdx.x; i < W; i += stride) {
-    unsigned r, q;
-    if (kfast) {
-      pack_item(i, fQ, fR, true, r, q);
-    } else {
-      const unsigned j = i >> 1, tk = fast_div(j, fR);
-      r = j - tk * fR.d;
-      q = 2u * tk + (i & 1u);
+  int most = 0;  // largest sum of squared digits of one row's 16 k (the window rule)
+  for (unsigned long long base = blockIdx.x * PACK_T; base < W; base += stride) {
+    const unsigned i = (unsigned)base + threadIdx.x;
+    int sq = 0;
+    if (base + threadIdx.x < W) {
+      unsigned r, q;
+      if (kfast) {
+        pack_item(i, fQ, fR, true, r, q);
+      } else {
+        const unsigned j = i >> 1, tk = fast_div(j, fR);
+        r = j - tk * fR.d;
+        q = 2u * tk + (i & 1u);
+      }
+      sq = digits_item<S>(p, eu, dst, r, q);
     }
-    digits_item<S>(p, eu, dst, r, q);
+    // items 2 j and 2 j + 1 are the halves of one row's 16 k
+    sq += __shfl_xor_sync(0xffffffffu, sq, 1);
+    most = sq > most ? sq : most;
+  }
+  most = __reduce_max_sync(0xffffffffu, most);
+  __shared__ int part[PACK_T / 32];
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = most;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < PACK_T / 32; ++w) most = part[w] > most ? part[w] : most;
+    if (most > 0) atomicMax(pp.sq + o, (unsigned)most);
   }
 }
 
@@ -864,15 +945,20 @@ inline int oz_grid(long long n) {
   return (int)b;
 }
 
-size_t oz_smem_bytes(int S, int BN) {
-  const size_t tiles = OZ_NBUF * ((size_t)S * OZ_TILE_BYTES + (size_t)S * BN * OZ_BK * 2);  // stage buffers
-  const size_t stage = (size_t)OZ_BM * (BN + 1) * sizeof(double);  // epilogue tile
-  return (tiles > stage ? tiles : stage) + 1024;
+// stage buffers that fit beside the staging rows and the static tables
+int oz_buffers(int S, int BN) {
+  const int stage = S * (OZ_TILE_BYTES + BN * OZ_BK * 2);
+  const int n = (227 * 1024 - 4096 - 1024 - OZ_STAGE_BYTES) / stage;
+  return n < OZ_MAXBUF ? n : OZ_MAXBUF;
 }
 
-// the largest dynamic shared memory any launch of k_ozaki_mma<BN> asks for,
-// set once per device (kept out of the launch path, which may be captured)
-template <int BN>
+size_t oz_smem_bytes(int S, int BN, int nbuf) {
+  return (size_t)nbuf * S * (OZ_TILE_BYTES + BN * OZ_BK * 2) + OZ_STAGE_BYTES + 1024;
+}
+
+// the largest dynamic shared memory any launch of a kernel asks for, set once
+// per device (kept out of the launch path, which may be captured)
+template <int BN, int S>
 void oz_smem_attribute() {
   static std::mutex mu;
   static bool done[64] = {};
@@ -880,18 +966,39 @@ void oz_smem_attribute() {
   check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
   std::lock_guard<std::mutex> lock(mu);
   if (dev < 0 || dev >= 64 || done[dev]) return;
-  check_cuda(cudaFuncSetAttribute(k_ozaki_mma<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 4096),
+  check_cuda(cudaFuncSetAttribute(k_ozaki_mma<BN, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 4096),
              "cudaFuncSetAttribute (ozaki)");
+  // the kernel's register split draws on exactly this launch total
+  cudaFuncAttributes fa{};
+  check_cuda(cudaFuncGetAttributes(&fa, k_ozaki_mma<BN, S>), "cudaFuncGetAttributes (ozaki)");
+  if (fa.numRegs != OZ_REGS) throw std::runtime_error("split-precision kernel: unexpected register count");
   done[dev] = true;
 }
 
-template <int BN>
-void oz_launch_bn(const OzArgs& a, int MT, int NT, cudaStream_t st) {
+template <int BN, int S>
+void oz_launch_bn_s(const OzArgs& a, cudaStream_t st) {
   // at least 120 KiB so that one CTA (one TMEM allocation) occupies an SM
-  size_t smem = oz_smem_bytes(a.S, BN);
+  size_t smem = oz_smem_bytes(S, BN, a.nbuf);
   if (smem < 120 * 1024) smem = 120 * 1024;
-  oz_smem_attribute<BN>();
-  k_ozaki_mma<BN><<<dim3(MT, NT, a.splits > 1 ? a.splits : 1), OZ_CTA_THREADS, smem, st>>>(a);
+  oz_smem_attribute<BN, S>();
+  const unsigned grid = (unsigned)(a.tiles < 152 ? a.tiles : 152);
+  k_ozaki_mma<BN, S><<<grid, OZ_CTA_THREADS, smem, st>>>(a);
+}
+
+template <int BN>
+void oz_launch_bn(OzArgs a, int MT, int NT, cudaStream_t st) {
+  a.tiles = (long long)MT * NT * a.splits;
+  a.nbuf = oz_buffers(a.S, BN);
+  switch (a.S) {
+    case 1: oz_launch_bn_s<BN, 1>(a, st); break;
+    case 2: oz_launch_bn_s<BN, 2>(a, st); break;
+    case 3: oz_launch_bn_s<BN, 3>(a, st); break;
+    case 4: oz_launch_bn_s<BN, 4>(a, st); break;
+    case 5: oz_launch_bn_s<BN, 5>(a, st); break;
+    case 6: oz_launch_bn_s<BN, 6>(a, st); break;
+    case 7: oz_launch_bn_s<BN, 7>(a, st); break;
+    default: oz_launch_bn_s<BN, 8>(a, st); break;
+  }
   if (a.splits > 1) {
     // few outputs, many splits: a warp per output keeps loads in flight
     if (a.splits >= 32 && a.M * a.N < 152LL * 256)
@@ -994,8 +1101,6 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
   pa.vec = pack_vec_ok(pa);
   pb.vec = pack_vec_ok(pb);
   int BN = ch.bn ? ch.bn : N <= 32 ? 32 : 64;
-  // shared memory per CTA is capped at 227 KiB (static arrays take up to 4 KiB)
-  while (BN > 32 && oz_smem_bytes(S, BN) + 4096 > 227 * 1024) BN /= 2;
   const int MT = (int)((M + OZ_BM - 1) / OZ_BM), NT = (int)((N + BN - 1) / BN);
   const int KT = (int)((g0.K + OZ_BK - 1) / OZ_BK);
   pa.R = M;
@@ -1007,7 +1112,7 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
   pb.TR = BN;
   pb.KT = KT;
   // spread a short output over more CTAs by splitting the k tiles
-  int splits = 1, ktper = KT;
+  int splits = 1, ktper = KT;  // K < 2^31: the integer sums of a tile stay below 2^(31 + 12 + 21)
   const long long ctas = (long long)MT * NT;
   if (ch.split_mode != 1 && ctas < 2 * 152 && KT >= 2 * OZ_SPLIT_MIN) {
     long long sp = (2 * 152 + ctas - 1) / ctas;
@@ -1024,7 +1129,7 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
   double* bufA = ws.get((nA + 3) / 4, capA);  // bf16 digit tiles in double-sized blocks
   double* bufB = ws.get((nB + 3) / 4, capB);
   const size_t nE = (size_t)MT * OZ_BM + (size_t)NT * BN;
-  double* bufE = ws.get((nE + 1) / 2, capE);
+  double* bufE = ws.get((nE + 2 + 1) / 2, capE);
   double* part = nullptr;
   if (splits > 1) part = ws.get((size_t)splits * MT * OZ_BM * NT * BN, capP);
   int* ea = (int*)bufE;
@@ -1036,10 +1141,11 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
     ws.recs[r].n = N;
     ws.recs[r].k = g0.K;
   }
-  check_cuda(cudaMemsetAsync(ea, 0, nE * sizeof(int), st), "cudaMemsetAsync (exponents)");
+  check_cuda(cudaMemsetAsync(ea, 0, (nE + 2) * sizeof(int), st), "cudaMemsetAsync (exponents)");
   PackPass pp{};
   long long w1max = 1, w2max = 1;
   PackPass pd{};
+  pd.sq = (unsigned*)ea + nE;
   for (int o = 0; o < 2; ++o) {
     const OzPack& p = o ? pb : pa;
     const long long rows = (long long)p.T * p.TR;
@@ -1074,6 +1180,7 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
   a.Bs = (const __nv_bfloat16*)bufB;
   a.ea = ea;
   a.fb = fb;
+  a.sq = (const unsigned*)ea + nE;
   a.S = S;
   a.MT = MT;
   a.NT = NT;
@@ -1081,6 +1188,10 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
   a.M = M;
   a.N = N;
   a.alpha = g0.alpha;
+  for (int d = 0; d < 4; ++d) {
+    a.fM[d] = make_fastdiv(d < a.nM ? (unsigned)a.eM[d] : 1u);
+    a.fN[d] = make_fastdiv(d < a.nN ? (unsigned)a.eN[d] : 1u);
+  }
   a.C = g0.C;
   a.status = ws.oz_status;
   a.wait_cycles = ws.wait_cycles > 0 ? ws.wait_cycles : OZ_WAIT_CYCLES;

@@ -3,16 +3,13 @@
 // matrix multiplication by using fast routines of matrix multiplication and
 // its applications" (Numer. Algorithms 59, 2012).
 //
-// Each row of A (and each column of B) is scaled by a power of two so that
-// its largest element is below one in magnitude, and cut into S signed
-// digits of 7 bits: x = 2^e * sum_t d_t 2^(-7t), |d_t| <= 127, each digit
-// exact in BF16.  Products of digits summed over 64 consecutive k stay below
-// 2^24 and are therefore exact in the FP32 accumulator of tcgen05.mma
-// kind::f16.  The pairs (t,u) of one level c = t + u are accumulated
-// together (still exact), levels c <= S + 1 are kept, and each level sum is
-// added into a float-float (two FP32) running sum in tensor memory.  The
-// result carries about 7 S bits relative to the row/column maxima.  S <= 8
-// keeps every level sum exact: 8 pairs x 64 x 127^2 < 2^24.
+// Each row of A (and each column of B) is scaled by a power of two and cut
+// into S balanced base-128 digits, x = 2^(e + 1) sum_t d_t 2^(-7t), |d_t| <= 64,
+// each digit exact in BF16.  The digit pairs (t,u) of one level c = t + u are
+// accumulated together by tcgen05.mma kind::f16, levels c <= S + 1 are kept;
+// over a window of k whose level sums stay within 2^24 they are exact in FP32,
+// and the windows are added in 64-bit integers.  The result carries about 7 S
+// bits relative to the row/column maxima.
 #pragma once
 #include "engine.cuh"
 
