@@ -260,7 +260,8 @@ long long dsrg_peak_bytes(const dsrg_handle *h);
  * alpha-beta block of the spin-free first-order amplitudes this is the
  * spatial ladder from which the energy driver assembles all spin blocks.
  * The (pr|qs) rows are formed in batches in a scratch buffer of at most
- * 1 GiB obtained with cudaMalloc and released before return; the call
+ * 1 GiB from the library's stream-ordered memory pool, given back before
+ * return (the pool keeps at most 1 GiB per device between calls); the call
  * synchronises `stream`.  Errors: DSRG_ERR_ARG (sizes, p0 + np > n, NULL
  * pointers), DSRG_ERR_OOM (scratch), DSRG_ERR_CUDA.
  */
@@ -308,7 +309,7 @@ int dsrg_df_ladder_noalloc(int n, int naux, int p0, int np, int nh, const double
  * Corrections are summed over Q' in increasing order with one rounding per
  * product and per sum (no fused multiply-add), so results are reproducible
  * operation by operation.  Scratch (N + max_vecs + a few thousand doubles)
- * is allocated and released inside the call; synchronises `stream`.
+ * comes from the library's memory pool; synchronises `stream`.
  * Errors: DSRG_ERR_ARG (sizes, tau < 0, NULL pointers), DSRG_ERR_OOM,
  * DSRG_ERR_CUDA.
  */
@@ -323,12 +324,12 @@ int dsrg_cholesky(long long N, const double *V, double tau, int max_vecs, double
  * ldc), all FP64 device memory, row-major.  Every row of A and column of B is
  * scaled by a power of two, rounded to a grid of 2^(7*slices - 1) steps and
  * cut into `slices` (1..8) balanced base-128 digits (|d| <= 64) held exactly
- * in BF16; digit products are accumulated exactly in FP32 over 480-long
- * windows of k by tcgen05.mma and added into a two-float running sum, so the
- * result carries about 7*slices bits relative to the product of the row and
+ * in BF16; digit products are accumulated exactly in FP32 over windows of k
+ * by tcgen05.mma and the windows in 64-bit integers, so the result carries about 7*slices bits relative to the product of the row and
  * column maxima (Ozaki et al., Numer. Algorithms 59 (2012) 95).  With one
  * slice, integers |x| <= 63 are held exactly.
- * Scratch is allocated and released inside the call; synchronises `stream`.
+ * Scratch comes from the library's memory pool (it keeps at most 1 GiB per
+ * device between calls); synchronises `stream`.
  * Errors: DSRG_ERR_ARG (sizes >= 2^31, slices, NULL), DSRG_ERR_OOM (scratch),
  * DSRG_ERR_CUDA (launch failure), DSRG_ERR_TIMEOUT (a bounded wait inside the
  * kernel ran out, default budget).

@@ -2,6 +2,8 @@
 #include "engine.cuh"
 #include "ozaki.cuh"
 
+#include <cuda.h>
+
 #include <algorithm>
 #include <array>
 #include <cstdio>
@@ -17,6 +19,80 @@ void check_cuda(cudaError_t e, const char* what) {
   if (e != cudaSuccess)
     throw Error(e == cudaErrorMemoryAllocation ? DSRG_ERR_OOM : DSRG_ERR_CUDA,
                 std::string(what) + ": " + cudaGetErrorString(e));
+}
+
+// The current context's process-unique id, through driver entry points the
+// runtime hands out (the library does not link the driver library itself).
+// 0 if the driver cannot tell.
+unsigned long long current_context_id() {
+  using GetCurrent = CUresult (*)(CUcontext*);
+  using GetId = CUresult (*)(CUcontext, unsigned long long*);
+  static std::mutex mu;
+  static GetCurrent get_current = nullptr;
+  static GetId get_id = nullptr;
+  static bool looked_up = false;
+  std::lock_guard<std::mutex> lock(mu);
+  if (!looked_up) {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      get_current = reinterpret_cast<GetCurrent>(f);
+    f = nullptr;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      get_id = reinterpret_cast<GetId>(f);
+    cudaGetLastError();
+    looked_up = true;
+  }
+  CUcontext ctx = nullptr;
+  unsigned long long id = 0;
+  if (get_current && get_id && get_current(&ctx) == CUDA_SUCCESS && ctx && get_id(ctx, &id) == CUDA_SUCCESS)
+    return id;
+  return 0;
+}
+
+namespace {
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[64] = {};
+unsigned long long g_pool_ctx[64] = {};
+constexpr unsigned long long kPoolKeep = 1ULL << 30;  // bytes kept between calls
+
+// gives the memory that the current device's pool keeps back to the driver
+void scratch_trim() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  if (g_pool[dev] && g_pool_ctx[dev] == current_context_id()) cudaMemPoolTrimTo(g_pool[dev], 0);
+  cudaGetLastError();
+}
+}  // namespace
+
+cudaMemPool_t scratch_pool() {
+  int dev = 0;
+  check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
+  if (dev < 0 || dev >= 64) return nullptr;
+  check_cuda(cudaFree(nullptr), "context");  // the runtime's context exists from here on
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  // a pool dies with its context (cudaDeviceReset)
+  const unsigned long long ctx = current_context_id();
+  if (ctx == 0) return nullptr;
+  if (g_pool[dev] && g_pool_ctx[dev] == ctx) return g_pool[dev];
+  cudaMemPoolProps props{};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.handleTypes = cudaMemHandleTypeNone;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = dev;
+  cudaMemPool_t pool = nullptr;
+  unsigned long long keep = kPoolKeep;
+  if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) cudaGetLastError();
+  g_pool[dev] = pool;
+  g_pool_ctx[dev] = ctx;
+  return pool;
 }
 
 namespace {
@@ -399,9 +475,19 @@ Workspace::~Workspace() {
     cudaEventDestroy(r.b);
   }
   for (auto e : ev_pool) cudaEventDestroy(e);
-  for (auto& b : free_) cudaFree(b.p);
+  for (auto& b : free_) release(b.p);
   if (results) cudaFree(results);
   if (dot_scratch) cudaFree(dot_scratch);
+}
+
+cudaError_t Workspace::allocate(double** p, size_t n) {
+  return pool_ ? cudaMallocFromPoolAsync((void**)p, n * sizeof(double), pool_, stream)
+               : cudaMalloc((void**)p, n * sizeof(double));
+}
+
+void Workspace::release(double* p) {
+  if (pool_) cudaFreeAsync(p, stream);
+  else cudaFree(p);
 }
 
 double* Workspace::get(size_t n, size_t& cap) {
@@ -420,14 +506,14 @@ double* Workspace::get(size_t n, size_t& cap) {
     got = free_[bi].n;
     free_.erase(free_.begin() + bi);
   } else {
-    cudaError_t e = cudaMalloc(&p, n * sizeof(double));
-    if (e != cudaSuccess) {
-      // drop cached blocks and retry once
+    if (allocate(&p, n) != cudaSuccess) {
+      // drop cached blocks, here and in the scratch pool, and retry once
       cudaGetLastError();
-      for (auto& b : free_) cudaFree(b.p);
+      for (auto& b : free_) release(b.p);
       free_.clear();
       ++generation;
-      check_cuda(cudaMalloc(&p, n * sizeof(double)), "cudaMalloc");
+      scratch_trim();
+      check_cuda(allocate(&p, n), "cudaMalloc");
     }
   }
   in_use_ += got * sizeof(double);

@@ -86,7 +86,9 @@ struct Tensor {
 // the first energy evaluation no further cudaMalloc happens.
 class Workspace {
  public:
-  explicit Workspace(cudaStream_t st) : stream(st) {}
+  // pool: blocks come from this stream-ordered pool and go back to it (the
+  // entry points that own no handle), else from cudaMalloc
+  explicit Workspace(cudaStream_t st, cudaMemPool_t pool = nullptr) : stream(st), pool_(pool) {}
   ~Workspace();
   double* get(size_t n, size_t& cap);
   void put(double* p, size_t cap);
@@ -99,7 +101,7 @@ class Workspace {
   double* dot_scratch = nullptr;  // dot_scratch_len doubles, then the ticket of the one-launch dot
   int dot_scratch_len = 0;
   unsigned* dot_ticket = nullptr;  // zero between launches
-  int* oz_status = nullptr;        // split-precision kernels' error flag (device; nullptr: file-scope flag)
+  int* oz_status = nullptr;        // split-precision kernels' error flag (device)
   long long wait_cycles = 0;       // budget of the split kernels' bounded waits (0: default)
   bool tune = false;               // time tile/split candidates of new split-product shapes
   unsigned long long generation = 0;  // bumped when cached blocks are freed (captured graphs go stale)
@@ -129,10 +131,24 @@ class Workspace {
   void prof_collect();  // after the stream is synchronised
 
  private:
+  cudaError_t allocate(double** p, size_t n);
+  void release(double* p);
   struct Blk { double* p; size_t n; };
+  cudaMemPool_t pool_ = nullptr;
   std::vector<Blk> free_;
   size_t in_use_ = 0, peak_ = 0;
   const char* peak_tag_ = "";  // step being issued when the peak was reached
+};
+
+// A block of a workspace, put back when it goes out of scope.
+struct WorkspaceBlock {
+  Workspace& ws;
+  size_t cap = 0;
+  double* p;
+  WorkspaceBlock(Workspace& w, size_t n) : ws(w), p(w.get(n, cap)) {}
+  ~WorkspaceBlock() { ws.put(p, cap); }
+  WorkspaceBlock(const WorkspaceBlock&) = delete;
+  WorkspaceBlock& operator=(const WorkspaceBlock&) = delete;
 };
 
 // Names the step issued while it is in scope (restores the outer name).
@@ -203,6 +219,16 @@ void fetch_x2(Workspace& ws, double alpha, const Op2& X, Tensor& out);
 View w_place(const Tensor& W, int herm);
 
 void check_cuda(cudaError_t e, const char* what);
+
+// Stream-ordered memory pool of the current device for the scratch of calls
+// that own no handle.  Such a call allocates, runs and synchronises, so with
+// cudaMalloc and cudaFree a small product spent 300 of 380 us on its scratch.
+// The pool keeps at most 1 GiB between calls and gives that back when an
+// allocation of this library fails; the driver orders reuse across streams
+// and threads.  nullptr (plain cudaMalloc) where no pool can be had.
+cudaMemPool_t scratch_pool();
+// the current context's process-unique id, 0 if the driver cannot tell
+unsigned long long current_context_id();
 
 // Persistent record of tuning decisions (file named by DSRG_TUNE_CACHE; no
 // file: decisions live for the process only).  A decision is a few integers

@@ -175,24 +175,20 @@ extern "C" int dsrg_df_ladder(int n, int naux, int p0, int np, int nh, const dou
   if (np == 0 || nh == 0) return DSRG_OK;
   cudaStream_t st = (cudaStream_t)stream;
   const long long p3 = (long long)np * np * np;
-  long long bp = ladder_batch_rows(np, 1LL << 27);  // at most 1 GiB of (pr|qs) per batch
+  long long bp = ladder_batch_rows(np, 1LL << 27);  // at most 1 GiB of scratch
   if (bp < 1) bp = 1;
-  double* G = nullptr;
-  cudaError_t e = cudaMalloc(&G, (size_t)(bp * p3) * sizeof(double));
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return set_error(DSRG_ERR_OOM, (std::string("ladder scratch: ") + cudaGetErrorString(e)).c_str());
-  }
   try {
+    Workspace ws(st, scratch_pool());
+    const WorkspaceBlock rows(ws, (size_t)(bp * p3));
     check_cuda(cudaMemsetAsync(L, 0, (size_t)np * np * nh * nh * sizeof(double), st), "cudaMemsetAsync");
     const long long tst[4] = {(long long)np * nh * nh, (long long)nh * nh, nh, 1};
-    ladder_core(B, n, naux, p0, np, nh, t, tst, L, G, bp, st, nullptr);
+    ladder_core(B, n, naux, p0, np, nh, t, tst, L, rows.p, bp, st, nullptr);
     check_cuda(cudaGetLastError(), "ladder launch");
     check_cuda(cudaStreamSynchronize(st), "cudaStreamSynchronize");
+  } catch (const Error& ex) {
+    return set_error(ex.code, ex.what());
   } catch (const std::exception& ex) {
-    cudaFree(G);
     return set_error(DSRG_ERR_CUDA, ex.what());
   }
-  cudaFree(G);
   return DSRG_OK;
 }

@@ -6,8 +6,6 @@
 // pool), and embedded or real-time runtimes that forbid allocation after
 // start-up.  This entry point takes inputs and outputs from the caller and
 // keeps its own scratch in a fixed, file-scope device array instead.
-#include <cuda.h>
-
 #include <cstdio>
 #include <mutex>
 #include <string>
@@ -25,35 +23,6 @@ constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 double* g_addr[kMaxDevices] = {};
 unsigned long long g_ctx_id[kMaxDevices] = {};
-
-// The current context's process-unique id, through driver entry points the
-// runtime hands out (the library does not link the driver library itself).
-// 0 if the driver cannot tell.
-unsigned long long current_context_id() {
-  using GetCurrent = CUresult (*)(CUcontext*);
-  using GetId = CUresult (*)(CUcontext, unsigned long long*);
-  static GetCurrent get_current = nullptr;
-  static GetId get_id = nullptr;
-  static bool looked_up = false;
-  if (!looked_up) {
-    void* f = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      get_current = reinterpret_cast<GetCurrent>(f);
-    f = nullptr;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      get_id = reinterpret_cast<GetId>(f);
-    cudaGetLastError();
-    looked_up = true;
-  }
-  CUcontext ctx = nullptr;
-  unsigned long long id = 0;
-  if (get_current && get_id && get_current(&ctx) == CUDA_SUCCESS && ctx && get_id(ctx, &id) == CUDA_SUCCESS)
-    return id;
-  return 0;
-}
 
 // Host code cannot use g_ladder_scratch directly: its name here denotes a
 // host-side shadow, not device memory.  The device address is looked up at
@@ -73,7 +42,7 @@ int scratch_address(double** out, std::string& msg) {
     return DSRG_ERR_ARG;
   }
   std::lock_guard<std::mutex> lock(g_mu);
-  const unsigned long long ctx = g_addr[dev] ? current_context_id() : 0;
+  const unsigned long long ctx = g_addr[dev] ? dsrg::current_context_id() : 0;
   if (!g_addr[dev] || ctx == 0 || ctx != g_ctx_id[dev]) {
     double* p = nullptr;
     e = cudaGetSymbolAddress((void**)&p, g_ladder_scratch);
@@ -83,7 +52,7 @@ int scratch_address(double** out, std::string& msg) {
       return DSRG_ERR_CUDA;
     }
     g_addr[dev] = p;
-    g_ctx_id[dev] = current_context_id();
+    g_ctx_id[dev] = dsrg::current_context_id();
   }
   *out = g_addr[dev];
   return DSRG_OK;

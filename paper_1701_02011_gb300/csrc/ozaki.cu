@@ -39,8 +39,6 @@ constexpr unsigned OZ_EBIAS = 2048;
 // about 2 s at 2 GHz)
 constexpr long long OZ_WAIT_CYCLES = 1LL << 32;
 
-__device__ int g_oz_status;
-
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // Shared-memory matrix descriptor: K-major operand in the 32-byte swizzled
@@ -585,7 +583,7 @@ __global__ void __launch_bounds__(OZ_CTA_THREADS, 1) k_ozaki_mma(const OzArgs a)
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm), "r"(TMEM_COLS)
                               : "memory");
-  if (stop && tid == 0) atomicExch(a.status ? a.status : &g_oz_status, 1);
+  if (stop && tid == 0) atomicExch(a.status, 1);
 }
 
 // C[m, n] += alpha * sum_z part[z][m][n] (z in order)
@@ -1014,14 +1012,9 @@ void oz_launch_mma(const OzArgs& a, int MT, int NT, int BN, cudaStream_t st) {
 }
 }  // namespace
 
-const void* g_oz_status_alias() { return (const void*)&g_oz_status; }
-
 int ozaki_status(cudaStream_t st, const int* flag) {
   int v = 0;
-  if (flag)
-    check_cuda(cudaMemcpyAsync(&v, flag, sizeof(int), cudaMemcpyDeviceToHost, st), "status");
-  else
-    check_cuda(cudaMemcpyFromSymbolAsync(&v, g_oz_status, sizeof(int), 0, cudaMemcpyDeviceToHost, st), "status");
+  check_cuda(cudaMemcpyAsync(&v, flag, sizeof(int), cudaMemcpyDeviceToHost, st), "status");
   check_cuda(cudaStreamSynchronize(st), "sync");
   return v;
 }
@@ -1344,10 +1337,10 @@ extern "C" int dsrg_split_gemm(long long M, long long N, long long K, const doub
   if (!A || !B || !C) return set_error(DSRG_ERR_ARG, "split gemm: NULL pointer");
   cudaStream_t st = (cudaStream_t)stream;
   try {
-    Workspace ws(st);
-    int zero = 0;
-    check_cuda(cudaMemcpyToSymbolAsync(g_oz_status_alias(), &zero, sizeof(int), 0, cudaMemcpyHostToDevice, st),
-               "status reset");
+    Workspace ws(st, scratch_pool());
+    const WorkspaceBlock flag(ws, 1);
+    ws.oz_status = reinterpret_cast<int*>(flag.p);
+    check_cuda(cudaMemsetAsync(ws.oz_status, 0, sizeof(int), st), "status reset");
     GemmArgs g{};
     g.A = A;
     g.B = B;
@@ -1371,7 +1364,7 @@ extern "C" int dsrg_split_gemm(long long M, long long N, long long K, const doub
     g.nbatch = 1;
     ozaki_gemm(ws, g, slices, K_OZAKI_MMA);
     check_cuda(cudaGetLastError(), "split gemm launch");
-    if (ozaki_status(st, nullptr))
+    if (ozaki_status(st, ws.oz_status))
       return set_error(DSRG_ERR_TIMEOUT, "split gemm: a bounded wait in the kernel ran out");
   } catch (const Error& e) {
     return set_error(e.code, e.what());

@@ -18,10 +18,8 @@ namespace dsrg {
 constexpr int kOzakiMaxSlices = 8;
 
 // Error status of the split-precision kernels (device flag set when a bounded
-// wait runs out; flag nullptr: the file-scope flag); 0 = ok.  Synchronises st.
+// wait runs out); 0 = ok.  Synchronises st.
 int ozaki_status(cudaStream_t st, const int* flag);
-// the status flag's symbol (for cudaMemcpyToSymbol)
-const void* g_oz_status_alias();
 
 // C[m,n] += alpha * sum_k A[m,k] B[k,n] for the multi-index contraction g
 // (nbatch must be 1) with `slices` digits per operand.  Scratch comes from ws.
