@@ -35,15 +35,15 @@ constexpr int LZ_MAX_STEPS = 300;  // Krylov dimension per Lanczos run
 constexpr int LZ_MAX_RUNS = 6;     // restarts from the Ritz vector
 constexpr long long RELAX_MAX_DET = 20000;
 
-// fixed-order sum of one value per thread of an RX_T-thread block
+// fixed-order sum of one value per thread of an RX_T-thread block, in every thread
 __device__ double block_sum(double v, double* sh) {
-  sh[threadIdx.x] = v;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
   __syncthreads();
-  for (int w = RX_T / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-    __syncthreads();
-  }
-  const double r = sh[0];
+  double r = 0.0;
+#pragma unroll
+  for (int w = 0; w < RX_T / 32; ++w) r += sh[w];
   __syncthreads();
   return r;
 }
@@ -168,98 +168,180 @@ __global__ void __launch_bounds__(RX_T) k_dots(long long n, const double* V, con
   if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
-// x -= sum_{k < nv} coef[k] V[k]
-__global__ void k_subtract(long long n, int nv, const double* __restrict__ V, const double* __restrict__ coef,
-                           double* __restrict__ x, const LzState* st) {
+// x -= sum_{k < nv} coef[k] V[k].  A CTA takes 32 elements, one per lane, and
+// its eight warps every eighth vector each: with one thread per element the
+// 300 dependent loads of a step took 22 us at 400 determinants.
+// LAST (the second pass of a Lanczos step): the CTA that finishes last (atomic
+// ticket, no CTA waits) adds the CTAs' shares of |x|^2 in order, writes
+// alpha_j and beta_j = |x|, tests for breakdown or length, and sets
+// V[j + 1] = x / beta_j.
+struct LzStep {
+  int j, mmax;
+  const double* coef;  // V . H v_j, its j-th entry is alpha_j
+  double *alpha, *beta, *partial;
+  unsigned* ticket;  // zero between launches
+};
+
+template <bool LAST>
+__global__ void __launch_bounds__(RX_T) k_subtract(long long n, int nv, double* V, const double* __restrict__ coef,
+                                                   double* x, LzState* st, const LzStep p) {
   if (st && st->done) return;
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  double t = x[i];
-  for (int k = 0; k < nv; ++k) t -= coef[k] * V[k * n + i];
-  x[i] = t;
+  constexpr int NW = RX_T / 32;
+  __shared__ double sh[NW][32];
+  __shared__ double red[NW];
+  __shared__ bool last, go_on;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long i = blockIdx.x * 32LL + lane;
+  double s = 0.0;
+  if (i < n) {
+#pragma unroll 8
+    for (int k = warp; k < nv; k += NW) s += coef[k] * V[k * n + i];
+  }
+  sh[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) t += sh[w][lane];
+    double v = 0.0;
+    if (i < n) {
+      v = x[i] - t;
+      x[i] = v;
+    }
+    if (LAST) {
+      v *= v;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      __threadfence();  // x before the ticket
+      __syncwarp();
+      if (lane == 0) {
+        p.partial[blockIdx.x] = v;
+        __threadfence();
+        last = atomicAdd(p.ticket, 1u) == gridDim.x - 1;
+      }
+    }
+  }
+  if (!LAST) return;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  s = 0.0;
+  for (unsigned c = threadIdx.x; c < gridDim.x; c += RX_T) s += __ldcg(p.partial + c);
+  s = block_sum(s, red);
+  if (threadIdx.x == 0) {
+    const double a = p.coef[p.j], b = sqrt(fmax(s, 0.0));
+    p.alpha[p.j] = a;
+    p.beta[p.j] = b;
+    st->hmax = fmax(st->hmax, fmax(fabs(a), b));
+    st->steps = p.j + 1;
+    go_on = !(b <= 1e-12 * st->hmax || p.j + 1 >= p.mmax);
+    if (!go_on) st->done = 1;
+    red[0] = b;
+    *p.ticket = 0u;
+  }
+  __syncthreads();
+  if (!go_on) return;
+  const double b = red[0];
+  for (long long c = threadIdx.x; c < n; c += RX_T) V[(p.j + 1) * n + c] = __ldcg(x + c) / b;
 }
 
-// alpha_j, beta_j = |w|, breakdown / length test
-__global__ void k_lz_next(int j, int mmax, const double* coef, const double* nrm2, double* alpha, double* beta,
-                          LzState* st) {
-  if (st->done) return;
-  const double a = coef[j], b = sqrt(fmax(*nrm2, 0.0));
-  alpha[j] = a;
-  beta[j] = b;
-  st->hmax = fmax(st->hmax, fmax(fabs(a), b));
-  st->steps = j + 1;
-  if (b <= 1e-12 * st->hmax || j + 1 >= mmax) st->done = 1;
-}
-
-// V[j + 1] = w / beta_j
-__global__ void k_lz_scale(long long n, int j, const double* __restrict__ w, const double* __restrict__ beta,
-                           double* __restrict__ V, const LzState* st) {
-  if (st->done) return;
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i < n) V[(j + 1) * n + i] = w[i] / beta[j];
-}
-
-// number of eigenvalues of the tridiagonal (a, b) below x (Sturm sequence)
-__device__ int sturm_count(int k, const double* a, const double* b, double x) {
-  int cnt = 0;
+// whether the tridiagonal (a, squared off-diagonals b2) has an eigenvalue
+// below x (Sturm sequence: the first negative quotient)
+__device__ bool any_below(int k, const double* a, const double* b2, double x) {
   double q = a[0] - x;
   for (int i = 0;; ++i) {
-    if (q < 0.0) ++cnt;
-    if (i + 1 >= k) break;
+    if (q < 0.0) return true;
+    if (i + 1 >= k) return false;
     if (q == 0.0) q = 1e-300;
-    q = (a[i + 1] - x) - b[i] * b[i] / q;
+    q = (a[i + 1] - x) - b2[i] / q;
   }
-  return cnt;
 }
 
-// lowest eigenvalue of the tridiagonal matrix and its unit eigenvector y
-// (single thread; work: 3 k doubles)
-__global__ void k_lz_tridiag(const double* __restrict__ a, const double* __restrict__ b, LzState* st,
-                             double* __restrict__ y, double* __restrict__ work) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// lowest eigenvalue of the tridiagonal matrix and its unit eigenvector y (one
+// warp).  The bracket shrinks 33-fold a pass, one Sturm sequence per lane; the
+// vectors of the inverse iteration live in shared memory.  (One thread
+// bisecting, with its vectors in global memory, took 8.7 ms at 300 steps.)
+__global__ void __launch_bounds__(32) k_lz_tridiag(const double* __restrict__ a_, const double* __restrict__ b_,
+                                                   LzState* st, double* __restrict__ y_) {
+  __shared__ double a[LZ_MAX_STEPS], b[LZ_MAX_STEPS], b2[LZ_MAX_STEPS], d[LZ_MAX_STEPS], l[LZ_MAX_STEPS],
+      z[LZ_MAX_STEPS], y[LZ_MAX_STEPS];
+  const int lane = threadIdx.x;
   const int k = st->steps;
   double lo = INFINITY, hi = -INFINITY;
-  for (int i = 0; i < k; ++i) {
+  for (int i = lane; i < k; i += 32) {
+    a[i] = a_[i];
+    b[i] = b_[i];
+    b2[i] = b_[i] * b_[i];
+  }
+  __syncwarp();
+  for (int i = lane; i < k; i += 32) {
     const double r = (i > 0 ? fabs(b[i - 1]) : 0.0) + (i + 1 < k ? fabs(b[i]) : 0.0);
     lo = fmin(lo, a[i] - r);
     hi = fmax(hi, a[i] + r);
   }
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
   for (int it = 0; it < 4000; ++it) {
     const double mid = 0.5 * (lo + hi);
     if (!(mid > lo && mid < hi)) break;
-    if (sturm_count(k, a, b, mid) >= 1) hi = mid;
-    else lo = mid;
+    // 32 points inside the bracket, in increasing order; equal neighbours are harmless
+    const double x = lane == 15 ? mid : fmin(fmax(lo + (hi - lo) * ((lane + 1) / 33.0), lo), hi);
+    const bool in = x > lo && x < hi;
+    const unsigned below = __ballot_sync(0xffffffffu, in && any_below(k, a, b2, x));
+    const unsigned inside = __ballot_sync(0xffffffffu, in);
+    // new bracket: the smallest point with an eigenvalue below it, the largest without
+    double nh = (below >> lane) & 1 ? x : hi, nl = ((inside & ~below) >> lane) & 1 ? x : lo;
+    for (int o = 16; o > 0; o >>= 1) {
+      nh = fmin(nh, __shfl_xor_sync(0xffffffffu, nh, o));
+      nl = fmax(nl, __shfl_xor_sync(0xffffffffu, nl, o));
+    }
+    if (!(nl < nh)) nl = lo;  // rounding made the sequence non-monotonic: keep the lower end
+    lo = nl;
+    hi = nh;
   }
   const double lam = 0.5 * (lo + hi);
-  // inverse iteration with the shift sigma just below lam: T - sigma is
-  // positive definite, so its LDL^T factorisation needs no pivoting
-  const double scale = fmax(st->hmax, 1e-300);
-  const double sigma = lam - 1e-10 * scale;
-  double* d = work;
-  double* l = work + k;
-  double* z = work + 2 * k;
-  d[0] = a[0] - sigma;
-  for (int i = 0; i + 1 < k; ++i) {
-    l[i] = b[i] / d[i];
-    d[i + 1] = (a[i + 1] - sigma) - l[i] * b[i];
+  if (lane == 0) {
+    // inverse iteration with the shift sigma just below lam: T - sigma is
+    // positive definite, so its LDL^T factorisation needs no pivoting
+    const double scale = fmax(st->hmax, 1e-300);
+    const double sigma = lam - 1e-10 * scale;
+    d[0] = a[0] - sigma;
+    for (int i = 0; i + 1 < k; ++i) {
+      l[i] = b[i] / d[i];
+      d[i + 1] = (a[i + 1] - sigma) - l[i] * b[i];
+    }
   }
-  for (int i = 0; i < k; ++i) y[i] = 1.0;
+  __syncwarp();
+  for (int i = lane; i < k; i += 32) y[i] = 1.0;
+  __syncwarp();
   for (int it = 0; it < 4; ++it) {
     // L z' = y, D z'' = z', L^T z = z''
-    z[0] = y[0];
-    for (int i = 1; i < k; ++i) z[i] = y[i] - l[i - 1] * z[i - 1];
-    for (int i = 0; i < k; ++i) z[i] /= d[i];
-    for (int i = k - 2; i >= 0; --i) z[i] -= l[i] * z[i + 1];
+    if (lane == 0) {
+      z[0] = y[0];
+      for (int i = 1; i < k; ++i) z[i] = y[i] - l[i - 1] * z[i - 1];
+    }
+    __syncwarp();
+    for (int i = lane; i < k; i += 32) z[i] /= d[i];
+    __syncwarp();
+    if (lane == 0)
+      for (int i = k - 2; i >= 0; --i) z[i] -= l[i] * z[i + 1];
+    __syncwarp();
     double nrm = 0.0;
-    for (int i = 0; i < k; ++i) nrm += z[i] * z[i];
+    for (int i = lane; i < k; i += 32) nrm += z[i] * z[i];
+    for (int o = 16; o > 0; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
     nrm = sqrt(nrm);
     if (!(nrm > 0.0) || !isfinite(nrm)) {  // degenerate scale (e.g. a zero matrix): first basis vector
-      for (int i = 0; i < k; ++i) y[i] = i == 0 ? 1.0 : 0.0;
+      for (int i = lane; i < k; i += 32) y[i] = i == 0 ? 1.0 : 0.0;
       break;
     }
-    for (int i = 0; i < k; ++i) y[i] = z[i] / nrm;
+    for (int i = lane; i < k; i += 32) y[i] = z[i] / nrm;
+    __syncwarp();
   }
-  st->lambda = lam;
+  __syncwarp();
+  for (int i = lane; i < k; i += 32) y_[i] = y[i];
+  if (lane == 0) st->lambda = lam;
 }
 
 // x = sum_k y[k] V[k]
@@ -397,7 +479,11 @@ RelaxResult relaxed_ci(Handle& h, int order, int n_alpha, int n_beta) {
   ws.launches += 1;
   // Lanczos with full reorthogonalisation (Gram-Schmidt applied twice)
   const int mmax = (int)(ndet < LZ_MAX_STEPS ? ndet : LZ_MAX_STEPS);
-  Scratch V(ws, (size_t)(mmax + 1) * ndet), w(ws, ndet), x(ws, ndet), work(ws, 3 * LZ_MAX_STEPS);
+  Scratch V(ws, (size_t)(mmax + 1) * ndet), w(ws, ndet), x(ws, ndet);
+  const unsigned gs = grid_for(ndet, 32);
+  Scratch part(ws, (size_t)gs + 1);  // shares of |w|^2, then the ticket of the CTA that finishes last
+  unsigned* ticket = reinterpret_cast<unsigned*>(part.p + gs);
+  check_cuda(cudaMemsetAsync(ticket, 0, sizeof(unsigned), st), "cudaMemsetAsync (lanczos)");
   Scratch sc(ws, 5 * LZ_MAX_STEPS + 16);
   double* coef = sc.p;
   double* coef2 = sc.p + LZ_MAX_STEPS;
@@ -423,16 +509,14 @@ RelaxResult relaxed_ci(Handle& h, int order, int n_alpha, int n_beta) {
       k_matvec<<<gw, 256, 0, st>>>(ndet, H.p, vj, w.p, lst);
       ws.end(rec);
       k_dots<<<j + 1, RX_T, 0, st>>>(ndet, V.p, w.p, coef, lst);
-      k_subtract<<<gn, 256, 0, st>>>(ndet, j + 1, V.p, coef, w.p, lst);
+      const LzStep step{j, mmax, coef, alpha, beta, part.p, ticket};
+      k_subtract<false><<<gs, RX_T, 0, st>>>(ndet, j + 1, V.p, coef, w.p, lst, step);
       k_dots<<<j + 1, RX_T, 0, st>>>(ndet, V.p, w.p, coef2, lst);
-      k_subtract<<<gn, 256, 0, st>>>(ndet, j + 1, V.p, coef2, w.p, lst);
-      k_dots<<<1, RX_T, 0, st>>>(ndet, w.p, w.p, nrm, lst);
-      k_lz_next<<<1, 1, 0, st>>>(j, mmax, coef, nrm, alpha, beta, lst);
-      k_lz_scale<<<gn, 256, 0, st>>>(ndet, j, w.p, beta, V.p, lst);
-      ws.launches += 7;
+      k_subtract<true><<<gs, RX_T, 0, st>>>(ndet, j + 1, V.p, coef2, w.p, lst, step);
+      ws.launches += 4;
     }
     check_cuda(cudaGetLastError(), "lanczos launch");
-    k_lz_tridiag<<<1, 1, 0, st>>>(alpha, beta, lst, y, work.p);
+    k_lz_tridiag<<<1, 32, 0, st>>>(alpha, beta, lst, y);
     LzState hs{};
     check_cuda(cudaMemcpyAsync(&hs, lst, sizeof hs, cudaMemcpyDeviceToHost, st), "copy lanczos state");
     check_cuda(cudaStreamSynchronize(st), "sync");
