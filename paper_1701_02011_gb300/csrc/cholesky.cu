@@ -18,8 +18,14 @@
 
 namespace {
 
-constexpr int CH_T = 256;
 constexpr int CH_MAX_CTAS = 152 * 4;
+// Threads per CTA.  Every correction is one rounded product and one rounded
+// sum, and an SM retires two FP64 operations a clock, so a step lasts as long
+// as the SM with the most rows: up to N = 152 x 96 each SM gets one CTA of 96
+// rows (with 256 threads at N = 13456 the factorisation used 53 of the 152
+// SMs, 40 us a vector on average; now 24 us).  Larger N fill the chip with 256.
+constexpr long long CH_SMALL_N = 152LL * 96;
+constexpr int CH_Q = 512;  // earlier vectors whose pivot entries are held at a time
 
 struct ChState {
   long long J;     // pivot of the vector being formed
@@ -35,31 +41,44 @@ __device__ __forceinline__ bool better(double v, long long i, double bv, long lo
   return v > bv || (v == bv && i < bi);
 }
 
-// in-CTA reduction of (value, index) pairs; result in v[0], ix[0]
-__device__ void cta_argmax(double* v, long long* ix) {
-  for (int w = CH_T / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w && better(v[threadIdx.x + w], ix[threadIdx.x + w], v[threadIdx.x], ix[threadIdx.x])) {
-      v[threadIdx.x] = v[threadIdx.x + w];
-      ix[threadIdx.x] = ix[threadIdx.x + w];
+// in-CTA maximum of one (value, index) pair per thread; valid in thread 0
+template <int CH_T>
+__device__ void cta_argmax(double& v, long long& i) {
+  __shared__ double sv[CH_T / 32];
+  __shared__ long long si[CH_T / 32];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double ov = __shfl_down_sync(0xffffffffu, v, o);
+    const long long oi = __shfl_down_sync(0xffffffffu, i, o);
+    if (better(ov, oi, v, i)) {
+      v = ov;
+      i = oi;
     }
-    __syncthreads();
   }
+  __syncthreads();  // an earlier call's values are no longer read
+  if ((threadIdx.x & 31) == 0) {
+    sv[threadIdx.x >> 5] = v;
+    si[threadIdx.x >> 5] = i;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int w = 1; w < CH_T / 32; ++w)
+      if (better(sv[w], si[w], v, i)) {
+        v = sv[w];
+        i = si[w];
+      }
 }
 
 // The CTA that finishes last combines the per-CTA maxima (fixed order) and
 // sets the next pivot, or stops.  finish: the vector of this launch is done.
+template <int CH_T>
 __device__ void last_cta_pivot(double bv, long long bi, double* pv, long long* pi, ChState* st, double tau,
                                int max_vecs, long long* piv, bool finish) {
-  __shared__ double sv[CH_T];
-  __shared__ long long si[CH_T];
   __shared__ bool last;
-  sv[threadIdx.x] = bv;
-  si[threadIdx.x] = bi;
-  __syncthreads();
-  cta_argmax(sv, si);
+  cta_argmax<CH_T>(bv, bi);
   if (threadIdx.x == 0) {
-    pv[blockIdx.x] = sv[0];
-    pi[blockIdx.x] = si[0];
+    pv[blockIdx.x] = bv;
+    pi[blockIdx.x] = bi;
     __threadfence();
     last = atomicAdd(&st->ticket, 1u) == gridDim.x - 1;
   }
@@ -76,24 +95,22 @@ __device__ void last_cta_pivot(double bv, long long bi, double* pv, long long* p
       i = ci;
     }
   }
-  sv[threadIdx.x] = v;
-  si[threadIdx.x] = i;
-  __syncthreads();
-  cta_argmax(sv, si);
+  cta_argmax<CH_T>(v, i);
   if (threadIdx.x == 0) {
     if (finish) st->nvec += 1;
-    if (!(sv[0] > tau) || si[0] < 0 || st->nvec >= max_vecs) {
+    if (!(v > tau) || i < 0 || st->nvec >= max_vecs) {
       st->done = 1;
     } else {
-      st->J = si[0];
-      st->dJ = sv[0];
-      piv[st->nvec] = si[0];
+      st->J = i;
+      st->dJ = v;
+      piv[st->nvec] = i;
     }
     st->ticket = 0u;
   }
 }
 
 // D = diag(V) and the first pivot
+template <int CH_T>
 __global__ void __launch_bounds__(CH_T) k_chol_init(const double* __restrict__ V, long long N, double* __restrict__ D,
                                                    double* pv, long long* pi, ChState* st, double tau, int max_vecs,
                                                    long long* piv) {
@@ -107,10 +124,11 @@ __global__ void __launch_bounds__(CH_T) k_chol_init(const double* __restrict__ V
       bi = i;
     }
   }
-  last_cta_pivot(bv, bi, pv, pi, st, tau, max_vecs, piv, false);
+  last_cta_pivot<CH_T>(bv, bi, pv, pi, st, tau, max_vecs, piv, false);
 }
 
 // one vector: B[nvec][i], D[i] -= B[nvec][i]^2, and the next pivot
+template <int CH_T>
 __global__ void __launch_bounds__(CH_T) k_chol_step(const double* __restrict__ V, long long N, double* __restrict__ B,
                                                    double* __restrict__ D, double* pv, long long* pi, ChState* st,
                                                    double tau, int max_vecs, long long* piv) {
@@ -121,20 +139,44 @@ __global__ void __launch_bounds__(CH_T) k_chol_step(const double* __restrict__ V
   const double* __restrict__ bJ = B + J;  // B[q][J] at bJ[q * N]
   double bv = -INFINITY;
   long long bi = -1;
-  for (long long i = blockIdx.x * (long long)CH_T + threadIdx.x; i < N; i += (long long)gridDim.x * CH_T) {
-    // the products of 16 vectors are loaded and formed ahead of their
-    // (sequential, increasing-q) additions, so many loads are in flight
+  // the pivot's column of the earlier vectors goes through shared memory, CH_Q
+  // at a time (each entry its own DRAM sector: one round of loads, not one a
+  // product); this thread's column is loaded 16 vectors ahead of the products
+  // being formed and added (sequentially, in increasing q)
+  __shared__ double yj[CH_Q];
+  for (long long i0 = blockIdx.x * (long long)CH_T; i0 < N; i0 += (long long)gridDim.x * CH_T) {
+    const long long i = i0 + threadIdx.x;
+    const bool live = i < N;
+    const double* __restrict__ bi_ = B + (live ? i : 0);
+    constexpr int U = 16;
     double acc = 0.0;
-    int q = 0;
-    for (; q + 16 <= Q; q += 16) {
-      double pr[16];
+    for (int q0 = 0; q0 < Q; q0 += CH_Q) {
+      const int nq = Q - q0 < CH_Q ? Q - q0 : CH_Q;
+      double x[U];
+      const int full = nq / U * U;
+      if (full > 0) {
 #pragma unroll
-      for (int u = 0; u < 16; ++u)
-        pr[u] = __dmul_rn(__ldg(B + (long long)(q + u) * N + i), __ldg(bJ + (long long)(q + u) * N));
+        for (int u = 0; u < U; ++u) x[u] = __ldg(bi_ + (long long)(q0 + u) * N);
+      }
+      __syncthreads();  // the last block's entries are no longer read
+      for (int q = threadIdx.x; q < nq; q += CH_T) yj[q] = __ldg(bJ + (long long)(q0 + q) * N);
+      __syncthreads();
+      for (int q = 0; q < full; q += U) {
+        double nx[U];
+        if (q + U < full) {
 #pragma unroll
-      for (int u = 0; u < 16; ++u) acc = __dadd_rn(acc, pr[u]);
+          for (int u = 0; u < U; ++u) nx[u] = __ldg(bi_ + (long long)(q0 + q + U + u) * N);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) x[u] = __dmul_rn(x[u], yj[q + u]);
+#pragma unroll
+        for (int u = 0; u < U; ++u) acc = __dadd_rn(acc, x[u]);
+#pragma unroll
+        for (int u = 0; u < U; ++u) x[u] = nx[u];
+      }
+      for (int q = full; q < nq; ++q) acc = __dadd_rn(acc, __dmul_rn(__ldg(bi_ + (long long)(q0 + q) * N), yj[q]));
     }
-    for (; q < Q; ++q) acc = __dadd_rn(acc, __dmul_rn(__ldg(B + (long long)q * N + i), __ldg(bJ + (long long)q * N)));
+    if (!live) continue;
     const double L = __ddiv_rn(__dsub_rn(V[J * N + i], acc), sq);
     B[(long long)Q * N + i] = L;
     const double d = __dsub_rn(D[i], __dmul_rn(L, L));
@@ -144,11 +186,11 @@ __global__ void __launch_bounds__(CH_T) k_chol_step(const double* __restrict__ V
       bi = i;
     }
   }
-  last_cta_pivot(bv, bi, pv, pi, st, tau, max_vecs, piv, true);
+  last_cta_pivot<CH_T>(bv, bi, pv, pi, st, tau, max_vecs, piv, true);
 }
 
-inline int ch_grid(long long N) {
-  long long g = (N + CH_T - 1) / CH_T;
+inline int ch_grid(long long N, int threads) {
+  long long g = (N + threads - 1) / threads;
   if (g < 1) g = 1;
   if (g > CH_MAX_CTAS) g = CH_MAX_CTAS;
   return (int)g;
@@ -165,27 +207,24 @@ extern "C" int dsrg_cholesky(long long N, const double* V, double tau, int max_v
   if (!V || !B) return set_error(DSRG_ERR_ARG, "cholesky: V and B must be device pointers");
   if (N > (1LL << 40) / N) return set_error(DSRG_ERR_ARG, "cholesky: N too large");
   cudaStream_t st = (cudaStream_t)stream;
-  const int grid = ch_grid(N);
+  const bool small = N <= CH_SMALL_N;
+  const int grid = ch_grid(N, small ? 96 : 256);
   // scratch: D [N], per-CTA maxima, pivots [max_vecs], state
-  double* D = nullptr;
   const size_t bytes = (size_t)N * 8 + (size_t)grid * 16 + (size_t)max_vecs * 8 + sizeof(ChState) + 64;
-  cudaError_t e = cudaMalloc(&D, bytes);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return set_error(DSRG_ERR_OOM, (std::string("cholesky scratch: ") + cudaGetErrorString(e)).c_str());
-  }
-  double* pv = D + N;
-  long long* pi = reinterpret_cast<long long*>(pv + grid);
-  long long* piv = pi + grid;
-  ChState* cs = reinterpret_cast<ChState*>(piv + max_vecs);
-  int rc = DSRG_OK;
   try {
+    Workspace ws(st, scratch_pool());
+    const WorkspaceBlock scratch(ws, (bytes + 7) / 8);
+    double* D = scratch.p;
+    double* pv = D + N;
+    long long* pi = reinterpret_cast<long long*>(pv + grid);
+    long long* piv = pi + grid;
+    ChState* cs = reinterpret_cast<ChState*>(piv + max_vecs);
     check_cuda(cudaMemsetAsync(cs, 0, sizeof(ChState), st), "cudaMemsetAsync (cholesky)");
-    k_chol_init<<<grid, CH_T, 0, st>>>(V, N, D, pv, pi, cs, tau, max_vecs, piv);
+    (small ? k_chol_init<96> : k_chol_init<256>)<<<grid, small ? 96 : 256, 0, st>>>(V, N, D, pv, pi, cs, tau, max_vecs, piv);
     check_cuda(cudaGetLastError(), "cholesky launch");
     ChState h{};
     for (int q = 0; q < max_vecs; ++q) {
-      k_chol_step<<<grid, CH_T, 0, st>>>(V, N, B, D, pv, pi, cs, tau, max_vecs, piv);
+      (small ? k_chol_step<96> : k_chol_step<256>)<<<grid, small ? 96 : 256, 0, st>>>(V, N, B, D, pv, pi, cs, tau, max_vecs, piv);
       check_cuda(cudaGetLastError(), "cholesky launch");
       // every 32 vectors: stop launching once the factorisation has stopped
       if ((q & 31) == 31 || q == max_vecs - 1) {
@@ -201,10 +240,9 @@ extern "C" int dsrg_cholesky(long long N, const double* V, double tau, int max_v
       check_cuda(cudaMemcpy(pivots, piv, (size_t)h.nvec * sizeof(long long), cudaMemcpyDeviceToHost),
                  "cudaMemcpy (pivots)");
   } catch (const Error& ex) {
-    rc = set_error(ex.code, ex.what());
+    return set_error(ex.code, ex.what());
   } catch (const std::exception& ex) {
-    rc = set_error(DSRG_ERR_INTERNAL, ex.what());
+    return set_error(DSRG_ERR_INTERNAL, ex.what());
   }
-  cudaFree(D);
-  return rc;
+  return DSRG_OK;
 }
