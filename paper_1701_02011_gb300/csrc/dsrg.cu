@@ -135,11 +135,7 @@ void build_v(Handle& h, unsigned classes, Sym2& V, bool on_demand) {
   if (const char* env = getenv("DSRG_V_CLASS_BUDGET_MB")) {
     budget = atof(env) * 1048576.0;
   } else {
-    int dev = 0;
-    check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
-    cudaDeviceProp prop{};
-    check_cuda(cudaGetDeviceProperties(&prop, dev), "cudaGetDeviceProperties");
-    budget = 0.2 * (double)prop.totalGlobalMem;
+    budget = 0.2 * h.device_bytes;
     if (budget > 64.0 * 1073741824.0) budget = 64.0 * 1073741824.0;
     if (budget < 8.0 * 1073741824.0) budget = 8.0 * 1073741824.0;
   }
@@ -314,20 +310,25 @@ void df_ladder(Handle& h, const Tensor& T2, Tensor& C2, double coef) {
   size_t capL;
   size_t nL = (size_t)p * p * hh * hh;
   double* L = h.ws.get(nL, capL);
-  check_cuda(cudaMemsetAsync(L, 0, nL * sizeof(double), h.ws.stream), "memset");
-  // (pr|qs) in batches of rows within a budget (DSRG_LADDER_BUDGET_MB,
-  // default 1024 MB); the first-order alpha-beta amplitudes have
-  // t[r,s,i,j] = t[s,r,j,i], so the pair-symmetric form applies
-  double budget_mb = 1024.0;
-  if (const char* env = getenv("DSRG_LADDER_BUDGET_MB")) budget_mb = atof(env);
+  // batches of rows within a budget (DSRG_LADDER_BUDGET_MB, default 1024 MB);
+  // the first-order alpha-beta amplitudes have t[r,s,i,j] = t[s,r,j,i], so the
+  // pair-symmetric forms apply: with (pr|qs) over pairs held whole where that
+  // takes at most an eighth of the device (p <= 364 on 284 GB) or the stated
+  // budget, else in batches
+  double budget_mb = 1024.0, whole = h.device_bytes / 8.0;
+  if (const char* env = getenv("DSRG_LADDER_BUDGET_MB")) {
+    budget_mb = atof(env);
+    whole = budget_mb * 1048576.0;
+  }
   long long maxd = (long long)(budget_mb * 131072.0);
-  const long long p3 = (long long)p * p * p;
-  if (maxd < p3) maxd = p3;  // one row p with every q >= p0 (the first batch)
-  size_t capG;
-  double* G = h.ws.get((size_t)maxd, capG);
   const long long tst[4] = {tv.st[0], tv.st[1], tv.st[2], tv.st[3]};
-  ladder_core_sym(h.B, h.n, h.naux, h.nc, p, hh, t, tst, L, G, maxd, h.ws.stream, &h.ws);
-  h.ws.put(G, capG);
+  if (!ladder_core_pairs(h.B, h.n, h.naux, h.nc, p, hh, t, tst, L, maxd, whole, h.ws)) {
+    check_cuda(cudaMemsetAsync(L, 0, nL * sizeof(double), h.ws.stream), "memset");
+    const long long p3 = (long long)p * p * p;
+    if (maxd < p3) maxd = p3;  // one row p with every q >= p0 (the first batch)
+    WorkspaceBlock G(h.ws, (size_t)maxd);
+    ladder_core_sym(h.B, h.n, h.naux, h.nc, p, hh, t, tst, L, G.p, maxd, h.ws.stream, &h.ws);
+  }
   // scatter into the spin blocks of C2 [2p][2p][2h][2h]
   const View& c = C2.v;
   int ext[4] = {p, p, hh, hh};

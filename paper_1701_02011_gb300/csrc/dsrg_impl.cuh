@@ -8,6 +8,7 @@ struct Handle {
   int nc = 0, na = 0, nv = 0, n = 0, naux = 0;
   double s = 0.0;
   Iv C, A, V, H, P, G;  // core, active, virtual, hole, particle, general
+  double device_bytes = 0.0;  // memory of the device (bounds what is stored rather than rebuilt)
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   Workspace ws;

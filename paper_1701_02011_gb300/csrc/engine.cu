@@ -394,7 +394,10 @@ void run_gemm(Workspace& ws, const GemmArgs& g0, int kind) {
 
 namespace {
 void run_gemm_fp64(Workspace& ws, const GemmArgs& g0, int kind) {
-  if (kind == K_GEMM && gemm_use_flat(g0)) {
+  // the ladder's products too while they are small: its tiles of a 16-orbital
+  // particle space took 77 + 40 us on 16 CTAs
+  const double fl = 2.0 * (double)g0.M * (double)g0.N * (double)g0.K;
+  if ((kind == K_GEMM || fl < 2e8) && gemm_use_flat(g0)) {
     FlatTable tab{};
     tab.a[0] = g0.A;
     tab.b[0] = g0.B;
@@ -409,8 +412,8 @@ void run_gemm_fp64(Workspace& ws, const GemmArgs& g0, int kind) {
   // Few output tiles but a long contraction: split K over extra CTAs so the
   // whole GPU works on it (partials reduced in a fixed order).  Tiny outputs
   // go to the one-CTA-per-element kernel instead.
-  int bm = 64, bn = 64;
-  if (kind == K_GEMM) gemm_tile(g.M, g.N, &bm, &bn);
+  int bm, bn;
+  gemm_tile(g.M, g.N, kind == K_LADDER_BUILD ? 1 : kind == K_LADDER_CONTRACT ? 2 : 0, &bm, &bn);
   const long long tiles = ((g.M + bm - 1) / bm) * ((g.N + bn - 1) / bn) * g.nbatch;
   double* part = nullptr;
   size_t cap = 0;

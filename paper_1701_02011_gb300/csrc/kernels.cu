@@ -745,7 +745,15 @@ inline int grid_for(long long n, int threads, int cap = 152 * 16) {
 }
 }  // namespace
 
-void gemm_tile(long long M, long long N, int* bm, int* bn) {
+void gemm_tile(long long M, long long N, int kind, int* bm, int* bn) {
+  if (kind != 0) {
+    // the DF build and the ladder contraction: 64 x 64, or 128 x 32 where the
+    // last column tile of 64 would be mostly padding (N = 136: 192 against 160)
+    const long long w64 = (N + 63) / 64 * 64, w32 = (N + 31) / 32 * 32;
+    *bm = w64 * 10 > w32 * 11 ? 128 : 64;
+    *bn = *bm == 128 ? 32 : 64;
+    return;
+  }
   if (N <= 16) { *bm = 256; *bn = 16; }
   else if (M <= 16) { *bm = 16; *bn = 256; }
   else if (N <= 32) { *bm = 128; *bn = 32; }
@@ -828,8 +836,7 @@ void launch_gemm_flat(const GemmArgs& g, const FlatPlan& p, const FlatTable& tab
 void launch_gemm(const GemmArgs& g, cudaStream_t st, int kind) {
   if (g.M <= 0 || g.N <= 0 || g.K <= 0 || g.nbatch <= 0) return;
   int bm, bn;
-  gemm_tile(g.M, g.N, &bm, &bn);
-  if (kind != 0) { bm = 64; bn = 64; }
+  gemm_tile(g.M, g.N, kind, &bm, &bn);
   dim3 grid((unsigned)((g.M + bm - 1) / bm), (unsigned)((g.N + bn - 1) / bn),
             (unsigned)(g.splits > 1 ? g.splits : g.nbatch));
   if (kind == 0 && gemm_is_small(g)) {
@@ -845,7 +852,8 @@ void launch_gemm(const GemmArgs& g, cudaStream_t st, int kind) {
     k_gemm_tpo<<<grid_for(g.M * g.N * g.nbatch, TPO_T, 152 * 32), TPO_T, 0, st>>>(g, sm < sn ? 1 : 0);
     return;
   }
-  if (kind == 1) k_gemm<64, 64, 1><<<grid, NT, 0, st>>>(g);        // (pr|qs) build from B
+  if (kind != 0 && bn == 32) k_gemm<128, 32, 0><<<grid, NT, 0, st>>>(g);
+  else if (kind == 1) k_gemm<64, 64, 1><<<grid, NT, 0, st>>>(g);        // (pr|qs) build from B
   else if (kind == 2) k_gemm<64, 64, 2><<<grid, NT, 0, st>>>(g);   // ladder contraction with T2
   else if (bn == 16) k_gemm<256, 16, 0><<<grid, NT, 0, st>>>(g);    // narrow outputs
   else if (bm == 16) k_gemm<16, 256, 0><<<grid, NT, 0, st>>>(g);

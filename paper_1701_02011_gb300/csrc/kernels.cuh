@@ -99,9 +99,9 @@ void launch_axpy_blocks(const NdArgs& g, double alpha, const AxpyBlocks& p, cuda
 // afterwards; no CTA waits) adds them in a fixed order.
 void launch_dot_blocks(const NdArgs& g, double alpha, const DotBlocks& p, double* scratch, int scratch_len,
                        unsigned* ticket, double* out, cudaStream_t st);
-// Output tile of the generic contraction for an M x N output (kinds 1, 2
-// always use 64 x 64).
-void gemm_tile(long long M, long long N, int* bm, int* bn);
+// Output tile of the generic contraction for an M x N output (kind as in
+// launch_gemm).
+void gemm_tile(long long M, long long N, int kind, int* bm, int* bn);
 // true when the output is small enough for one CTA per output element
 bool gemm_is_small(const GemmArgs& g);
 // true when K is short enough for one thread per output element

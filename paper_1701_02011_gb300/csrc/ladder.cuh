@@ -20,6 +20,14 @@ void ladder_core(const double* B, long long n, int naux, int p0, int np, int nh,
 void ladder_core_sym(const double* B, long long n, int naux, int p0, int np, int nh, const double* t,
                      const long long* tst, double* L, double* G, long long max_doubles, cudaStream_t st,
                      Workspace* ws);
+// The same sums in pair form (see ladder.cu); false, and nothing done, where
+// the memory named does not suffice.  _pairs: B symmetric in its last two
+// indices and t as for ladder_core_sym; _general: any B and t (contiguous).
+// L is overwritten.
+bool ladder_core_pairs(const double* B, long long n, int naux, int p0, int np, int nh, const double* t,
+                       const long long* tst, double* L, long long max_doubles, double m_bytes, Workspace& ws);
+bool ladder_core_general(const double* B, long long n, int naux, int p0, int np, int nh, const double* t, double* L,
+                         long long max_doubles, Workspace& ws);
 // Largest batch of p rows whose (pr|qs) fits in max_doubles (0 if none).
 long long ladder_batch_rows(int np, long long max_doubles);
 int ladder_check_args(int n, int naux, int p0, int np, int nh, const void* B, const void* t, const void* L,
