@@ -365,8 +365,25 @@ bool split_route(Workspace& ws, const GemmArgs& g) {
 
 // one flat launch over the output blocks of tab (npairs operand pairs)
 void run_gemm_flat(Workspace& ws, const GemmArgs& g, const FlatTable& tab, int npairs) {
-  const FlatPlan fp = gemm_flat_plan(g, tab.ngroups);
   const size_t O = (size_t)(g.M * g.N * g.nbatch);
+  if (gemm_use_narrow(g)) {
+    const NarrowPlan np = gemm_narrow_plan(g, tab.ngroups);
+    double* npart = nullptr;
+    size_t ncap = 0;
+    if (np.z > 1) npart = ws.get((size_t)tab.ngroups * np.z * O, ncap);
+    const int r = ws.begin(K_GEMM, 2.0 * (double)g.M * (double)g.N * (double)g.K * npairs, 0.0);
+    if (r >= 0) {
+      ws.recs[r].m = g.M;
+      ws.recs[r].n = g.N;
+      ws.recs[r].k = g.K * npairs;
+    }
+    launch_gemm_narrow(g, np, tab, npart, ws.stream);
+    ws.end(r);
+    if (np.z > 1) ws.launches++;
+    if (npart) ws.put(npart, ncap);
+    return;
+  }
+  const FlatPlan fp = gemm_flat_plan(g, tab.ngroups);
   double* fpart = nullptr;
   size_t fcap = 0;
   if (fp.z > 1) fpart = ws.get((size_t)tab.ngroups * fp.z * O, fcap);

@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cmath>
 #include <stdexcept>
+#include <type_traits>
 
 namespace dsrg {
 
@@ -422,6 +423,133 @@ __global__ void k_gemm_flat_reduce(const GemmArgs g, const FlatK fk, const FlatT
   }
 }
 
+// Narrow contraction: outputs with one short side of at most NS <= 48.  A thread
+// owns one index m of the long side and keeps all its NS sums in registers,
+// so each element of the long operand is read once (the flat kernel reads it
+// once per output column: at 11236 x 36 x 2560 the long operand does not fit
+// L2 and the FP64 units ran at 0.57 of 1.26 TFLOP/s).  The short operand goes
+// through shared memory NKB k at a time and is read by broadcast; lanes walk
+// m.  gridDim.y > 1: k chunks, partials reduced as for the flat kernel.
+// Outputs leave through shared memory so that consecutive lanes touch
+// consecutive elements of C whichever side is contiguous there.
+// 11236 x 36 x 2560: 3.6 -> 0.91 ms; 1722112 x 8 x 48 (six spin blocks of k = 8):
+// 1.75 -> 1.24 ms, of 1.05 ms at the FP64 rate.
+constexpr int NARROW_T = 128, NKB = 32, NARROW_EPC = 4;
+template <int NS>
+__global__ void __launch_bounds__(NARROW_T) k_gemm_narrow(const NarrowArgs a, const FlatTable tab, double* part) {
+  __shared__ double Bs[NKB][NS];
+  __shared__ long long ka[NKB], kb[NKB], nb[NS], nc[NS], mc[NARROW_T];
+  __shared__ double stg[NARROW_T][NARROW_EPC + 1];
+  const int tid = threadIdx.x;
+  const unsigned m = blockIdx.x * (unsigned)NARROW_T + tid;
+  const bool live = m < (unsigned)a.M;
+  auto offsets = [](unsigned lin, int nd, const FastDiv* f, const long long* s1, const long long* s2, long long& o1,
+                    long long& o2) {
+    o1 = 0;
+    o2 = 0;
+    for (int d = nd - 1; d >= 0; --d) {
+      const unsigned q = fast_div(lin, f[d]);
+      const long long r = lin - q * f[d].d;
+      o1 += r * s1[d];
+      o2 += r * s2[d];
+      lin = q;
+    }
+  };
+  long long am = 0, cm = 0;
+  if (live) offsets(m, a.nM, a.fm, a.aM, a.cM, am, cm);
+  mc[tid] = live ? cm : -1;
+  for (int n = tid; n < NS; n += NARROW_T) {
+    long long o1 = -1, o2 = -1;
+    if (n < a.N) offsets((unsigned)n, a.nN, a.fn, a.bN, a.cN, o1, o2);
+    nb[n] = o1;
+    nc[n] = o2;
+  }
+  const long long klo = blockIdx.y * a.len, khi = klo + a.len < a.K ? klo + a.len : a.K;
+  const int grp = blockIdx.z;
+  double acc[NS];
+#pragma unroll
+  for (int n = 0; n < NS; ++n) acc[n] = 0.0;
+  for (long long k0 = klo; k0 < khi; k0 += NKB) {
+    const int nk = khi - k0 < NKB ? (int)(khi - k0) : NKB;
+    __syncthreads();  // the last chunk's tables and B are no longer read
+    if (tid < nk) {
+      long long o1, o2;
+      offsets((unsigned)(k0 + tid), a.nK, a.fk, a.aK, a.bK, o1, o2);
+      ka[tid] = o1;
+      kb[tid] = o2;
+    }
+    for (int pr = tab.first[grp]; pr < tab.first[grp + 1]; ++pr) {
+      const double* __restrict__ B = tab.b[pr];
+      const double* __restrict__ A = tab.a[pr] + am;
+      __syncthreads();
+      for (int e = tid; e < nk * NS; e += NARROW_T) {
+        const int k = a.bkfast ? e % nk : e / NS, n = a.bkfast ? e / nk : e % NS;
+        Bs[k][n] = nb[n] >= 0 ? __ldg(B + kb[k] + nb[n]) : 0.0;
+      }
+      __syncthreads();
+      if (!live) continue;
+      int k = 0;
+      for (; k + 4 <= nk; k += 4) {
+        double x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = __ldg(A + ka[k + u]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int n = 0; n < NS; ++n) acc[n] = fma(x[u], Bs[k + u][n], acc[n]);
+      }
+      for (; k < nk; ++k) {
+        const double x = __ldg(A + ka[k]);
+#pragma unroll
+        for (int n = 0; n < NS; ++n) acc[n] = fma(x, Bs[k][n], acc[n]);
+      }
+    }
+  }
+  // write-back, NARROW_EPC columns at a time through this warp's staging rows
+  const int warp = tid >> 5, lane = tid & 31;
+  __syncthreads();
+  double* C = gridDim.y > 1 ? part + ((long long)grp * gridDim.y + blockIdx.y) * a.M * a.N : tab.c[grp];
+#pragma unroll
+  for (int c0 = 0; c0 < NS; c0 += NARROW_EPC) {
+#pragma unroll
+    for (int j = 0; j < NARROW_EPC; ++j) stg[tid][j] = acc[c0 + j];
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < NARROW_EPC; ++j) {
+      const int i = j * 32 + lane;
+      const int r = warp * 32 + (a.cmfast ? lane : i / NARROW_EPC), c = c0 + (a.cmfast ? j : i % NARROW_EPC);
+      const double v = stg[r][c - c0];
+      if (mc[r] < 0 || nc[c] < 0) continue;
+      if (gridDim.y > 1) C[(long long)(blockIdx.x * (unsigned)NARROW_T + r) * a.N + c] = v;
+      else C[mc[r] + nc[c]] += a.alpha * v;
+    }
+    __syncwarp();
+  }
+}
+
+// C_grp[m, n] += alpha * sum_z part[grp][z][m][n], z in increasing order
+__global__ void k_gemm_narrow_reduce(const NarrowArgs a, const FlatTable tab, int Z, const double* part) {
+  const int grp = blockIdx.y;
+  const long long O = a.M * a.N;
+  for (long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x; o < O; o += (long long)gridDim.x * blockDim.x) {
+    double s = 0.0;
+    for (int z = 0; z < Z; ++z) s += part[((long long)grp * Z + z) * O + o];
+    unsigned m = (unsigned)(o / a.N), n = (unsigned)(o - (long long)m * a.N);
+    long long oc = 0;
+    for (int d = a.nM - 1; d >= 0; --d) {
+      const unsigned q = fast_div(m, a.fm[d]);
+      oc += (long long)(m - q * a.fm[d].d) * a.cM[d];
+      m = q;
+    }
+    for (int d = a.nN - 1; d >= 0; --d) {
+      const unsigned q = fast_div(n, a.fn[d]);
+      oc += (long long)(n - q * a.fn[d].d) * a.cN[d];
+      n = q;
+    }
+    tab.c[grp][oc] += a.alpha * s;
+  }
+}
+
 // C[m, n] += alpha * sum_z part[z][m][n], z in increasing order
 __global__ void k_gemm_splitk_reduce(const GemmArgs g) {
   const long long MN = g.M * g.N;
@@ -471,14 +599,50 @@ __device__ __forceinline__ void nd_off(const NdArgs& g, long long lin, long long
   }
 }
 
-template <bool FAST>
-__global__ void k_axpy(const NdArgs g, double alpha, const double* __restrict__ A, double* __restrict__ C) {
+// V consecutive doubles, 16 bytes at a time (V > 1: 16-byte aligned)
+template <int V>
+__device__ __forceinline__ void load_run(const double* p, double (&x)[V]) {
+  if (V == 1) {
+    x[0] = *p;
+  } else {
+#pragma unroll
+    for (int v = 0; v < V; v += 2) {
+      const double2 t = *reinterpret_cast<const double2*>(p + v);
+      x[v] = t.x;
+      x[v + 1] = t.y;
+    }
+  }
+}
+template <int V>
+__device__ __forceinline__ void store_run(double* p, const double (&x)[V]) {
+  if (V == 1) {
+    *p = x[0];
+  } else {
+#pragma unroll
+    for (int v = 0; v < V; v += 2) *reinterpret_cast<double2*>(p + v) = make_double2(x[v], x[v + 1]);
+  }
+}
+
+// C += alpha A; an index of g stands for V consecutive elements (nd_runs)
+template <bool FAST, int V>
+__device__ __forceinline__ void axpy_items(const NdArgs& g, double alpha, const double* __restrict__ A,
+                                           double* __restrict__ C) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < g.total;
        i += (long long)gridDim.x * blockDim.x) {
     long long oa, oc;
     nd_off<FAST>(g, i, oa, oc);
-    C[oc] += alpha * A[oa];
+    double a[V], c[V];
+    load_run<V>(A + oa, a);
+    load_run<V>(C + oc, c);
+#pragma unroll
+    for (int v = 0; v < V; ++v) c[v] += alpha * a[v];
+    store_run<V>(C + oc, c);
   }
+}
+
+template <bool FAST, int V>
+__global__ void k_axpy(const NdArgs g, double alpha, const double* __restrict__ A, double* __restrict__ C) {
+  axpy_items<FAST, V>(g, alpha, A, C);
 }
 
 // Compensated (Neumaier) per-thread sums, then a fixed-order tree.
@@ -491,16 +655,9 @@ __device__ __forceinline__ void neumaier(double& s, double& c, double x) {
 
 constexpr int DOT_THREADS = 256;
 
-template <bool FAST>
+template <bool FAST, int V>
 __global__ void k_axpy_blocks(const NdArgs g, double alpha, const AxpyBlocks p) {
-  const double* __restrict__ A = p.a[blockIdx.y];
-  double* __restrict__ C = p.c[blockIdx.y];
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < g.total;
-       i += (long long)gridDim.x * blockDim.x) {
-    long long oa, oc;
-    nd_off<FAST>(g, i, oa, oc);
-    C[oc] += alpha * A[oa];
-  }
+  axpy_items<FAST, V>(g, alpha, p.a[blockIdx.y], p.c[blockIdx.y]);
 }
 
 // fixed-order compensated tree over the DOT_THREADS pairs (s, c) in shared memory
@@ -517,7 +674,13 @@ __device__ __forceinline__ void dot_tree(double* sh_s, double* sh_c) {
   }
 }
 
-template <bool FAST>
+// The terms go into a running sum s and a correction c with four FP64
+// operations a term: with t = fma(a, b, s), fma(a, b, s - t) is what the sum
+// and the product lost, exactly where |s| >= |a b| and to a rounding of t
+// elsewhere (a plain product would lose as much on every term).  The FP64
+// pipe bounds this kernel (two operations a clock and SM), not memory; with
+// a rounded product and Neumaier's branch it took six.
+template <bool FAST, int V>
 __global__ void __launch_bounds__(DOT_THREADS) k_dot_blocks(const NdArgs g, const DotBlocks p, double* partial,
                                                            unsigned* ticket, double alpha, double* out) {
   const double* __restrict__ A = p.a[blockIdx.y];
@@ -527,7 +690,15 @@ __global__ void __launch_bounds__(DOT_THREADS) k_dot_blocks(const NdArgs g, cons
        i += (long long)gridDim.x * blockDim.x) {
     long long oa, ob;
     nd_off<FAST>(g, i, oa, ob);
-    neumaier(s, c, A[oa] * B[ob]);
+    double a[V], b[V];
+    load_run<V>(A + oa, a);
+    load_run<V>(B + ob, b);
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      const double t = fma(a[v], b[v], s);
+      c += fma(a[v], b[v], s - t);
+      s = t;
+    }
   }
   __shared__ double sh_s[DOT_THREADS], sh_c[DOT_THREADS];
   __shared__ bool last;
@@ -833,6 +1004,71 @@ void launch_gemm_flat(const GemmArgs& g, const FlatPlan& p, const FlatTable& tab
   }
 }
 
+bool gemm_use_narrow(const GemmArgs& g) {
+  // one short side of at most 48 (its sums fit a thread's registers) and a
+  // long one that gives at least a warp to every SM; k long enough to pay for
+  // the tables.  At most 32 k chunks (65535 column blocks are never reached).
+  const long long s = g.M < g.N ? g.M : g.N, l = g.M < g.N ? g.N : g.M;
+  return g.nbatch == 1 && s >= 3 && s <= 48 && l >= 152 * 32 && l < (1LL << 31) && g.K >= 4 && g.K < (1LL << 31);
+}
+
+NarrowPlan gemm_narrow_plan(const GemmArgs& g, int groups) {
+  NarrowPlan p{};
+  const long long l = g.M < g.N ? g.N : g.M;
+  const long long ctas = (l + NARROW_T - 1) / NARROW_T * (groups > 1 ? groups : 1);
+  // about four CTAs per SM, at least 4 NKB of k each
+  long long z = (4 * 152 + ctas - 1) / ctas;
+  if (z > g.K / (4 * NKB)) z = g.K / (4 * NKB);
+  if (z > 32) z = 32;
+  if (z < 1) z = 1;
+  p.len = (g.K + z - 1) / z;
+  p.z = (int)((g.K + p.len - 1) / p.len);
+  return p;
+}
+
+void launch_gemm_narrow(const GemmArgs& g, const NarrowPlan& p, const FlatTable& tab0, double* part, cudaStream_t st) {
+  if (g.M <= 0 || g.N <= 0 || g.K <= 0 || tab0.ngroups <= 0) return;
+  const bool swap = g.N > g.M;  // the long side is m
+  NarrowArgs a{};
+  FlatTable tab = tab0;
+  a.nM = swap ? g.nN : g.nM;
+  a.nN = swap ? g.nM : g.nN;
+  a.nK = g.nK;
+  a.M = swap ? g.N : g.M;
+  a.N = swap ? g.M : g.N;
+  a.K = g.K;
+  a.len = p.len;
+  a.alpha = g.alpha;
+  for (int d = 0; d < 4; ++d) {
+    a.fm[d] = make_fastdiv(d < a.nM ? (unsigned)(swap ? g.eN[d] : g.eM[d]) : 1u);
+    a.fn[d] = make_fastdiv(d < a.nN ? (unsigned)(swap ? g.eM[d] : g.eN[d]) : 1u);
+    a.fk[d] = make_fastdiv(d < a.nK ? (unsigned)g.eK[d] : 1u);
+    a.aM[d] = swap ? g.bN[d] : g.aM[d];
+    a.cM[d] = swap ? g.cN[d] : g.cM[d];
+    a.aK[d] = swap ? g.bK[d] : g.aK[d];
+    a.bN[d] = swap ? g.aM[d] : g.bN[d];
+    a.cN[d] = swap ? g.cM[d] : g.cN[d];
+    a.bK[d] = swap ? g.aK[d] : g.bK[d];
+  }
+  if (swap)
+    for (int i = 0; i < kFlatMaxPairs; ++i) std::swap(tab.a[i], tab.b[i]);
+  a.bkfast = a.nK > 0 && (a.nN == 0 || a.bK[a.nK - 1] < a.bN[a.nN - 1]);
+  a.cmfast = a.nM > 0 && (a.nN == 0 || a.cM[a.nM - 1] < a.cN[a.nN - 1]);
+  const dim3 grid((unsigned)((a.M + NARROW_T - 1) / NARROW_T), (unsigned)p.z, (unsigned)tab.ngroups);
+  switch ((int)((a.N + 3) / 4)) {
+#define DSRG_NARROW(n) \
+  case n: k_gemm_narrow<4 * n><<<grid, NARROW_T, 0, st>>>(a, tab, part); break;
+    DSRG_NARROW(1) DSRG_NARROW(2) DSRG_NARROW(3) DSRG_NARROW(4) DSRG_NARROW(5) DSRG_NARROW(6)
+    DSRG_NARROW(7) DSRG_NARROW(8) DSRG_NARROW(9) DSRG_NARROW(10) DSRG_NARROW(11)
+    default: k_gemm_narrow<48><<<grid, NARROW_T, 0, st>>>(a, tab, part); break;
+#undef DSRG_NARROW
+  }
+  if (p.z > 1) {
+    const dim3 rg((unsigned)grid_for(a.M * a.N, 256, (152 * 16 + tab.ngroups - 1) / tab.ngroups), (unsigned)tab.ngroups);
+    k_gemm_narrow_reduce<<<rg, 256, 0, st>>>(a, tab, p.z, part);
+  }
+}
+
 void launch_gemm(const GemmArgs& g, cudaStream_t st, int kind) {
   if (g.M <= 0 || g.N <= 0 || g.K <= 0 || g.nbatch <= 0) return;
   int bm, bn;
@@ -888,30 +1124,93 @@ void nd_order(NdArgs& g, long long wb) {
   }
 }
 
-// orders the dimensions and fills the fast divisors; true when every linear
-// index fits 31 bits
-bool nd_prepare(NdArgs& g, long long wb) {
+// Joins neighbouring dimensions that are one run in both operands, and makes
+// an index stand for V = 4 or 2 consecutive elements where the last dimension
+// is contiguous in both, a multiple of V long, and every run 16-byte aligned
+// (aligned: the base pointers are): fewer divisions an element and 16-byte
+// accesses.  Returns V.
+int nd_runs(NdArgs& g, bool aligned) {
+  int nd = 0;
+  for (int d = 0; d < g.nd; ++d) {  // extents of one go
+    if (g.e[d] == 1) continue;
+    g.e[nd] = g.e[d];
+    g.sa[nd] = g.sa[d];
+    g.sb[nd++] = g.sb[d];
+  }
+  g.nd = nd;
+  for (int d = g.nd - 1; d > 0; --d) {
+    const bool run = g.sa[d - 1] == g.e[d] * g.sa[d] && g.sb[d - 1] == g.e[d] * g.sb[d] &&
+                     (long long)g.e[d - 1] * g.e[d] < (1LL << 30);
+    if (!run) continue;
+    g.e[d - 1] *= g.e[d];
+    g.sa[d - 1] = g.sa[d];
+    g.sb[d - 1] = g.sb[d];
+    for (int k = d; k + 1 < g.nd; ++k) {
+      g.e[k] = g.e[k + 1];
+      g.sa[k] = g.sa[k + 1];
+      g.sb[k] = g.sb[k + 1];
+    }
+    --g.nd;
+  }
+  const int last = g.nd - 1;
+  if (last < 0 || !aligned || g.sa[last] != 1 || g.sb[last] != 1 || g.e[last] % 2) return 1;
+  for (int d = 0; d < last; ++d)
+    if (g.sa[d] % 2 || g.sb[d] % 2) return 1;
+  const int V = g.e[last] % 4 ? 2 : 4;
+  g.e[last] /= V;
+  g.sa[last] = g.sb[last] = V;
+  g.total /= V;
+  return V;
+}
+
+bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
+
+// orders the dimensions, forms runs (V elements an index) and fills the fast
+// divisors; true when every linear index fits 31 bits
+bool nd_prepare(NdArgs& g, long long wb, bool aligned, int& V) {
   nd_order(g, wb);
+  V = nd_runs(g, aligned);
   if (g.total >= (1LL << 31)) return false;
   for (int d = 0; d < g.nd; ++d) g.fe[d] = make_fastdiv((unsigned)g.e[d]);
   return true;
 }
 }  // namespace
 
+namespace {
+// f(V as a constant, FAST as a constant)
+template <class F>
+void nd_dispatch(bool fast, int V, F&& f) {
+  auto with = [&](auto v) {
+    if (fast) f(v, std::true_type{});
+    else f(v, std::false_type{});
+  };
+  if (V == 4) with(std::integral_constant<int, 4>{});
+  else if (V == 2) with(std::integral_constant<int, 2>{});
+  else with(std::integral_constant<int, 1>{});
+}
+}  // namespace
+
 void launch_axpy(const NdArgs& g0, double alpha, const double* A, double* C, cudaStream_t st) {
   if (g0.total <= 0) return;
   NdArgs g = g0;
-  if (nd_prepare(g, 2)) k_axpy<true><<<grid_for(g.total, 256), 256, 0, st>>>(g, alpha, A, C);
-  else k_axpy<false><<<grid_for(g.total, 256), 256, 0, st>>>(g, alpha, A, C);
+  int V;
+  const bool fast = nd_prepare(g, 2, aligned16(A) && aligned16(C), V);
+  nd_dispatch(fast, V, [&](auto v, auto f) {
+    k_axpy<decltype(f)::value, decltype(v)::value><<<grid_for(g.total, 256), 256, 0, st>>>(g, alpha, A, C);
+  });
 }
 
 void launch_axpy_blocks(const NdArgs& g0, double alpha, const AxpyBlocks& p, cudaStream_t st) {
   if (g0.total <= 0 || p.n <= 0) return;
   NdArgs g = g0;
-  const int gx = grid_for(g.total, 256, (152 * 16 + p.n - 1) / p.n);
-  const dim3 grid((unsigned)gx, (unsigned)p.n);
-  if (nd_prepare(g, 2)) k_axpy_blocks<true><<<grid, 256, 0, st>>>(g, alpha, p);
-  else k_axpy_blocks<false><<<grid, 256, 0, st>>>(g, alpha, p);
+  bool al = true;
+  for (int k = 0; k < p.n; ++k) al = al && aligned16(p.a[k]) && aligned16(p.c[k]);
+  int V;
+  const bool fast = nd_prepare(g, 2, al, V);
+  const dim3 grid((unsigned)grid_for(g.total, 256, (152 * 16 + p.n - 1) / p.n), (unsigned)p.n);
+  nd_dispatch(fast, V, [&](auto v, auto f) {
+    k_axpy_blocks<decltype(f)::value, decltype(v)::value><<<grid, 256, 0, st>>>(g, alpha, p);
+  });
 }
 
 void launch_dot_blocks(const NdArgs& g0, double alpha, const DotBlocks& p, double* scratch, int scratch_len,
@@ -920,10 +1219,16 @@ void launch_dot_blocks(const NdArgs& g0, double alpha, const DotBlocks& p, doubl
   NdArgs g = g0;
   int cap = scratch_len / 2 / p.n;
   if (cap < 1) throw std::runtime_error("dot: scratch too small for the spin blocks");
+  bool al = true;
+  for (int k = 0; k < p.n; ++k) al = al && aligned16(p.a[k]) && aligned16(p.b[k]);
+  int V = 1;
+  const bool fast = nd_prepare(g, 1, al, V);
   const int gx = grid_for(g.total > 0 ? g.total : 1, DOT_THREADS, cap);
   const dim3 grid((unsigned)gx, (unsigned)p.n);
-  if (nd_prepare(g, 1)) k_dot_blocks<true><<<grid, DOT_THREADS, 0, st>>>(g, p, scratch, ticket, alpha, out);
-  else k_dot_blocks<false><<<grid, DOT_THREADS, 0, st>>>(g, p, scratch, ticket, alpha, out);
+  nd_dispatch(fast, V, [&](auto v, auto f) {
+    k_dot_blocks<decltype(f)::value, decltype(v)::value>
+        <<<grid, DOT_THREADS, 0, st>>>(g, p, scratch, ticket, alpha, out);
+  });
 }
 
 void launch_sum_slots(const double* slots, const int* r, double* out, cudaStream_t st) {

@@ -131,6 +131,23 @@ bool gemm_use_flat(const GemmArgs& g);
 FlatPlan gemm_flat_plan(const GemmArgs& g, int groups = 1);
 // part needs groups * z * M*N*nbatch doubles when the plan has z > 1
 void launch_gemm_flat(const GemmArgs& g, const FlatPlan& p, const FlatTable& tab, double* part, cudaStream_t st);
+// Narrow contraction: an output with a short side of at most 48 and a long one.
+// part needs groups * z * M*N doubles when the plan has z > 1.
+struct NarrowArgs {
+  int nM, nN, nK;
+  FastDiv fm[4], fn[4], fk[4];
+  long long aM[4], cM[4], aK[4], bN[4], cN[4], bK[4];
+  long long M, N, K, len;  // M long, N short; k per chunk
+  double alpha;
+  int bkfast, cmfast;  // B's contiguous index is k; C's is m
+};
+struct NarrowPlan {
+  int z;          // k chunks
+  long long len;  // k per chunk
+};
+bool gemm_use_narrow(const GemmArgs& g);
+NarrowPlan gemm_narrow_plan(const GemmArgs& g, int groups);
+void launch_gemm_narrow(const GemmArgs& g, const NarrowPlan& p, const FlatTable& tab, double* part, cudaStream_t st);
 // kind 0: generic contraction, 1: DF build of (pr|qs), 2: ladder contraction
 void launch_gemm(const GemmArgs& g, cudaStream_t st, int kind = 0);
 void launch_fill(double* p, long long n, double v, cudaStream_t st);
