@@ -7,6 +7,7 @@
 #include "ozaki.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <map>
 #include <mutex>
 #include <type_traits>
@@ -113,8 +114,11 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
                : "memory");
 }
 
-// *p += v without a load of *p into the SM (one addition per element and
-// launch, so the result does not depend on any order)
+// *p += v in L2, off the FP64 pipe and without a load into the SM (one addition
+// per element and launch, so the result does not depend on any order).  It goes
+// at about 110 G/s on the whole chip, which bounds the short-k products; loads,
+// additions and stores by the summing warps were slower at every width (1722112 x
+// 28 x 8: 550 against 513 us, 61504 x 784 x 64: 570 against 450 us).
 __device__ __forceinline__ void red_add(double* p, double v) {
   asm volatile("red.global.add.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
 }
@@ -174,6 +178,10 @@ struct OzArgs {
   int S, MT, NT, KT;
   long long M, N;
   double alpha;
+  // alpha = +-2^alpha_exp (its effect is on sign and exponent) unless alpha_mul;
+  // split-k partials carry no alpha
+  int alpha_exp;
+  bool alpha_neg, alpha_mul;
   double* C;
   // C offsets: row m -> decoded with (nM, eM, cM), column n -> (nN, eN, cN)
   int nM, nN;
@@ -187,7 +195,8 @@ struct OzArgs {
   // scaled partial tile to part[z][MT*128][NT*BN] instead of C
   int splits, ktper;
   double* part;
-  long long tiles;  // MT * NT * splits
+  unsigned tiles;   // MT * NT * splits < 2^31
+  FastDiv f_z, f_group, f_full, f_tail;  // divisors of the work list (oz_tile)
   int nbuf;         // stage buffers
 };
 
@@ -201,9 +210,10 @@ __device__ __forceinline__ long long c_offset(long long lin, int nd, const int* 
   return o;
 }
 
-// barrier 1 over the 8 warps of the tile (the copy warp does not take part);
-// the _and form returns whether every thread's pred was true
-__device__ __forceinline__ void tile_sync() { asm volatile("bar.sync 1, %0;" ::"n"(OZ_THREADS) : "memory"); }
+// barrier 1 over the 8 warps of the tile; whether every thread's pred was true
+// barrier 2: the tile's warps and the two that write its tables.  Every one
+// of them passes it once per tile, whatever happened before.
+__device__ __forceinline__ void table_sync() { asm volatile("bar.sync 2, %0;" ::"n"(OZ_THREADS + 64) : "memory"); }
 __device__ __forceinline__ bool tile_sync_and(bool pred) {
   uint32_t r;
   asm volatile(
@@ -242,60 +252,64 @@ __device__ __forceinline__ void oz_issue(uint32_t tm, uint64_t dA, uint64_t dB) 
 // tile `lin` of the work list -> (k split z, row tile, column tile).  Grouped
 // rasterisation: consecutive tiles walk the columns of a group of OZ_GROUP row
 // tiles, so the CTAs running together share their digit tiles in L2.
-__device__ __forceinline__ void oz_tile(const OzArgs& a, long long lin, int& z, int& mt, int& nt) {
-  const long long per_z = (long long)a.MT * a.NT;
-  z = (int)(lin / per_z);
-  const long long l = lin - z * per_z;
-  const long long per = (long long)OZ_GROUP * a.NT;
-  const int first = (int)(l / per) * OZ_GROUP;
-  const int gm = a.MT - first < OZ_GROUP ? a.MT - first : OZ_GROUP;
-  const int within = (int)(l - (l / per) * per);
-  mt = first + within % gm;
-  nt = within / gm;
+__device__ __forceinline__ void oz_tile(const OzArgs& a, unsigned lin, int& z, int& mt, int& nt) {
+  const unsigned zz = fast_div(lin, a.f_z), l = lin - zz * a.f_z.d;
+  const unsigned grp = fast_div(l, a.f_group), within = l - grp * a.f_group.d;
+  const bool tail = (int)(grp + 1) * OZ_GROUP > a.MT;
+  const FastDiv& f = tail ? a.f_tail : a.f_full;  // row tiles of this group
+  const unsigned c = fast_div(within, f);
+  z = (int)zz;
+  mt = (int)(grp * OZ_GROUP + within - c * f.d);
+  nt = (int)c;
 }
 
-// (top 2^SH + bot) 2^k as a double, assembled with integer instructions and
-// rounded to nearest (bits beyond the 64th are dropped): the FP64 pipe has two
-// lanes a clock, and a conversion or an addition per element would bind it.
+// (top 2^SH + bot) 2^k, negated if flip, as a double, assembled with integer
+// instructions and rounded to nearest (bits beyond the 64th are dropped): the
+// FP64 pipe has two lanes a clock.  No branches, so that several elements
+// overlap (with branches a 128 x 32 tile's 16 elements a lane took 8400 clocks);
+// odd is set where the result is subnormal or out of range (oz_value_odd).
 template <int SH>
-__device__ __forceinline__ double oz_value(long long top, long long bot, int k) {
-  // 128-bit two's complement hi:lo = (top << SH) + bot
+__device__ __forceinline__ double oz_value(long long top, long long bot, int k, bool flip, bool& odd) {
+  // 128-bit two's complement hi:lo = (top << SH) + bot, then its magnitude
   unsigned long long lo = (unsigned long long)top << SH;
   long long hi = top >> (SH ? 64 - SH : 63);
-  const unsigned long long l2 = lo + (unsigned long long)bot;
-  hi += (bot >> 63) + (l2 < lo ? 1 : 0);
-  lo = l2;
-  const bool neg = hi < 0;
-  if (neg) {
-    lo = 0ULL - lo;
-    hi = ~hi + (lo == 0 ? 1 : 0);
-  }
-  int e = k;
-  unsigned long long m = lo;
-  if (hi) {
-    const int n = __clzll(hi);  // hi >= 0 here, n >= 1
-    m = ((unsigned long long)hi << n) | (lo >> (64 - n));
-    e += 64 - n;
-  } else {
-    if (!lo) return 0.0;
-    const int n = __clzll((long long)lo);
-    m = lo << n;
-    e -= n;
-  }
-  // m in [2^63, 2^64): value m 2^e
+  lo += (unsigned long long)bot;
+  hi += (bot >> 63) + (lo < (unsigned long long)bot ? 1 : 0);
+  const unsigned long long neg = (unsigned long long)(hi >> 63);
+  lo ^= neg;
+  hi ^= (long long)neg;
+  lo -= neg;
+  hi += neg && lo == 0 ? 1 : 0;
+  // its leading 64 bits m in [2^63, 2^64), value m 2^e
+  const bool wide = hi != 0;
+  const unsigned long long H = wide ? (unsigned long long)hi : lo, L = wide ? lo : 0ULL;
+  const int n = __clzll((long long)H) & 63;
+  const unsigned long long m = (H << n) | ((L >> 1) >> (63 - n));
+  const int ex = k + (wide ? 64 : 0) - n + 63 + 1023;
   const unsigned long long r = (m >> 11) + ((m >> 10) & 1ULL);  // in [2^52, 2^53]
-  const int ex = e + 63 + 1023;
-  if (ex <= 0 || ex >= 2046) {  // subnormal or out of range: scaled in exact steps but the last
-    double v = (double)(neg ? -(long long)r : (long long)r);
-    for (int s = e + 11; s != 0;) {
-      const int t = s > 1000 ? 1000 : s < -1000 ? -1000 : s;
-      v *= __longlong_as_double((long long)(t + 1023) << 52);
-      s -= t;
+  // the leading bit of r adds one to ex - 1
+  const unsigned long long bits = ((unsigned long long)(unsigned)(ex - 1) << 52) + r;
+  const unsigned long long sign = (neg ^ (flip ? ~0ULL : 0ULL)) & (1ULL << 63);
+  odd = odd || (H != 0 && (ex <= 0 || ex >= 2046));
+  return __longlong_as_double((long long)(H == 0 ? 0ULL : bits | sign));
+}
+
+// the same where it is subnormal or out of range: scaled in exact steps but the last
+template <int SH>
+__device__ __noinline__ double oz_value_odd(long long top, long long bot, int k, bool flip) {
+  // |top 2^SH + bot| < 2^96: two halves, each exact in its own double
+  const long long t = top >> 20, u = ((top & 0xFFFFF) << SH) + bot;
+  double v = 0.0;
+  for (int part = 0; part < 2; ++part) {
+    double w = (double)(part ? u : t);
+    for (int s = (part ? 0 : SH + 20) + k; s != 0;) {
+      const int d = s > 1000 ? 1000 : s < -1000 ? -1000 : s;
+      w *= __longlong_as_double((long long)(d + 1023) << 52);
+      s -= d;
     }
-    return v;
+    v += w;
   }
-  const unsigned long long bits = ((unsigned long long)(ex - 1) << 52) + r;  // the leading bit of r adds one to ex - 1
-  return __longlong_as_double((long long)(bits | (neg ? 1ULL << 63 : 0ULL)));
+  return flip ? -v : v;
 }
 
 // Bounded wait that also gives up once another role of the CTA has.
@@ -314,6 +328,7 @@ __device__ __forceinline__ bool oz_wait(uint64_t* bar, uint32_t phase, long long
 constexpr int OZ_EPC = 8;                  // columns per warp staged at a time in the epilogue
 constexpr int OZ_STAGE_LD = OZ_EPC + 1;    // padded against bank conflicts
 constexpr int OZ_STAGE_BYTES = (OZ_THREADS / 32) * 32 * OZ_STAGE_LD * 8;
+constexpr int OZ_STATIC_BYTES = 6144;     // more than the static tables and barriers take
 
 // Stages per exact window: the level sums over the window must stay within
 // 2^24.  With m the largest sum of squared digits (all slices) over any row's
@@ -329,11 +344,64 @@ __device__ __forceinline__ int oz_window(const OzArgs& a) {
   return n > OZ_WIN ? n : OZ_WIN;
 }
 
+// stages whose level sums stay within 2^22, by the same bound
+__device__ __forceinline__ int oz_quick(const OzArgs& a) {
+  const float p = sqrtf((float)a.sq[0]) * sqrtf((float)a.sq[1]);
+  return (int)fminf(4194304.0f * 0.9999f / fmaxf(p, 1.0f), 1048576.0f);
+}
+
+// Adds a window's level sums to top and bot.  QUICK (sums within 2^22): a sum
+// becomes an integer by an addition of 1.5 2^23, whose bit pattern carries it
+// in the low bits (the constant is taken off at the end); the conversion
+// instruction, needed above that, runs at an eighth of the rate.
+template <int BN, int S, int NCH, int CH, bool QUICK>
+__device__ __forceinline__ void oz_sum(uint32_t taddr, long long (&top)[NCH][CH], long long (&bot)[NCH][CH]) {
+  constexpr int CT = (S + 1) / 2;
+  constexpr int MAGIC = 0x4B400000;  // 1.5 2^23
+  long long bias_top = 0, bias_bot = 0;
+#pragma unroll
+  for (int c = 0; c < S; ++c) {
+    if (c < CT) bias_top += (long long)MAGIC << (7 * (CT - 1 - c));
+    else bias_bot += (long long)MAGIC << (7 * (S - 1 - c));
+  }
+  // chunks of CH columns, PER of them per wait (level by level)
+  constexpr int PER = BN == 32 ? 2 : 1;
+#pragma unroll
+  for (int i0 = 0; i0 < S * NCH; i0 += PER) {
+    uint32_t acc[PER][CH];
+#pragma unroll
+    for (int i = i0; i < i0 + PER && i < S * NCH; ++i)
+      tmem_ld16(taddr + (uint32_t)(i / NCH * BN + i % NCH * CH), acc[i - i0]);
+    tmem_wait_ld();
+#pragma unroll
+    for (int i = i0; i < i0 + PER && i < S * NCH; ++i) {
+      const int c = i / NCH, j = i % NCH;
+#pragma unroll
+      for (int q = 0; q < CH; ++q) {
+        const float f = __uint_as_float(acc[i - i0][q]);
+        const int v = QUICK ? __float_as_int(f + __int_as_float(MAGIC)) : __float2int_rn(f);
+        if (c < CT) top[j][q] += (long long)v * (1 << (7 * (CT - 1 - c)));
+        else bot[j][q] += (long long)v * (1 << (7 * (S - 1 - c)));
+      }
+    }
+  }
+  if (QUICK) {
+#pragma unroll
+    for (int j = 0; j < NCH; ++j)
+#pragma unroll
+      for (int q = 0; q < CH; ++q) {
+        top[j][q] -= bias_top;
+        bot[j][q] -= bias_bot;
+      }
+  }
+}
+
 // Persistent CTAs: each walks the 128 x BN tiles of C (and k splits)
-// blockIdx.x, blockIdx.x + gridDim.x, ...  Three roles run concurrently:
+// blockIdx.x, blockIdx.x + gridDim.x, ...  Four roles run concurrently:
 //  * warp 8 (lane 0) issues two bulk copies per 16-k stage (the S digit tiles
 //    of A and of B are contiguous) into a ring of nbuf buffers;
 //  * warp 9 (lane 0) issues the stage's MMAs as soon as its data are there;
+//  * warps 10 and 11 write the tiles' tables of C offsets and exponents;
 //  * warps 0-7 (warp w: TMEM lanes 32 (w % 4) .., column half w / 4) take the
 //    level sums of every exact window (oz_window) out of TMEM into two 64-bit
 //    integers per element, then write the tile while the next tile's MMAs run.
@@ -346,8 +414,8 @@ __device__ __forceinline__ int oz_window(const OzArgs& a) {
 // of it were the copies alone (14 copies of 2-4 KB a stage), 21 ms the MMAs
 // alone (a shared issue thread).  Now 11.0 / 14.4 ms, 2090 / 2140 TFLOP/s
 // executed (above the measured bf16 burst rate of a library GEMM); 4096^3 at 8
-// slices 4.2 -> 2.4 ms.  11236 x 256 x 36 (2.3 tiles a CTA, 3 stages each): 50 us,
-// bound by the latency of a tile's set-up, sums and write.
+// slices 4.2 -> 2.4 ms.  Short contractions are bound by the write-back of C: the
+// reductions in L2 (red_add).
 template <int BN, int S>
 __global__ void __launch_bounds__(OZ_CTA_THREADS, 1) k_ozaki_mma(const OzArgs a) {
   constexpr uint32_t TMEM_COLS = 512;
@@ -356,13 +424,16 @@ __global__ void __launch_bounds__(OZ_CTA_THREADS, 1) k_ozaki_mma(const OzArgs a)
   constexpr int HALF = BN / 2;               // columns per warp
   constexpr int CH = 16, NCH = HALF / CH;    // TMEM columns per load
   constexpr int CT = (S + 1) / 2, SH = 7 * (S - CT);  // levels in top; unit of top over that of bot
+  // sets of accumulators: with two, the MMAs of the next window (or tile) run
+  // while this one's sums are read
+  constexpr int NACC = 2 * S * BN <= (int)TMEM_COLS ? 2 : 1;
   static_assert(S * BN <= (int)TMEM_COLS && HALF % CH == 0, "tile");
   extern __shared__ unsigned char oz_smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)oz_smem_raw + 1023) & ~(uintptr_t)1023);
-  __shared__ uint64_t bar_full[OZ_MAXBUF], bar_free[OZ_MAXBUF], bar_acc, bar_read, bar_drain;
+  __shared__ uint64_t bar_full[OZ_MAXBUF], bar_free[OZ_MAXBUF], bar_acc[NACC], bar_read[NACC], bar_drain;
   __shared__ uint32_t tmem_base;
-  __shared__ long long colC[BN], rowC[OZ_BM];
-  __shared__ int colE[BN], rowE[OZ_BM];
+  __shared__ long long colC[2][BN], rowC[2][OZ_BM];  // C offsets and exponents of a tile and the next
+  __shared__ int colE[2][BN], rowE[2][OZ_BM];
   __shared__ volatile int stop;  // a bounded wait ran out
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nbuf = a.nbuf;
@@ -378,8 +449,10 @@ __global__ void __launch_bounds__(OZ_CTA_THREADS, 1) k_ozaki_mma(const OzArgs a)
       mbar_init(&bar_full[i], 1);
       mbar_init(&bar_free[i], 1);
     }
-    mbar_init(&bar_acc, 1);
-    mbar_init(&bar_read, OZ_THREADS / 32);
+    for (int i = 0; i < NACC; ++i) {
+      mbar_init(&bar_acc[i], 1);
+      mbar_init(&bar_read[i], OZ_THREADS / 32);
+    }
     mbar_init(&bar_drain, 1);
     stop = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -396,7 +469,7 @@ __global__ void __launch_bounds__(OZ_CTA_THREADS, 1) k_ozaki_mma(const OzArgs a)
       int b = 0;
       uint32_t lap = 0;  // times the ring has been walked
       bool ok = true;
-      for (long long lin = blockIdx.x; ok && lin < a.tiles; lin += gridDim.x) {
+      for (unsigned lin = blockIdx.x; ok && lin < a.tiles; lin += gridDim.x) {
         int z, mt, nt;
         oz_tile(a, lin, z, mt, nt);
         const int kt0 = z * a.ktper, kt1 = kt0 + a.ktper < a.KT ? kt0 + a.ktper : a.KT;
@@ -449,27 +522,29 @@ __global__ void __launch_bounds__(OZ_CTA_THREADS, 1) k_ozaki_mma(const OzArgs a)
         }
         dA = descA0 + (uint64_t)((uint32_t)(b * STAGE_BYTES) >> 4);
         dB = descB0 + (uint64_t)((uint32_t)(b * STAGE_BYTES) >> 4);
+        const uint32_t acc = NACC == 2 ? tm + (win & 1) * (uint32_t)(S * BN) : tm;
         if (elect_one()) {
-          if (FRESH) oz_issue<BN, S, 1, MID, FRESH>(tm, cA, cB);
-          else oz_issue<BN, S, MID + 1, S, FRESH>(tm, cA, cB);
+          if (FRESH) oz_issue<BN, S, 1, MID, FRESH>(acc, cA, cB);
+          else oz_issue<BN, S, MID + 1, S, FRESH>(acc, cA, cB);
         }
         const bool next = mbar_test(&bar_full[b], ph);
         if (elect_one()) {
-          if (FRESH) oz_issue<BN, S, MID + 1, S, FRESH>(tm, cA, cB);
-          else oz_issue<BN, S, 1, MID, FRESH>(tm, cA, cB);
+          if (FRESH) oz_issue<BN, S, MID + 1, S, FRESH>(acc, cA, cB);
+          else oz_issue<BN, S, 1, MID, FRESH>(acc, cA, cB);
           mma_commit(free);  // the buffer is free once these complete
         }
         there = __all_sync(0xffffffffu, next);
         return true;
       };
       bool ok = true;
-      for (long long lin = blockIdx.x; ok && lin < a.tiles; lin += gridDim.x) {
-        const int z = (int)(lin / ((long long)a.MT * a.NT));
+      for (unsigned lin = blockIdx.x; ok && lin < a.tiles; lin += gridDim.x) {
+        const int z = (int)fast_div(lin, a.f_z);
         const int kt0 = z * a.ktper;
         int left = (kt0 + a.ktper < a.KT ? kt0 + a.ktper : a.KT) - kt0;
         while (ok && left > 0) {
-          // the last window's level sums have been read
-          if (win > 0 && !__all_sync(0xffffffffu, oz_wait(&bar_read, (win - 1) & 1, a.wait_cycles, &stop))) {
+          // the level sums of these accumulators' last window have been read
+          const uint32_t set = win % NACC, use = win / NACC;
+          if (use > 0 && !__all_sync(0xffffffffu, oz_wait(&bar_read[set], (use - 1) & 1, a.wait_cycles, &stop))) {
             ok = false;
             break;
           }
@@ -478,7 +553,7 @@ __global__ void __launch_bounds__(OZ_CTA_THREADS, 1) k_ozaki_mma(const OzArgs a)
           left -= n;
           ok = stage(std::true_type{});
           for (int i = 1; ok && i < n; ++i) ok = stage(std::false_type{});
-          if (ok && elect_one()) mma_commit(&bar_acc);  // completes once every MMA issued so far has
+          if (ok && elect_one()) mma_commit(&bar_acc[set]);  // completes once every MMA issued so far has
           ++win;
         }
       }
@@ -486,6 +561,30 @@ __global__ void __launch_bounds__(OZ_CTA_THREADS, 1) k_ozaki_mma(const OzArgs a)
       __syncwarp();
       if (elect_one()) mma_commit(&bar_drain);
       mbar_wait(&bar_drain, 0, OZ_WAIT_CYCLES);
+    }
+    if (warp >= OZ_THREADS / 32 + 2) {
+      // ---- tables: C offsets and exponents of a tile's rows and columns, one
+      // tile ahead of the summing warps (which spent 1200 clocks a tile on them)
+      const int t0 = tid - (OZ_THREADS + 64);
+      int tb = 0;
+      for (unsigned lin = blockIdx.x; lin < a.tiles; lin += gridDim.x, tb ^= 1) {
+        int z, mt, nt;
+        oz_tile(a, lin, z, mt, nt);
+        for (int i = t0; i < BN + OZ_BM; i += 64) {
+          if (i < BN) {
+            const long long n = (long long)nt * BN + i;
+            colE[tb][i] = a.fb[n] - (int)OZ_EBIAS;
+            colC[tb][i] = a.splits > 1 ? n : n < a.N ? c_offset32((unsigned)n, a.nN, a.fN, a.cN) : -1;
+          } else {
+            const long long m = (long long)mt * OZ_BM + i - BN;
+            rowE[tb][i - BN] = a.ea[m] - (int)OZ_EBIAS;
+            rowC[tb][i - BN] = a.splits > 1 ? ((long long)z * a.MT * OZ_BM + m) * ((long long)a.NT * BN)
+                               : m < a.M   ? c_offset32((unsigned)m, a.nM, a.fM, a.cM)
+                                           : -1;
+          }
+        }
+        table_sync();
+      }
     }
     __syncwarp();
   } else {
@@ -496,83 +595,84 @@ __global__ void __launch_bounds__(OZ_CTA_THREADS, 1) k_ozaki_mma(const OzArgs a)
     const uint32_t taddr = tm + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * HALF);
     double* stg = reinterpret_cast<double*>(smem + (size_t)nbuf * STAGE_BYTES) + warp * 32 * OZ_STAGE_LD;
     uint32_t win = 0;
-    const int window = oz_window(a);
-    for (long long lin = blockIdx.x; lin < a.tiles; lin += gridDim.x) {
+    const int window = oz_window(a), quick = oz_quick(a);
+    int tb = 0;  // tables of this tile
+    bool ok = true;
+    for (unsigned lin = blockIdx.x; lin < a.tiles; lin += gridDim.x, tb ^= 1) {
       int z, mt, nt;
       oz_tile(a, lin, z, mt, nt);
       const int kt0 = z * a.ktper;
-      const int ns = (kt0 + a.ktper < a.KT ? kt0 + a.ktper : a.KT) - kt0;
-      const int nwin = (ns + window - 1) / window;
-      tile_sync();  // the last tile's tables are no longer read
-      if (tid < BN) {
-        const long long n = (long long)nt * BN + tid;
-        if (a.splits > 1) colC[tid] = n;
-        else colC[tid] = n < a.N ? c_offset32((unsigned)n, a.nN, a.fN, a.cN) : -1;
-        colE[tid] = a.fb[n] - (int)OZ_EBIAS;
-      } else if (tid >= OZ_THREADS - OZ_BM) {
-        const int t = tid - (OZ_THREADS - OZ_BM);
-        const long long m = (long long)mt * OZ_BM + t;
-        if (a.splits > 1) rowC[t] = ((long long)z * a.MT * OZ_BM + m) * ((long long)a.NT * BN);
-        else rowC[t] = m < a.M ? c_offset32((unsigned)m, a.nM, a.fM, a.cM) : -1;
-        rowE[t] = a.ea[m] - (int)OZ_EBIAS;
-      }
+      int left = (kt0 + a.ktper < a.KT ? kt0 + a.ktper : a.KT) - kt0;
+      // a warp whose rows or columns all lie outside C sums and writes nothing
+      const bool used = (long long)nt * BN + half * HALF < a.N && (long long)mt * OZ_BM + quad * 32 < a.M;
+      table_sync();  // this tile's tables are written, the last one's may be overwritten
+      if (!ok) continue;
+      double* const out = a.splits > 1 ? a.part : a.C;
+      // element u of a lane in a group of OZ_EPC columns: along the columns of
+      // rows 4 u + lane / 8, or along the rows of column u
+      auto place = [&](int c0, int u) -> long long {
+        const long long fix = a.rowfast ? rowC[tb][quad * 32 + lane] : colC[tb][c0 + lane % OZ_EPC];
+        const long long var = a.rowfast ? colC[tb][c0 + u] : rowC[tb][quad * 32 + u * (32 / OZ_EPC) + lane / OZ_EPC];
+        return fix >= 0 && var >= 0 ? fix + var : -1;
+      };
+      const double* const sp =
+          stg + (a.rowfast ? lane * OZ_STAGE_LD : lane / OZ_EPC * OZ_STAGE_LD + lane % OZ_EPC);
+      const int sstep = a.rowfast ? 1 : 32 / OZ_EPC * OZ_STAGE_LD;
+      constexpr int NG = HALF / OZ_EPC;
       long long top[NCH][CH], bot[NCH][CH];
 #pragma unroll
       for (int j = 0; j < NCH; ++j)
 #pragma unroll
         for (int q = 0; q < CH; ++q) top[j][q] = bot[j][q] = 0;
-      bool ok = true;
-      for (int w = 0; w < nwin; ++w, ++win) {
-        // one thread polls, the others sleep at the barrier: polling by all
-        // eight warps slowed the MMA warp's issue
-        if (tid == 0) ok = oz_wait(&bar_acc, win & 1, a.wait_cycles, &stop);
+      for (; left > 0; left -= window, ++win) {
+        // one thread polls, the others sleep at the barrier
+        const uint32_t set = win % NACC;
+        if (tid == 0) ok = oz_wait(&bar_acc[set], (win / NACC) & 1, a.wait_cycles, &stop);
         ok = tile_sync_and(ok);
         if (!ok) break;
         tc_fence_after();
-#pragma unroll
-        for (int c = 0; c < S; ++c) {
-#pragma unroll
-          for (int j = 0; j < NCH; ++j) {
-            uint32_t acc[CH];
-            tmem_ld16(taddr + (uint32_t)(c * BN + j * CH), acc);
-            tmem_wait_ld();
-#pragma unroll
-            for (int q = 0; q < CH; ++q) {
-              const int v = __float2int_rn(__uint_as_float(acc[q]));
-              if (c < CT) top[j][q] += (long long)v * (1 << (7 * (CT - 1 - c)));
-              else bot[j][q] += (long long)v * (1 << (7 * (S - 1 - c)));
-            }
-          }
+        const int n = left < window ? left : window;
+        if (used) {
+          const uint32_t t = taddr + set * (uint32_t)(S * BN);
+          if (n <= quick) oz_sum<BN, S, NCH, CH, true>(t, top, bot);
+          else oz_sum<BN, S, NCH, CH, false>(t, top, bot);
         }
         // the accumulators are read; the next window may overwrite them
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&bar_read);
+        if (lane == 0) mbar_arrive(&bar_read[set]);
       }
-      if (!tile_sync_and(ok)) break;  // and the tables are written
-      // 2^(ea[m] + fb[n] + 2 - 7 (S + 1)) (top 2^SH + bot), OZ_EPC columns at
+      if (!ok) continue;
+      // alpha 2^(ea[m] + fb[n] + 2 - 7 (S + 1)) (top 2^SH + bot), OZ_EPC columns at
       // a time through this warp's staging rows, so that consecutive lanes
       // touch consecutive elements of C (or of the split-k partial)
-      const int em = rowE[row] + 2 - 7 * (S + 1);
+      if (used) {
+        const int em = rowE[tb][row] + 2 - 7 * (S + 1) + a.alpha_exp;
 #pragma unroll
-      for (int j = 0; j < NCH; ++j) {
-#pragma unroll
-        for (int g = 0; g < CH / OZ_EPC; ++g) {
-          const int c0 = half * HALF + j * CH + g * OZ_EPC;
+        for (int g = 0; g < NG; ++g) {
+          const int c0 = half * HALF + g * OZ_EPC;
+          bool odd = false;
 #pragma unroll
           for (int q = 0; q < OZ_EPC; ++q)
             stg[lane * OZ_STAGE_LD + q] =
-                oz_value<SH>(top[j][g * OZ_EPC + q], bot[j][g * OZ_EPC + q], em + colE[c0 + q]);
+                oz_value<SH>(top[g * OZ_EPC / CH][g * OZ_EPC % CH + q], bot[g * OZ_EPC / CH][g * OZ_EPC % CH + q],
+                             em + colE[tb][c0 + q], a.alpha_neg, odd);
+          if (__any_sync(0xffffffffu, odd)) {
+#pragma unroll
+            for (int q = 0; q < OZ_EPC; ++q)
+              stg[lane * OZ_STAGE_LD + q] = oz_value_odd<SH>(top[g * OZ_EPC / CH][g * OZ_EPC % CH + q],
+                                                             bot[g * OZ_EPC / CH][g * OZ_EPC % CH + q],
+                                                             em + colE[tb][c0 + q], a.alpha_neg);
+          }
           __syncwarp();
-          double* const out = a.splits > 1 ? a.part : a.C;
 #pragma unroll
           for (int u = 0; u < OZ_EPC; ++u) {
-            const int i = u * 32 + lane;
-            const int r = a.rowfast ? lane : i / OZ_EPC, c = a.rowfast ? u : i % OZ_EPC;
-            const long long oc = colC[c0 + c], orow = rowC[quad * 32 + r];
-            const double t = stg[r * OZ_STAGE_LD + c];
-            if (a.splits > 1) out[orow + oc] = t;
-            else if (oc >= 0 && orow >= 0) red_add(out + orow + oc, a.alpha * t);
+            const long long o = place(c0, u);
+            const double t = sp[u * sstep];
+            if (o >= 0) {
+              if (a.splits > 1) out[o] = t;
+              else red_add(out + o, a.alpha_mul ? a.alpha * t : t);
+            }
           }
           __syncwarp();
         }
@@ -632,22 +732,23 @@ struct OzPack {
   int T, KT;           // tiles along rows (TR each) and k (64 each)
   int TR;              // rows per tile: 128 (A) or BN (B)
   int S;
-  int vec;             // 1: every full 8-group is 64 contiguous, 16-byte aligned bytes
+  int vec;             // 1: every full 8-group is 64 contiguous, 16-byte aligned bytes; 2: 32-byte aligned
   FastDiv fR[4], fK[4];  // divisors of eR, eK
 };
 
-// whether pack_load8 may read a full k group with 16-byte loads: unit
-// innermost k stride, groups that never cross a carry of the k multi-index
-// (innermost extent a multiple of 8), every other stride even and the base
-// 16-byte aligned, so every group starts on a 16-byte boundary
+// whether pack_load8 may read a full k group with 32-byte (2) or 16-byte (1)
+// loads: unit innermost k stride, groups that never cross a carry of the k
+// multi-index (innermost extent a multiple of 8), every other stride a
+// multiple of 4 (2) and the base aligned, so every group starts on a boundary
 inline int pack_vec_ok(const OzPack& p) {
   if (p.nK < 1 || p.sK[p.nK - 1] != 1 || p.eK[p.nK - 1] % 8 != 0) return 0;
-  if (reinterpret_cast<uintptr_t>(p.src) % 16 != 0) return 0;
-  for (int d = 0; d < p.nK - 1; ++d)
-    if (p.sK[d] % 2 != 0) return 0;
-  for (int d = 0; d < p.nR; ++d)
-    if (p.sR[d] % 2 != 0) return 0;
-  return 1;
+  for (int v = 2; v > 0; --v) {
+    bool ok = reinterpret_cast<uintptr_t>(p.src) % (16 * v) == 0;
+    for (int d = 0; d < p.nK - 1; ++d) ok = ok && p.sK[d] % (2 * v) == 0;
+    for (int d = 0; d < p.nR; ++d) ok = ok && p.sR[d] % (2 * v) == 0;
+    if (ok) return v;
+  }
+  return 0;
 }
 
 // Operand preparation runs in two passes over the padded operand viewed as
@@ -710,6 +811,17 @@ __device__ __forceinline__ void pack_load8(const OzPack& p, unsigned r, unsigned
       lin = qd;
     }
   }
+  if (p.vec == 2 && k0 + 8 <= (unsigned long long)p.K) {
+    // one full sector per lane and load: with 16-byte loads at a 64-byte
+    // stride the row-maximum pass read 3.7 TB/s
+    const long long* v = src + roff + off;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      asm volatile("ld.global.v4.b64 {%0, %1, %2, %3}, [%4];"
+                   : "=l"(x[4 * h]), "=l"(x[4 * h + 1]), "=l"(x[4 * h + 2]), "=l"(x[4 * h + 3])
+                   : "l"(v + 4 * h));
+    return;
+  }
   if (p.vec && k0 + 8 <= (unsigned long long)p.K) {
     const longlong2* v = reinterpret_cast<const longlong2*>(src + roff + off);
 #pragma unroll
@@ -747,7 +859,8 @@ struct PackPass {
   int kfast[2];
   FastDiv fQ[2], fR[2];
   unsigned W[2];
-  unsigned* sq;  // [2] (pass 2)
+  unsigned* sq;  // [2] (pass 2 and the one-pass form)
+  int lpr[2];    // one-pass form: lanes per row, 0: one thread per row
 };
 
 // Each CTA walks one contiguous range of work items, 256 at a time, and each
@@ -805,13 +918,10 @@ __global__ void __launch_bounds__(PACK_T) k_ozaki_rowexp(const PackPass pp) {
 // stored as bf16 (exact: |d| <= 64).  One call: group q of row r, S 16-byte
 // stores (one per slice tile); returns the sum of the squared digits.
 template <int S>
-__device__ __forceinline__ int digits_item(const OzPack& p, const unsigned* eu, __nv_bfloat16* dst, unsigned r,
-                                            unsigned q) {
+__device__ __forceinline__ int digits_item(const OzPack& p, const long long (&x)[8], int e, __nv_bfloat16* dst,
+                                            unsigned r, unsigned q) {
   const long long tile_elems = (long long)p.TR * OZ_BK;
   constexpr int F = 7 * S - 1;
-  long long x[8];
-  pack_load8(p, r, q, x);
-  const int e = r < (unsigned long long)p.R ? (int)eu[r] - (int)OZ_EBIAS : 0;
   int dg[S][8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
@@ -906,7 +1016,9 @@ __global__ void __launch_bounds__(PACK_T) k_ozaki_digits(const PackPass pp) {
         r = j - tk * fR.d;
         q = 2u * tk + (i & 1u);
       }
-      sq = digits_item<S>(p, eu, dst, r, q);
+      long long x[8];
+      pack_load8(p, r, q, x);
+      sq = digits_item<S>(p, x, r < (unsigned long long)p.R ? (int)eu[r] - (int)OZ_EBIAS : 0, dst, r, q);
     }
     // items 2 j and 2 j + 1 are the halves of one row's 16 k
     sq += __shfl_xor_sync(0xffffffffu, sq, 1);
@@ -919,6 +1031,57 @@ __global__ void __launch_bounds__(PACK_T) k_ozaki_digits(const PackPass pp) {
   if (threadIdx.x == 0) {
     for (int w = 1; w < PACK_T / 32; ++w) most = part[w] > most ? part[w] : most;
     if (most > 0) atomicMax(pp.sq + o, (unsigned)most);
+  }
+}
+
+// Both passes in one for k up to PACK_SHORT: the exponent of a row is known
+// before its digits are cut.  Lanes along k (a row's groups in `lpr` adjacent
+// lanes, each group loaded once), or where the rows are the contiguous
+// direction and many, one thread per row, which reads it twice.  The window
+// rule gets the bound that holds for any digits (one window, and the quick
+// sums for k up to 128 at 8 slices).  Every padded row is written, so nothing
+// is cleared beforehand: one launch in place of three.
+constexpr int PACK_SHORT = 256, PACK_ROWS = 4096;
+template <int S>
+__global__ void __launch_bounds__(PACK_T) k_ozaki_pack_short(const PackPass pp) {
+  const int o = blockIdx.y;
+  const OzPack& p = pp.p[o];
+  unsigned* eu = pp.eu[o];
+  __nv_bfloat16* dst = pp.dst[o];
+  const unsigned rows = (unsigned)p.T * (unsigned)p.TR, groups = (unsigned)p.KT * (OZ_BK / 8);
+  if (blockIdx.x == 0 && threadIdx.x == 0) pp.sq[o] = (unsigned)(OZ_BK * S * 64 * 64);
+  const unsigned long long t0 = blockIdx.x * (unsigned long long)PACK_T + threadIdx.x;
+  const unsigned long long stride = (unsigned long long)gridDim.x * PACK_T;
+  if (pp.lpr[o]) {
+    const unsigned lpr = (unsigned)pp.lpr[o], sh = 31 - __clz(lpr), q = (unsigned)t0 & (lpr - 1);
+    // rows is a multiple of 32, so whole warps leave the loop together
+    for (unsigned long long t = t0; t < (unsigned long long)rows << sh; t += stride) {
+      const unsigned r = (unsigned)(t >> sh);
+      long long x[8];
+      pack_load8(p, r, q, x);  // zero beyond the operand
+      unsigned c = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) c = max(c, exp_code(x[j]));
+      for (unsigned d = lpr >> 1; d > 0; d >>= 1) c = max(c, __shfl_xor_sync(0xffffffffu, c, d));
+      if (q < groups) digits_item<S>(p, x, (int)c - (int)OZ_EBIAS, dst, r, q);
+      if (q == 0) eu[r] = c;
+    }
+  } else {
+    for (unsigned long long r = t0; r < rows; r += stride) {
+      unsigned c = 0;
+      for (unsigned q = 0; q < groups; ++q) {
+        long long x[8];
+        pack_load8(p, (unsigned)r, q, x);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) c = max(c, exp_code(x[j]));
+      }
+      for (unsigned q = 0; q < groups; ++q) {
+        long long x[8];
+        pack_load8(p, (unsigned)r, q, x);
+        digits_item<S>(p, x, (int)c - (int)OZ_EBIAS, dst, (unsigned)r, q);
+      }
+      eu[r] = c;
+    }
   }
 }
 
@@ -946,7 +1109,7 @@ inline int oz_grid(long long n) {
 // stage buffers that fit beside the staging rows and the static tables
 int oz_buffers(int S, int BN) {
   const int stage = S * (OZ_TILE_BYTES + BN * OZ_BK * 2);
-  const int n = (227 * 1024 - 4096 - 1024 - OZ_STAGE_BYTES) / stage;
+  const int n = (227 * 1024 - OZ_STATIC_BYTES - 1024 - OZ_STAGE_BYTES) / stage;
   return n < OZ_MAXBUF ? n : OZ_MAXBUF;
 }
 
@@ -964,7 +1127,7 @@ void oz_smem_attribute() {
   check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
   std::lock_guard<std::mutex> lock(mu);
   if (dev < 0 || dev >= 64 || done[dev]) return;
-  check_cuda(cudaFuncSetAttribute(k_ozaki_mma<BN, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 4096),
+  check_cuda(cudaFuncSetAttribute(k_ozaki_mma<BN, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - OZ_STATIC_BYTES),
              "cudaFuncSetAttribute (ozaki)");
   // the kernel's register split draws on exactly this launch total
   cudaFuncAttributes fa{};
@@ -985,7 +1148,13 @@ void oz_launch_bn_s(const OzArgs& a, cudaStream_t st) {
 
 template <int BN>
 void oz_launch_bn(OzArgs a, int MT, int NT, cudaStream_t st) {
-  a.tiles = (long long)MT * NT * a.splits;
+  const long long tiles = (long long)MT * NT * a.splits;
+  if (tiles >= (1LL << 31)) throw std::runtime_error("split-precision contraction: too many tiles");
+  a.tiles = (unsigned)tiles;
+  a.f_z = make_fastdiv((unsigned)(MT * NT));
+  a.f_group = make_fastdiv((unsigned)(OZ_GROUP * NT));
+  a.f_full = make_fastdiv((unsigned)(MT < OZ_GROUP ? MT : OZ_GROUP));
+  a.f_tail = make_fastdiv((unsigned)(MT % OZ_GROUP ? MT % OZ_GROUP : OZ_GROUP));
   a.nbuf = oz_buffers(a.S, BN);
   switch (a.S) {
     case 1: oz_launch_bn_s<BN, 1>(a, st); break;
@@ -1093,7 +1262,10 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
   }
   pa.vec = pack_vec_ok(pa);
   pb.vec = pack_vec_ok(pb);
-  int BN = ch.bn ? ch.bn : N <= 32 ? 32 : 64;
+  // 64 columns per tile, or 32 where the output is narrow or gives fewer tiles
+  // than SMs (257 x 131 x 700: 18 -> 10 us)
+  const long long wide = (M + OZ_BM - 1) / OZ_BM * ((N + 63) / 64);
+  int BN = ch.bn ? ch.bn : N <= 32 || wide < 152 ? 32 : 64;
   const int MT = (int)((M + OZ_BM - 1) / OZ_BM), NT = (int)((N + BN - 1) / BN);
   const int KT = (int)((g0.K + OZ_BK - 1) / OZ_BK);
   pa.R = M;
@@ -1127,14 +1299,15 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
   if (splits > 1) part = ws.get((size_t)splits * MT * OZ_BM * NT * BN, capP);
   int* ea = (int*)bufE;
   int* fb = ea + (size_t)MT * OZ_BM;
-  // algorithmic bytes: each operand element read twice (8 B each), S bf16 digits written
-  int r = ws.begin(K_OZAKI_PACK, 0.0, (16.0 + 2.0 * S) * (double)(M + N) * (double)g0.K);
+  // algorithmic bytes: each operand element read twice (8 B each; once in the
+  // one-pass form), S bf16 digits written
+  int r = ws.begin(K_OZAKI_PACK, 0.0,
+                   ((g0.K <= PACK_SHORT ? 8.0 : 16.0) + 2.0 * S) * (double)(M + N) * (double)g0.K);
   if (r >= 0) {
     ws.recs[r].m = M;
     ws.recs[r].n = N;
     ws.recs[r].k = g0.K;
   }
-  check_cuda(cudaMemsetAsync(ea, 0, (nE + 2) * sizeof(int), st), "cudaMemsetAsync (exponents)");
   PackPass pp{};
   long long w1max = 1, w2max = 1;
   PackPass pd{};
@@ -1155,20 +1328,44 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
     w1max = std::max(w1max, rows * q1);
     w2max = std::max(w2max, rows * q2);
   }
-  k_ozaki_rowexp<<<dim3((unsigned)oz_pack_grid(w1max), 2), PACK_T, 0, st>>>(pp);
-  const dim3 g2((unsigned)oz_pack_grid(w2max), 2);
-  switch (S) {
-    case 1: k_ozaki_digits<1><<<g2, PACK_T, 0, st>>>(pd); break;
-    case 2: k_ozaki_digits<2><<<g2, PACK_T, 0, st>>>(pd); break;
-    case 3: k_ozaki_digits<3><<<g2, PACK_T, 0, st>>>(pd); break;
-    case 4: k_ozaki_digits<4><<<g2, PACK_T, 0, st>>>(pd); break;
-    case 5: k_ozaki_digits<5><<<g2, PACK_T, 0, st>>>(pd); break;
-    case 6: k_ozaki_digits<6><<<g2, PACK_T, 0, st>>>(pd); break;
-    case 7: k_ozaki_digits<7><<<g2, PACK_T, 0, st>>>(pd); break;
-    default: k_ozaki_digits<8><<<g2, PACK_T, 0, st>>>(pd); break;
+  if (g0.K <= PACK_SHORT) {
+    unsigned lpr = 1;
+    while (lpr < (unsigned)KT * (OZ_BK / 8)) lpr *= 2;
+    long long wmax = 1;
+    for (int o = 0; o < 2; ++o) {
+      const OzPack& p = o ? pb : pa;
+      const long long rows = (long long)p.T * p.TR;
+      pd.lpr[o] = pd.kfast[o] || rows < PACK_ROWS ? (int)lpr : 0;
+      wmax = std::max(wmax, pd.lpr[o] ? rows * lpr : rows);
+    }
+    const dim3 gs((unsigned)oz_pack_grid(wmax), 2);
+    switch (S) {
+      case 1: k_ozaki_pack_short<1><<<gs, PACK_T, 0, st>>>(pd); break;
+      case 2: k_ozaki_pack_short<2><<<gs, PACK_T, 0, st>>>(pd); break;
+      case 3: k_ozaki_pack_short<3><<<gs, PACK_T, 0, st>>>(pd); break;
+      case 4: k_ozaki_pack_short<4><<<gs, PACK_T, 0, st>>>(pd); break;
+      case 5: k_ozaki_pack_short<5><<<gs, PACK_T, 0, st>>>(pd); break;
+      case 6: k_ozaki_pack_short<6><<<gs, PACK_T, 0, st>>>(pd); break;
+      case 7: k_ozaki_pack_short<7><<<gs, PACK_T, 0, st>>>(pd); break;
+      default: k_ozaki_pack_short<8><<<gs, PACK_T, 0, st>>>(pd); break;
+    }
+  } else {
+    check_cuda(cudaMemsetAsync(ea, 0, (nE + 2) * sizeof(int), st), "cudaMemsetAsync (exponents)");
+    k_ozaki_rowexp<<<dim3((unsigned)oz_pack_grid(w1max), 2), PACK_T, 0, st>>>(pp);
+    const dim3 g2((unsigned)oz_pack_grid(w2max), 2);
+    switch (S) {
+      case 1: k_ozaki_digits<1><<<g2, PACK_T, 0, st>>>(pd); break;
+      case 2: k_ozaki_digits<2><<<g2, PACK_T, 0, st>>>(pd); break;
+      case 3: k_ozaki_digits<3><<<g2, PACK_T, 0, st>>>(pd); break;
+      case 4: k_ozaki_digits<4><<<g2, PACK_T, 0, st>>>(pd); break;
+      case 5: k_ozaki_digits<5><<<g2, PACK_T, 0, st>>>(pd); break;
+      case 6: k_ozaki_digits<6><<<g2, PACK_T, 0, st>>>(pd); break;
+      case 7: k_ozaki_digits<7><<<g2, PACK_T, 0, st>>>(pd); break;
+      default: k_ozaki_digits<8><<<g2, PACK_T, 0, st>>>(pd); break;
+    }
+    ws.launches += 1;  // two pack kernels (begin() counts one; the memset is not a kernel)
   }
   ws.end(r);
-  ws.launches += 1;  // two pack kernels (begin() counted one; the memset is not a kernel)
   a.As = (const __nv_bfloat16*)bufA;
   a.Bs = (const __nv_bfloat16*)bufB;
   a.ea = ea;
@@ -1181,6 +1378,14 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
   a.M = M;
   a.N = N;
   a.alpha = g0.alpha;
+  {
+    int e = 0;
+    const double f = std::frexp(g0.alpha, &e);  // +-0.5 for a power of two
+    const bool pow2 = std::fabs(f) == 0.5 && e > -500 && e < 500;
+    a.alpha_mul = !pow2 && splits <= 1;
+    a.alpha_exp = pow2 && splits <= 1 ? e - 1 : 0;
+    a.alpha_neg = pow2 && splits <= 1 && f < 0.0;
+  }
   for (int d = 0; d < 4; ++d) {
     a.fM[d] = make_fastdiv(d < a.nM ? (unsigned)a.eM[d] : 1u);
     a.fN[d] = make_fastdiv(d < a.nN ? (unsigned)a.eN[d] : 1u);
