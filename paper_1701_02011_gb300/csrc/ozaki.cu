@@ -863,10 +863,12 @@ struct PackPass {
   int lpr[2];    // one-pass form: lanes per row, 0: one thread per row
 };
 
-// Each CTA walks one contiguous range of work items, 256 at a time, and each
-// thread keeps the maximum of its current row in a register, flushed by an
-// atomic max when its row changes and at the end: a few long rows (a short
-// side of 8 or 38) would otherwise send millions of atomics to a few words.
+// Each warp walks one contiguous range of steps of 32 work items, and each lane
+// keeps the maximum of its current row in a register.  When lanes move to
+// another row, those that leave the same row combine their maxima and one of
+// them issues the atomic max: with k along the lanes a warp crosses a row's end
+// every few steps, and an atomic per lane (6 million for 61504 x 784) held the
+// pass at 3.8 TB/s.
 __global__ void __launch_bounds__(PACK_T) k_ozaki_rowexp(const PackPass pp) {
   const int o = blockIdx.y;
   const OzPack& p = pp.p[o];
@@ -874,41 +876,59 @@ __global__ void __launch_bounds__(PACK_T) k_ozaki_rowexp(const PackPass pp) {
   const int kfast = pp.kfast[o];
   const FastDiv fQ = pp.fQ[o], fR = pp.fR[o];
   const unsigned W = pp.W[o];
-  const unsigned long long span = (unsigned long long)gridDim.x * PACK_T;
-  const unsigned long long per = (W + span - 1) / span * PACK_T;  // items per CTA
-  const unsigned long long lo = blockIdx.x * per;
-  const unsigned long long hi = lo + per < W ? lo + per : W;
-  long long held = -1;  // row whose maximum is in hv
-  unsigned hv = 0;
-  for (unsigned long long base = lo; base < hi; base += PACK_T) {
-    if (base + threadIdx.x >= hi) break;
-    const unsigned i = (unsigned)(base + threadIdx.x);
-    unsigned rr, q;
-    pack_item(i, fQ, fR, kfast != 0, rr, q);
-    if (rr >= (unsigned long long)p.R) continue;
-    long long x[8];
-    pack_load8(p, rr, q, x);
-    unsigned v = 0;
+  const unsigned lane = threadIdx.x & 31;
+  const unsigned long long warps = (unsigned long long)gridDim.x * (PACK_T / 32);
+  const unsigned long long steps = (W + 31ULL) / 32;  // of 32 items; W is a multiple of 32 when rows are along the lanes
+  const unsigned long long per = (steps + warps - 1) / warps;
+  const unsigned long long lo = (blockIdx.x * (unsigned long long)(PACK_T / 32) + (threadIdx.x >> 5)) * per;
+  const unsigned long long hi = lo + per < steps ? lo + per : steps;
+  unsigned held = ~0u, hv = 0;  // row (none: ~0) and the maximum so far
+  // lanes with `go` send (held, hv); a warp-wide step
+  auto flush = [&](bool go) {
+    go = go && hv;
+    const unsigned mask = __ballot_sync(0xffffffffu, go);
+    if (!mask) return;
+    const int lead = __ffs(mask) - 1;
+    const unsigned r0 = __shfl_sync(0xffffffffu, held, lead);
+    if (__all_sync(0xffffffffu, !go || held == r0)) {
+      const unsigned m = __reduce_max_sync(0xffffffffu, go ? hv : 0u);
+      if ((int)lane == lead) atomicMax(eu + r0, m);
+    } else if (go) {
+      atomicMax(eu + held, hv);
+    }
+  };
+  for (unsigned long long t = lo; t < hi; ++t) {
+    unsigned rr = ~0u, v = 0;
+    const unsigned long long i = t * 32 + lane;
+    if (i < W) {
+      // along k: item i is (row, group); along the rows: step t is the 32 rows
+      // of a block at one group, the groups of a block in a row
+      unsigned q;
+      if (kfast) {
+        pack_item((unsigned)i, fQ, fR, true, rr, q);
+      } else {
+        const unsigned rb = fast_div((unsigned)t, fQ);
+        q = (unsigned)t - rb * fQ.d;
+        rr = rb * 32 + lane;
+      }
+      if (rr < (unsigned long long)p.R) {
+        long long x[8];
+        pack_load8(p, rr, q, x);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const unsigned c = exp_code(x[j]);
-      v = c > v ? c : v;
+        for (int j = 0; j < 8; ++j) v = max(v, exp_code(x[j]));
+      }
     }
-    if ((long long)rr != held) {
-      if (held >= 0 && hv) atomicMax(eu + held, hv);
-      held = rr;
-      hv = 0;
+    const bool moved = rr != held;
+    if (__any_sync(0xffffffffu, moved)) {
+      flush(moved);
+      if (moved) {
+        held = rr;
+        hv = 0;
+      }
     }
-    hv = v > hv ? v : hv;
+    hv = max(hv, v);
   }
-  // final flush: one atomic per warp when every lane holds the same row
-  const long long r0 = __shfl_sync(0xffffffffu, held, 0);
-  if (__all_sync(0xffffffffu, held == r0)) {
-    const unsigned m = __reduce_max_sync(0xffffffffu, hv);
-    if ((threadIdx.x & 31) == 0 && r0 >= 0 && m) atomicMax(eu + r0, m);
-  } else if (held >= 0 && hv) {
-    atomicMax(eu + held, hv);
-  }
+  flush(true);
 }
 
 // S balanced base-128 digits of each element: V = round(x 2^(7S - 1 - e)),
