@@ -948,6 +948,7 @@ void issue_energy(Handle& h, bool pt3) {
   Workspace& ws = h.ws;
   ws.launches = 0;
   ws.nresults = 0;
+  ws.retire_arena();
   h.res_pt3 = pt3;
   const Iv& H = h.H;
   const Iv& P = h.P;

@@ -490,6 +490,8 @@ void run_axpy(Workspace& ws, const NdArgs& g, double alpha, const double* A, dou
 }
 
 Workspace::~Workspace() {
+  for (auto& a : arenas_)
+    if (a.p) release(a.p);
   for (auto& r : recs) {
     cudaEventDestroy(r.a);
     cudaEventDestroy(r.b);
@@ -545,6 +547,50 @@ double* Workspace::get(size_t n, size_t& cap) {
   return p;
 }
 
+double* Workspace::get_zeroed(size_t n, int& arena) {
+  n = (n + 3) / 4 * 4;  // 32-byte boundaries
+  if (open_ < 0 || arenas_[open_].used + n > kArenaSize) {
+    retire_arena();
+    for (int i = 0; i < (int)arenas_.size() && open_ < 0; ++i)
+      if (!arenas_[i].p) open_ = i;
+    if (open_ < 0) {
+      arenas_.push_back(Arena{});
+      open_ = (int)arenas_.size() - 1;
+    }
+    Arena& a = arenas_[open_];
+    const int mine = open_;
+    open_ = -1;
+    a.p = get(kArenaSize, a.cap);
+    a.used = 0;
+    a.live = 0;
+    open_ = mine;
+    check_cuda(cudaMemsetAsync(a.p, 0, kArenaSize * sizeof(double), stream), "memset (arena)");
+  }
+  Arena& a = arenas_[open_];
+  double* p = a.p + a.used;
+  a.used += n;
+  ++a.live;
+  arena = open_;
+  return p;
+}
+
+void Workspace::arena_put(int i) {
+  Arena& a = arenas_[i];
+  if (--a.live == 0 && i != open_) {
+    put(a.p, a.cap);
+    a = Arena{};
+  }
+}
+
+void Workspace::retire_arena() {
+  const int i = open_;
+  open_ = -1;
+  if (i >= 0 && arenas_[i].live == 0) {
+    put(arenas_[i].p, arenas_[i].cap);
+    arenas_[i] = Arena{};
+  }
+}
+
 void Workspace::put(double* p, size_t cap) {
   if (!p) return;
   in_use_ -= cap * sizeof(double);
@@ -558,6 +604,8 @@ Tensor& Tensor::operator=(Tensor&& o) noexcept {
     n = o.n;
     cap = o.cap;
     ws = o.ws;
+    arena = o.arena;
+    o.arena = -1;
     o.v.p = nullptr;
     o.n = 0;
     o.cap = 0;
@@ -569,7 +617,11 @@ Tensor& Tensor::operator=(Tensor&& o) noexcept {
 Tensor::~Tensor() { release(); }
 
 void Tensor::release() {
-  if (ws && v.p) ws->put(v.p, cap);
+  if (ws && v.p) {
+    if (arena >= 0) ws->arena_put(arena);
+    else ws->put(v.p, cap);
+  }
+  arena = -1;
   v.p = nullptr;
   ws = nullptr;
   n = 0;
@@ -618,6 +670,11 @@ Tensor make_tensor(Workspace& ws, int rank, const Iv* ivs, bool zero, bool dense
     t.n = (size_t)stride;
   }
   t.ws = &ws;
+  if (zero && t.n <= Workspace::kArenaMost) {
+    t.v.p = ws.get_zeroed(t.n, t.arena);
+    t.v.mask = 0;
+    return t;
+  }
   t.v.p = ws.get(t.n, t.cap);
   if (zero) check_cuda(cudaMemsetAsync(t.v.p, 0, t.n * sizeof(double), ws.stream), "memset");
   t.v.mask = 0;

@@ -73,6 +73,7 @@ struct Tensor {
   size_t n = 0;    // elements
   size_t cap = 0;  // elements of the underlying block
   Workspace* ws = nullptr;
+  int arena = -1;  // of the workspace's arenas of small zeroed tensors
   Tensor() = default;
   Tensor(const Tensor&) = delete;
   Tensor& operator=(const Tensor&) = delete;
@@ -92,6 +93,15 @@ class Workspace {
   ~Workspace();
   double* get(size_t n, size_t& cap);
   void put(double* p, size_t cap);
+  // n zeroed doubles (n <= kArenaMost) out of an arena that is cleared as a
+  // whole, so that the many small accumulators of an energy cost one memset;
+  // released by arena_put.  retire_arena() ends the use of the open arena:
+  // what follows clears its own (an energy captured as a graph must hold the
+  // memset of everything it relies on).
+  static constexpr size_t kArenaMost = 8192, kArenaSize = 1 << 19;
+  double* get_zeroed(size_t n, int& arena);
+  void arena_put(int arena);
+  void retire_arena();
   size_t bytes_in_use() const { return in_use_; }
   size_t peak_bytes() const { return peak_; }
   cudaStream_t stream;
@@ -136,6 +146,9 @@ class Workspace {
   struct Blk { double* p; size_t n; };
   cudaMemPool_t pool_ = nullptr;
   std::vector<Blk> free_;
+  struct Arena { double* p = nullptr; size_t cap = 0, used = 0; int live = 0; };
+  std::vector<Arena> arenas_;
+  int open_ = -1;  // arena that serves get_zeroed
   size_t in_use_ = 0, peak_ = 0;
   const char* peak_tag_ = "";  // step being issued when the peak was reached
 };
