@@ -23,7 +23,7 @@ constexpr int CH_MAX_CTAS = 152 * 4;
 // sum, and an SM retires two FP64 operations a clock, so a step lasts as long
 // as the SM with the most rows: up to N = 152 x 96 each SM gets one CTA of 96
 // rows (with 256 threads at N = 13456 the factorisation used 53 of the 152
-// SMs, 40 us a vector on average; now 24 us).  Larger N fill the chip with 256.
+// SMs, 40 us a vector on average; now 24 us, 22 us with chained launches).  Larger N fill the chip with 256.
 constexpr long long CH_SMALL_N = 152LL * 96;
 constexpr int CH_Q = 512;  // earlier vectors whose pivot entries are held at a time
 
@@ -129,14 +129,17 @@ __global__ void __launch_bounds__(CH_T) k_chol_init(const double* __restrict__ V
 
 // one vector: B[nvec][i], D[i] -= B[nvec][i]^2, and the next pivot
 template <int CH_T>
-__global__ void __launch_bounds__(CH_T) k_chol_step(const double* __restrict__ V, long long N, double* __restrict__ B,
-                                                   double* __restrict__ D, double* pv, long long* pi, ChState* st,
+__global__ void __launch_bounds__(CH_T) k_chol_step(const double* __restrict__ V, long long N, double* B,
+                                                   double* D, double* pv, long long* pi, ChState* st,
                                                    double tau, int max_vecs, long long* piv) {
-  if (st->done) return;
-  const long long J = st->J;
-  const int Q = st->nvec;
-  const double sq = sqrt(st->dJ);
-  const double* __restrict__ bJ = B + J;  // B[q][J] at bJ[q * N]
+  dsrg::wait_for_previous();
+  if (__ldcg(&st->done)) return;
+  const long long J = __ldcg(&st->J);
+  const int Q = __ldcg(&st->nvec);
+  const double sq = sqrt(__ldcg(&st->dJ));
+  // B and D are what earlier kernels of the chain wrote: read through L2 (the
+  // end of one vector and the start of the next may share a cache line)
+  const double* bJ = B + J;  // B[q][J] at bJ[q * N]
   double bv = -INFINITY;
   long long bi = -1;
   // the pivot's column of the earlier vectors goes through shared memory, CH_Q
@@ -147,7 +150,7 @@ __global__ void __launch_bounds__(CH_T) k_chol_step(const double* __restrict__ V
   for (long long i0 = blockIdx.x * (long long)CH_T; i0 < N; i0 += (long long)gridDim.x * CH_T) {
     const long long i = i0 + threadIdx.x;
     const bool live = i < N;
-    const double* __restrict__ bi_ = B + (live ? i : 0);
+    const double* bi_ = B + (live ? i : 0);
     constexpr int U = 16;
     double acc = 0.0;
     for (int q0 = 0; q0 < Q; q0 += CH_Q) {
@@ -156,16 +159,16 @@ __global__ void __launch_bounds__(CH_T) k_chol_step(const double* __restrict__ V
       const int full = nq / U * U;
       if (full > 0) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) x[u] = __ldg(bi_ + (long long)(q0 + u) * N);
+        for (int u = 0; u < U; ++u) x[u] = __ldcg(bi_ + (long long)(q0 + u) * N);
       }
       __syncthreads();  // the last block's entries are no longer read
-      for (int q = threadIdx.x; q < nq; q += CH_T) yj[q] = __ldg(bJ + (long long)(q0 + q) * N);
+      for (int q = threadIdx.x; q < nq; q += CH_T) yj[q] = __ldcg(bJ + (long long)(q0 + q) * N);
       __syncthreads();
       for (int q = 0; q < full; q += U) {
         double nx[U];
         if (q + U < full) {
 #pragma unroll
-          for (int u = 0; u < U; ++u) nx[u] = __ldg(bi_ + (long long)(q0 + q + U + u) * N);
+          for (int u = 0; u < U; ++u) nx[u] = __ldcg(bi_ + (long long)(q0 + q + U + u) * N);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) x[u] = __dmul_rn(x[u], yj[q + u]);
@@ -174,12 +177,12 @@ __global__ void __launch_bounds__(CH_T) k_chol_step(const double* __restrict__ V
 #pragma unroll
         for (int u = 0; u < U; ++u) x[u] = nx[u];
       }
-      for (int q = full; q < nq; ++q) acc = __dadd_rn(acc, __dmul_rn(__ldg(bi_ + (long long)(q0 + q) * N), yj[q]));
+      for (int q = full; q < nq; ++q) acc = __dadd_rn(acc, __dmul_rn(__ldcg(bi_ + (long long)(q0 + q) * N), yj[q]));
     }
     if (!live) continue;
     const double L = __ddiv_rn(__dsub_rn(V[J * N + i], acc), sq);
     B[(long long)Q * N + i] = L;
-    const double d = __dsub_rn(D[i], __dmul_rn(L, L));
+    const double d = __dsub_rn(__ldcg(D + i), __dmul_rn(L, L));
     D[i] = d;
     if (better(d, i, bv, bi)) {
       bv = d;
@@ -224,8 +227,9 @@ extern "C" int dsrg_cholesky(long long N, const double* V, double tau, int max_v
     check_cuda(cudaGetLastError(), "cholesky launch");
     ChState h{};
     for (int q = 0; q < max_vecs; ++q) {
-      (small ? k_chol_step<96> : k_chol_step<256>)<<<grid, small ? 96 : 256, 0, st>>>(V, N, B, D, pv, pi, cs, tau, max_vecs, piv);
-      check_cuda(cudaGetLastError(), "cholesky launch");
+      check_cuda(launch_chained(small ? k_chol_step<96> : k_chol_step<256>, grid, small ? 96 : 256, st, V, N, B, D, pv, pi,
+                                cs, tau, max_vecs, piv),
+                 "cholesky launch");
       // every 32 vectors: stop launching once the factorisation has stopped
       if ((q & 31) == 31 || q == max_vecs - 1) {
         check_cuda(cudaMemcpyAsync(&h, cs, sizeof h, cudaMemcpyDeviceToHost, st), "cudaMemcpyAsync (cholesky)");

@@ -45,6 +45,33 @@ inline
   return (unsigned)(((unsigned long long)hi + n) >> f.l);
 }
 
+#ifdef __CUDACC__
+// Chains of short dependent kernels.  A kernel that begins with
+// wait_for_previous() may be launched with launch_chained(): its blocks take
+// their places while the kernel before it still runs and wait there (in
+// hardware) until that one has completed and its writes are visible, so that a
+// step costs no launch latency.  The next kernel may do the same from then on.
+// What such a kernel reads of its predecessors' results it must not read through
+// the read-only path (__ldg, const __restrict__).
+__device__ __forceinline__ void wait_for_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t st, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#endif
+
 // C[m, n] += alpha * sum_k A[m, k] B[k, n] over multi-indices m, n, k and a
 // batch multi-index b present in all three operands.  Every group holds up
 // to four dimensions with an extent and one stride per operand.

@@ -143,8 +143,10 @@ struct LzState {
 };
 
 // y = H x, one warp per row
-__global__ void k_matvec(long long n, const double* __restrict__ H, const double* __restrict__ x,
-                         double* __restrict__ y, const LzState* st) {
+// (x and y without __restrict__: what the kernel before wrote must not come
+// through the read-only path of a chained launch; H is the same for all)
+__global__ void k_matvec(long long n, const double* __restrict__ H, const double* x, double* y, const LzState* st) {
+  wait_for_previous();
   if (st && st->done) return;
   const long long row = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32;
   const int lane = threadIdx.x & 31;
@@ -159,11 +161,12 @@ __global__ void k_matvec(long long n, const double* __restrict__ H, const double
 // out[k] = V[k] . x for k < nv (V rows of length n), one CTA per k
 __global__ void __launch_bounds__(RX_T) k_dots(long long n, const double* V, const double* x, double* out,
                                                const LzState* st) {
+  wait_for_previous();
   if (st && st->done) return;
   __shared__ double sh[RX_T];
   const double* v = V + blockIdx.x * n;
   double s = 0.0;
-  for (long long i = threadIdx.x; i < n; i += RX_T) s += v[i] * x[i];
+  for (long long i = threadIdx.x; i < n; i += RX_T) s += __ldcg(v + i) * __ldcg(x + i);
   s = block_sum(s, sh);
   if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
@@ -183,8 +186,9 @@ struct LzStep {
 };
 
 template <bool LAST>
-__global__ void __launch_bounds__(RX_T) k_subtract(long long n, int nv, double* V, const double* __restrict__ coef,
-                                                   double* x, LzState* st, const LzStep p) {
+__global__ void __launch_bounds__(RX_T) k_subtract(long long n, int nv, double* V, const double* coef, double* x,
+                                                   LzState* st, const LzStep p) {
+  wait_for_previous();
   if (st && st->done) return;
   constexpr int NW = RX_T / 32;
   __shared__ double sh[NW][32];
@@ -195,7 +199,7 @@ __global__ void __launch_bounds__(RX_T) k_subtract(long long n, int nv, double* 
   double s = 0.0;
   if (i < n) {
 #pragma unroll 8
-    for (int k = warp; k < nv; k += NW) s += coef[k] * V[k * n + i];
+    for (int k = warp; k < nv; k += NW) s += __ldcg(coef + k) * __ldcg(V + k * n + i);
   }
   sh[warp][lane] = s;
   __syncthreads();
@@ -506,13 +510,13 @@ RelaxResult relaxed_ci(Handle& h, int order, int n_alpha, int n_beta) {
     for (int j = 0; j < mmax; ++j) {
       const double* vj = V.p + (long long)j * ndet;
       const int rec = ws.begin(K_CI_MATVEC, 2.0 * (double)ndet * (double)ndet, mv_bytes);
-      k_matvec<<<gw, 256, 0, st>>>(ndet, H.p, vj, w.p, lst);
+      check_cuda(launch_chained(k_matvec, gw, 256, st, ndet, H.p, vj, w.p, lst), "lanczos launch");
       ws.end(rec);
-      k_dots<<<j + 1, RX_T, 0, st>>>(ndet, V.p, w.p, coef, lst);
+      check_cuda(launch_chained(k_dots, j + 1, RX_T, st, ndet, V.p, w.p, coef, lst), "lanczos launch");
       const LzStep step{j, mmax, coef, alpha, beta, part.p, ticket};
-      k_subtract<false><<<gs, RX_T, 0, st>>>(ndet, j + 1, V.p, coef, w.p, lst, step);
-      k_dots<<<j + 1, RX_T, 0, st>>>(ndet, V.p, w.p, coef2, lst);
-      k_subtract<true><<<gs, RX_T, 0, st>>>(ndet, j + 1, V.p, coef2, w.p, lst, step);
+      check_cuda(launch_chained(k_subtract<false>, gs, RX_T, st, ndet, j + 1, V.p, coef, w.p, lst, step), "lanczos launch");
+      check_cuda(launch_chained(k_dots, j + 1, RX_T, st, ndet, V.p, w.p, coef2, lst), "lanczos launch");
+      check_cuda(launch_chained(k_subtract<true>, gs, RX_T, st, ndet, j + 1, V.p, coef2, w.p, lst, step), "lanczos launch");
       ws.launches += 4;
     }
     check_cuda(cudaGetLastError(), "lanczos launch");
