@@ -23,7 +23,8 @@ constexpr int CH_MAX_CTAS = 152 * 4;
 // sum, and an SM retires two FP64 operations a clock, so a step lasts as long
 // as the SM with the most rows: up to N = 152 x 96 each SM gets one CTA of 96
 // rows (with 256 threads at N = 13456 the factorisation used 53 of the 152
-// SMs, 40 us a vector on average; now 24 us, 22 us with chained launches).  Larger N fill the chip with 256.
+// SMs, 40 us a vector on average; now 24 us, 22 us with chained launches).
+// Larger N fill the chip with 256.
 constexpr long long CH_SMALL_N = 152LL * 96;
 constexpr int CH_Q = 512;  // earlier vectors whose pivot entries are held at a time
 

@@ -514,7 +514,13 @@ extern "C" int dsrg_df_ladder(int n, int naux, int p0, int np, int nh, const dou
   if (bp < 1) bp = 1;
   try {
     Workspace ws(st, scratch_pool());
-    if (!ladder_core_general(B, n, naux, p0, np, nh, t, L, 1LL << 27, ws)) {
+    bool done = false;
+    try {
+      done = ladder_core_general(B, n, naux, p0, np, nh, t, L, 1LL << 27, ws);
+    } catch (const Error& e) {
+      if (e.code != DSRG_ERR_OOM) throw;  // too little memory: the batched form needs less
+    }
+    if (!done) {
       const WorkspaceBlock rows(ws, (size_t)(bp * p3));
       check_cuda(cudaMemsetAsync(L, 0, (size_t)np * np * nh * nh * sizeof(double), st), "cudaMemsetAsync");
       const long long tst[4] = {(long long)np * nh * nh, (long long)nh * nh, nh, 1};

@@ -1297,7 +1297,7 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
   pb.TR = BN;
   pb.KT = KT;
   // spread a short output over more CTAs by splitting the k tiles
-  int splits = 1, ktper = KT;  // K < 2^31: the integer sums of a tile stay below 2^(31 + 12 + 21)
+  int splits = 1, ktper = KT;
   const long long ctas = (long long)MT * NT;
   if (ch.split_mode != 1 && ctas < 2 * 152 && KT >= 2 * OZ_SPLIT_MIN) {
     long long sp = (2 * 152 + ctas - 1) / ctas;
@@ -1307,6 +1307,13 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
       ktper = (KT + (int)sp - 1) / (int)sp;
       splits = (KT + ktper - 1) / ktper;
     }
+  }
+  // a tile's integer sums stay within 64 bits for any digits up to 2^26 k: at 8
+  // slices the lower half holds 5 pairs of 2^12 a k in units of 2^21, and less
+  constexpr int KT_MOST = 1 << 22;
+  if (ktper > KT_MOST) {
+    ktper = KT_MOST;
+    splits = (KT + ktper - 1) / ktper;
   }
   cudaStream_t st = ws.stream;
   size_t capA, capB, capE, capP = 0;
