@@ -175,13 +175,7 @@ int dsrg_init(const dsrg_inputs* in, const dsrg_options* opts, dsrg_handle** out
     h->naux = in->naux;
     h->n = in->nc + in->na + in->nv;
     h->s = in->s;
-    {
-      int dev = 0;
-      cudaDeviceProp prop{};
-      dsrg::check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
-      dsrg::check_cuda(cudaGetDeviceProperties(&prop, dev), "cudaGetDeviceProperties");
-      h->device_bytes = (double)prop.totalGlobalMem;
-    }
+    h->device_bytes = dsrg::device_memory();
     h->C = {0, in->nc};
     h->A = {in->nc, in->nc + in->na};
     h->V = {in->nc + in->na, h->n};

@@ -52,6 +52,19 @@ unsigned long long current_context_id() {
   return 0;
 }
 
+double device_memory() {
+  static std::mutex mu;
+  static std::map<int, double> known;
+  int dev = 0;
+  check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
+  std::lock_guard<std::mutex> lock(mu);
+  const auto it = known.find(dev);
+  if (it != known.end()) return it->second;
+  cudaDeviceProp prop{};
+  check_cuda(cudaGetDeviceProperties(&prop, dev), "cudaGetDeviceProperties");
+  return known[dev] = (double)prop.totalGlobalMem;
+}
+
 namespace {
 std::mutex g_pool_mu;
 cudaMemPool_t g_pool[64] = {};
