@@ -263,7 +263,14 @@ void eager_energy(dsrg::Handle& h, bool pt3, dsrg_energies* out) {
 // Capture one PT3 energy of h (status reset included) as a CUDA graph.  The
 // workspace cache is warm, so the captured buffers are the ones the eager
 // energy used; they stay reserved by the handle until the graph is dropped.
+// The arena that the captured energy leaves open is retired, whether the
+// capture succeeds or not: its memset is a node of the graph, which may never
+// be launched, so nothing outside the graph may take zeroed tensors from it.
 void capture_energy(dsrg::Handle& h) {
+  struct Retire {
+    dsrg::Workspace& ws;
+    ~Retire() { ws.retire_arena(); }
+  } retire{h.ws};
   const bool prof = h.ws.profiling;
   h.ws.profiling = false;
   dsrg::check_cuda(cudaStreamBeginCapture(h.stream, cudaStreamCaptureModeRelaxed), "cudaStreamBeginCapture");

@@ -96,8 +96,10 @@ class Workspace {
   // n zeroed doubles (n <= kArenaMost) out of an arena that is cleared as a
   // whole, so that the many small accumulators of an energy cost one memset;
   // released by arena_put.  retire_arena() ends the use of the open arena:
-  // what follows clears its own (an energy captured as a graph must hold the
-  // memset of everything it relies on).  Arenas of 1 MiB, which cudaMalloc
+  // what follows clears its own.  It is called on both sides of a capture: an
+  // energy captured as a graph must hold the memset of everything it relies
+  // on, and eager work must not rely on a memset that was only captured (the
+  // graph may never run).  Arenas of 1 MiB, which cudaMalloc
   // takes from a 2 MiB slab: with 4 MiB a new handle's first second-order
   // energy of a small molecule took 1060 us instead of 975, later ones the same.
   static constexpr size_t kArenaMost = 8192, kArenaSize = 1 << 17;
