@@ -16,9 +16,11 @@
 namespace dsrg {
 
 void check_cuda(cudaError_t e, const char* what) {
-  if (e != cudaSuccess)
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // reported here: the launch check of a later call must not find it again
     throw Error(e == cudaErrorMemoryAllocation ? DSRG_ERR_OOM : DSRG_ERR_CUDA,
                 std::string(what) + ": " + cudaGetErrorString(e));
+  }
 }
 
 // The current context's process-unique id, through driver entry points the
