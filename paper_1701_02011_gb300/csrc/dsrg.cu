@@ -78,10 +78,10 @@ Tensor vclass(Handle& h, const Iv* ivs, double coef) {
   int L[4] = {ivs[0].len(), ivs[1].len(), ivs[2].len(), ivs[3].len()};
   for (int k = 0; k < 4; ++k)
     if (L[k] <= 0) return V;
-  size_t capJ, capK;
   size_t nJ = (size_t)L[0] * L[1] * L[2] * L[3];
-  double* J = h.ws.get(nJ, capJ);
-  double* K = h.ws.get(nJ, capK);
+  const WorkspaceBlock bj(h.ws, nJ), bk(h.ws, nJ);
+  double* J = bj.p;
+  double* K = bk.p;
   check_cuda(cudaMemsetAsync(J, 0, nJ * sizeof(double), h.ws.stream), "memset");
   check_cuda(cudaMemsetAsync(K, 0, nJ * sizeof(double), h.ws.stream), "memset");
   df_integrals(h, ivs[0], ivs[1], ivs[2], ivs[3], J);  // (pr|qs) at [p,q,r,s]
@@ -98,8 +98,6 @@ Tensor vclass(Handle& h, const Iv* ivs, double coef) {
       raw_axpy4(h, -coef, K, sK, dK, v.st, L);
     }
   V.v.mask = conserving_mask(4);
-  h.ws.put(J, capJ);
-  h.ws.put(K, capK);
   return V;
 }
 
@@ -307,9 +305,9 @@ void df_ladder(Handle& h, const Tensor& T2, Tensor& C2, double coef) {
   if (p == 0 || hh == 0) return;
   const View& tv = T2.v;
   const double* t = tv.p + tv.boff[0b1010];  // spins (alpha, beta, alpha, beta)
-  size_t capL;
   size_t nL = (size_t)p * p * hh * hh;
-  double* L = h.ws.get(nL, capL);
+  const WorkspaceBlock bl(h.ws, nL);
+  double* L = bl.p;
   // batches of rows within a budget (DSRG_LADDER_BUDGET_MB, default 1024 MB);
   // the first-order alpha-beta amplitudes have t[r,s,i,j] = t[s,r,j,i], so the
   // pair-symmetric forms apply: with (pr|qs) over pairs held whole where that
@@ -349,7 +347,6 @@ void df_ladder(Handle& h, const Tensor& T2, Tensor& C2, double coef) {
     raw_axpy4(h, -coef, L, sLqp, blk(s, s, s, s), c.st, ext);
   }
   C2.v.mask |= conserving_mask(4);
-  h.ws.put(L, capL);
 }
 
 // ---------------------------------------------------------------------------
@@ -420,9 +417,9 @@ static void df_x2t1(Handle& h, const Tensor& T1, Tensor& C2, double coef) {
   for (int sg = 0; sg < 2; ++sg) has[sg] = (t.mask >> (sg | sg << 1)) & 1;
   if (!has[0] && !has[1]) return;
   // U^s at U + 2s blk: [X^s, Bc]; W^s at W + 2s blk: [Bc, X^s]
-  size_t capU, capW;
-  double* U = h.ws.get((size_t)(4 * blk), capU);
-  double* W = h.ws.get((size_t)(4 * blk), capW);
+  const WorkspaceBlock bu(h.ws, (size_t)(4 * blk)), bw(h.ws, (size_t)(4 * blk));
+  double* U = bu.p;
+  double* W = bw.p;
   check_cuda(cudaMemsetAsync(U, 0, (size_t)(4 * blk) * sizeof(double), h.ws.stream), "memset");
   check_cuda(cudaMemsetAsync(W, 0, (size_t)(4 * blk) * sizeof(double), h.ws.stream), "memset");
   {  // Bc[Q][p][r] = B[Q][P0+p][r] into U^s[1] and W^s[0]
@@ -468,8 +465,6 @@ static void df_x2t1(Handle& h, const Tensor& T1, Tensor& C2, double coef) {
                Dims2{{p, hh}, {hh, 1}, {c.st[0], c.st[3]}}, Dims2{{p, hh}, {hh, 1}, {c.st[1], c.st[2]}}, 1, ek, kk,
                kk);
     }
-  h.ws.put(U, capU);
-  h.ws.put(W, capW);
 }
 
 // C1[p,j] += coef sum_{q,r,s} V[p,q,r,s] D[r,s,q,j] on the excitation block
@@ -481,8 +476,8 @@ static void df_vd_onebody(Handle& h, const Tensor& D, Tensor& C1, double coef) {
   if (p == 0 || hh == 0) return;
   const long long n = h.n, n2 = n * n, P0 = h.nc, ph = (long long)p * hh;
   const View& d = D.v;
-  size_t capY;
-  double* Y = h.ws.get((size_t)(2 * Q * ph), capY);
+  const WorkspaceBlock by(h.ws, (size_t)(2 * Q * ph));
+  double* Y = by.p;
   check_cuda(cudaMemsetAsync(Y, 0, (size_t)(2 * Q * ph) * sizeof(double), h.ws.stream), "memset");
   bool has[2] = {false, false};
   for (int sg = 0; sg < 2; ++sg)
@@ -508,7 +503,6 @@ static void df_vd_onebody(Handle& h, const Tensor& D, Tensor& C1, double coef) {
     gemm22(h, 2.0 * coef, h.B + P0 * n + P0, Y + sg * Q * ph, c.p + c.boff[cb], Dims2{{1, p}, {0, n}, {0, c.st[0]}},
            Dims2{{1, hh}, {0, 1}, {0, c.st[1]}}, 2, ek, ak, bk);
   }
-  h.ws.put(Y, capY);
 }
 
 // ---------------------------------------------------------------------------

@@ -329,27 +329,18 @@ bool split_faster(Workspace& ws, const GemmArgs& g) {
   if (cs != cudaStreamCaptureStatusNone) return false;
   GemmArgs gz = g;
   gz.alpha = 0.0;
-  const bool prof = ws.profiling;
-  const long long launches = ws.launches;
-  ws.profiling = false;
-  cudaEvent_t e0, e1;
-  check_cuda(cudaEventCreate(&e0), "cudaEventCreate");
-  check_cuda(cudaEventCreate(&e1), "cudaEventCreate");
+  const TimingScope ts(ws);
   float ms[2] = {0.f, 0.f};
   for (int path = 0; path < 2; ++path) {
     for (int rep = 0; rep < 2; ++rep) {  // the second run is timed
-      check_cuda(cudaEventRecord(e0, ws.stream), "cudaEventRecord");
+      check_cuda(cudaEventRecord(ts.e0, ws.stream), "cudaEventRecord");
       if (path == 0) run_gemm_fp64(ws, gz, K_GEMM);
       else ozaki_gemm(ws, gz, ws.slices, (int)K_OZAKI_MMA);
-      check_cuda(cudaEventRecord(e1, ws.stream), "cudaEventRecord");
+      check_cuda(cudaEventRecord(ts.e1, ws.stream), "cudaEventRecord");
     }
-    check_cuda(cudaEventSynchronize(e1), "cudaEventSynchronize");
-    check_cuda(cudaEventElapsedTime(&ms[path], e0, e1), "cudaEventElapsedTime");
+    check_cuda(cudaEventSynchronize(ts.e1), "cudaEventSynchronize");
+    check_cuda(cudaEventElapsedTime(&ms[path], ts.e0, ts.e1), "cudaEventElapsedTime");
   }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  ws.profiling = prof;
-  ws.launches = launches;
   const bool split = ms[1] < ms[0];
   const int v = split ? 1 : 0;
   tune_cache_store("route", g.M, g.N, g.K, ws.slices, 1, &v);
@@ -383,35 +374,29 @@ void run_gemm_flat(Workspace& ws, const GemmArgs& g, const FlatTable& tab, int n
   const size_t O = (size_t)(g.M * g.N * g.nbatch);
   if (gemm_use_narrow(g)) {
     const NarrowPlan np = gemm_narrow_plan(g, tab.ngroups);
-    double* npart = nullptr;
-    size_t ncap = 0;
-    if (np.z > 1) npart = ws.get((size_t)tab.ngroups * np.z * O, ncap);
+    const WorkspaceBlock npart(ws, np.z > 1 ? (size_t)tab.ngroups * np.z * O : 0);
     const int r = ws.begin(K_GEMM, 2.0 * (double)g.M * (double)g.N * (double)g.K * npairs, 0.0);
     if (r >= 0) {
       ws.recs[r].m = g.M;
       ws.recs[r].n = g.N;
       ws.recs[r].k = g.K * npairs;
     }
-    launch_gemm_narrow(g, np, tab, npart, ws.stream);
+    launch_gemm_narrow(g, np, tab, npart.p, ws.stream);
     ws.end(r);
     if (np.z > 1) ws.launches++;
-    if (npart) ws.put(npart, ncap);
     return;
   }
   const FlatPlan fp = gemm_flat_plan(g, tab.ngroups);
-  double* fpart = nullptr;
-  size_t fcap = 0;
-  if (fp.z > 1) fpart = ws.get((size_t)tab.ngroups * fp.z * O, fcap);
+  const WorkspaceBlock fpart(ws, fp.z > 1 ? (size_t)tab.ngroups * fp.z * O : 0);
   int r = ws.begin(K_GEMM, 2.0 * (double)g.M * (double)g.N * (double)g.K * (double)g.nbatch * npairs, 0.0);
   if (r >= 0) {
     ws.recs[r].m = g.M;
     ws.recs[r].n = g.N;
     ws.recs[r].k = g.K * g.nbatch * npairs;
   }
-  launch_gemm_flat(g, fp, tab, fpart, ws.stream);
+  launch_gemm_flat(g, fp, tab, fpart.p, ws.stream);
   ws.end(r);
   if (fp.z > 1) ws.launches++;
-  if (fpart) ws.put(fpart, fcap);
 }
 }  // namespace
 
@@ -447,8 +432,7 @@ void run_gemm_fp64(Workspace& ws, const GemmArgs& g0, int kind) {
   int bm, bn;
   gemm_tile(g.M, g.N, kind == K_LADDER_BUILD ? 1 : kind == K_LADDER_CONTRACT ? 2 : 0, &bm, &bn);
   const long long tiles = ((g.M + bm - 1) / bm) * ((g.N + bn - 1) / bn) * g.nbatch;
-  double* part = nullptr;
-  size_t cap = 0;
+  size_t npart = 0;  // partial sums
   const bool small = kind == K_GEMM && gemm_is_small(g);
   const bool shortk = kind == K_GEMM && gemm_is_short(g);
   if (small && g.nbatch == 1 && g.K >= 4096) {
@@ -460,10 +444,9 @@ void run_gemm_fp64(Workspace& ws, const GemmArgs& g0, int kind) {
       long long kper = (g.K + s - 1) / s;
       s = (g.K + kper - 1) / kper;
       if (s >= 2) {
-        part = ws.get((size_t)(s * outs), cap);
+        npart = (size_t)(s * outs);
         g.splits = (int)s;
         g.kper = kper;
-        g.part = part;
       }
     }
   } else if (!small && !shortk && g.nbatch == 1 && tiles < 2 * 152 && g.K >= 64) {
@@ -477,13 +460,14 @@ void run_gemm_fp64(Workspace& ws, const GemmArgs& g0, int kind) {
       kper = (kper + 15) / 16 * 16;
       s = (g.K + kper - 1) / kper;
       if (s >= 2) {
-        part = ws.get((size_t)(s * g.M * g.N), cap);
+        npart = (size_t)(s * g.M * g.N);
         g.splits = (int)s;
         g.kper = kper;
-        g.part = part;
       }
     }
   }
+  const WorkspaceBlock part(ws, npart);  // stream order keeps later reuse behind the reduction
+  if (npart) g.part = part.p;
   int r = ws.begin(kind, 2.0 * (double)g.M * (double)g.N * (double)g.K * (double)g.nbatch, 0.0);
   if (r >= 0) {
     ws.recs[r].m = g.M;
@@ -493,7 +477,6 @@ void run_gemm_fp64(Workspace& ws, const GemmArgs& g0, int kind) {
   launch_gemm(g, ws.stream, kind == K_LADDER_BUILD ? 1 : kind == K_LADDER_CONTRACT ? 2 : 0);
   ws.end(r);
   if (g.splits > 1) ws.launches++;  // the split-K reduction
-  if (part) ws.put(part, cap);  // stream order keeps later reuse behind the reduction
 }
 }  // namespace
 
@@ -515,6 +498,21 @@ Workspace::~Workspace() {
   for (auto& b : free_) release(b.p);
   if (results) cudaFree(results);
   if (dot_scratch) cudaFree(dot_scratch);
+}
+
+TimingScope::TimingScope(Workspace& w) : ws(w), prof(w.profiling), launches(w.launches) {
+  check_cuda(cudaEventCreate(&e0), "cudaEventCreate");
+  const cudaError_t e = cudaEventCreate(&e1);
+  if (e != cudaSuccess) cudaEventDestroy(e0);
+  check_cuda(e, "cudaEventCreate");
+  ws.profiling = false;
+}
+
+TimingScope::~TimingScope() {
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  ws.profiling = prof;
+  ws.launches = launches;
 }
 
 cudaError_t Workspace::allocate(double** p, size_t n) {

@@ -157,15 +157,29 @@ class Workspace {
   const char* peak_tag_ = "";  // step being issued when the peak was reached
 };
 
-// A block of a workspace, put back when it goes out of scope.
+// A block of a workspace (none for n = 0), put back when it goes out of scope,
+// so that a call which runs out of memory half-way loses nothing.
 struct WorkspaceBlock {
   Workspace& ws;
   size_t cap = 0;
   double* p;
-  WorkspaceBlock(Workspace& w, size_t n) : ws(w), p(w.get(n, cap)) {}
+  WorkspaceBlock(Workspace& w, size_t n) : ws(w), p(n > 0 ? w.get(n, cap) : nullptr) {}
   ~WorkspaceBlock() { ws.put(p, cap); }
   WorkspaceBlock(const WorkspaceBlock&) = delete;
   WorkspaceBlock& operator=(const WorkspaceBlock&) = delete;
+};
+
+// Two events and a workspace that neither profiles nor counts launches while
+// candidates are timed; all put back when it goes out of scope.
+struct TimingScope {
+  Workspace& ws;
+  const bool prof;
+  const long long launches;
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  explicit TimingScope(Workspace& w);
+  ~TimingScope();
+  TimingScope(const TimingScope&) = delete;
+  TimingScope& operator=(const TimingScope&) = delete;
 };
 
 // Names the step issued while it is in scope (restores the outer name).

@@ -1316,15 +1316,12 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
     splits = (KT + ktper - 1) / ktper;
   }
   cudaStream_t st = ws.stream;
-  size_t capA, capB, capE, capP = 0;
   const size_t nA = (size_t)S * MT * KT * OZ_TILE_ELEMS, nB = (size_t)S * NT * KT * BN * OZ_BK;
-  double* bufA = ws.get((nA + 3) / 4, capA);  // bf16 digit tiles in double-sized blocks
-  double* bufB = ws.get((nB + 3) / 4, capB);
+  const WorkspaceBlock bufA(ws, (nA + 3) / 4), bufB(ws, (nB + 3) / 4);  // bf16 digit tiles in double-sized blocks
   const size_t nE = (size_t)MT * OZ_BM + (size_t)NT * BN;
-  double* bufE = ws.get((nE + 2 + 1) / 2, capE);
-  double* part = nullptr;
-  if (splits > 1) part = ws.get((size_t)splits * MT * OZ_BM * NT * BN, capP);
-  int* ea = (int*)bufE;
+  const WorkspaceBlock bufE(ws, (nE + 2 + 1) / 2);
+  const WorkspaceBlock part(ws, splits > 1 ? (size_t)splits * MT * OZ_BM * NT * BN : 0);
+  int* ea = (int*)bufE.p;
   int* fb = ea + (size_t)MT * OZ_BM;
   // algorithmic bytes: each operand element read twice (8 B each; once in the
   // one-pass form), S bf16 digits written
@@ -1345,7 +1342,7 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
     const long long q1 = (p.K + 7) / 8, q2 = (long long)p.KT * (OZ_BK / 8);
     pp.p[o] = pd.p[o] = p;
     pp.eu[o] = pd.eu[o] = (unsigned*)(o ? fb : ea);
-    pp.dst[o] = pd.dst[o] = (__nv_bfloat16*)(o ? bufB : bufA);
+    pp.dst[o] = pd.dst[o] = (__nv_bfloat16*)(o ? bufB.p : bufA.p);
     pp.kfast[o] = pd.kfast[o] = pack_kfast(p);
     pp.fR[o] = pd.fR[o] = make_fastdiv((unsigned)rows);
     pp.fQ[o] = make_fastdiv((unsigned)q1);
@@ -1393,8 +1390,8 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
     ws.launches += 1;  // two pack kernels (begin() counts one; the memset is not a kernel)
   }
   ws.end(r);
-  a.As = (const __nv_bfloat16*)bufA;
-  a.Bs = (const __nv_bfloat16*)bufB;
+  a.As = (const __nv_bfloat16*)bufA.p;
+  a.Bs = (const __nv_bfloat16*)bufB.p;
   a.ea = ea;
   a.fb = fb;
   a.sq = (const unsigned*)ea + nE;
@@ -1422,7 +1419,7 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
   a.wait_cycles = ws.wait_cycles > 0 ? ws.wait_cycles : OZ_WAIT_CYCLES;
   a.splits = splits;
   a.ktper = ktper;
-  a.part = part;
+  a.part = part.p;
   a.rowfast = (a.nM > 0 && a.nN > 0 && a.cM[a.nM - 1] < a.cN[a.nN - 1]) || (a.nN == 0 && a.nM > 0) ? 1 : 0;
   // timed as the tensor-core kernel whatever the contraction (kind is the
   // step it belongs to); flops: the FP64 product it computes, executed:
@@ -1439,10 +1436,6 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
   oz_launch_mma(a, MT, NT, BN, st);
   ws.end(r);
   if (splits > 1) ws.launches++;
-  ws.put(bufA, capA);
-  ws.put(bufB, capB);
-  ws.put(bufE, capE);
-  if (part) ws.put(part, capP);
 }
 
 }  // namespace
@@ -1510,31 +1503,22 @@ OzChoice choose(Workspace& ws, const GemmArgs& g0, int S, int kind) {
   }
   GemmArgs gz = g0;
   gz.alpha = 0.0;
-  const bool prof = ws.profiling;
-  const long long launches = ws.launches;
-  ws.profiling = false;
-  cudaEvent_t e0, e1;
-  check_cuda(cudaEventCreate(&e0), "cudaEventCreate");
-  check_cuda(cudaEventCreate(&e1), "cudaEventCreate");
+  const TimingScope ts(ws);
   OzChoice best = def;
   float best_ms = 1e30f;
   for (const OzChoice& c : cands) {
     ozaki_run(ws, gz, S, kind, c);  // first run: packing buffers, caches
-    check_cuda(cudaEventRecord(e0, ws.stream), "cudaEventRecord");
+    check_cuda(cudaEventRecord(ts.e0, ws.stream), "cudaEventRecord");
     ozaki_run(ws, gz, S, kind, c);
-    check_cuda(cudaEventRecord(e1, ws.stream), "cudaEventRecord");
-    check_cuda(cudaEventSynchronize(e1), "cudaEventSynchronize");
+    check_cuda(cudaEventRecord(ts.e1, ws.stream), "cudaEventRecord");
+    check_cuda(cudaEventSynchronize(ts.e1), "cudaEventSynchronize");
     float ms = 0.f;
-    check_cuda(cudaEventElapsedTime(&ms, e0, e1), "cudaEventElapsedTime");
+    check_cuda(cudaEventElapsedTime(&ms, ts.e0, ts.e1), "cudaEventElapsedTime");
     if (ms < best_ms) {
       best_ms = ms;
       best = c;
     }
   }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  ws.profiling = prof;
-  ws.launches = launches;
   const int v[2] = {best.bn, best.split_mode};
   tune_cache_store("tile", g0.M, g0.N, g0.K, S, 2, v);
   std::lock_guard<std::mutex> lock(g_tune_mu);
