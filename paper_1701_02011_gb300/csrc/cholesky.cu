@@ -216,7 +216,8 @@ extern "C" int dsrg_cholesky(long long N, const double* V, double tau, int max_v
   // scratch: D [N], per-CTA maxima, pivots [max_vecs], state
   const size_t bytes = (size_t)N * 8 + (size_t)grid * 16 + (size_t)max_vecs * 8 + sizeof(ChState) + 64;
   try {
-    Workspace ws(st, scratch_pool());
+    CallWorkspace call(st);
+    Workspace& ws = *call.ws;
     const WorkspaceBlock scratch(ws, (bytes + 7) / 8);
     double* D = scratch.p;
     double* pv = D + N;

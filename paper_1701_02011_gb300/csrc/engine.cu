@@ -73,12 +73,18 @@ cudaMemPool_t g_pool[64] = {};
 unsigned long long g_pool_ctx[64] = {};
 constexpr unsigned long long kPoolKeep = 1ULL << 30;  // bytes kept between calls
 
+// the current device's pool, nullptr if there is none (a pool dies with its
+// context, by cudaDeviceReset); g_pool_mu is held
+cudaMemPool_t live_pool() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+  return g_pool[dev] && g_pool_ctx[dev] == current_context_id() ? g_pool[dev] : nullptr;
+}
+
 // gives the memory that the current device's pool keeps back to the driver
 void scratch_trim() {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
   std::lock_guard<std::mutex> lock(g_pool_mu);
-  if (g_pool[dev] && g_pool_ctx[dev] == current_context_id()) cudaMemPoolTrimTo(g_pool[dev], 0);
+  if (cudaMemPool_t pool = live_pool()) cudaMemPoolTrimTo(pool, 0);
   cudaGetLastError();
 }
 }  // namespace
@@ -108,6 +114,15 @@ cudaMemPool_t scratch_pool() {
   g_pool[dev] = pool;
   g_pool_ctx[dev] = ctx;
   return pool;
+}
+
+void scratch_settle(cudaStream_t st) {
+  unsigned long long held = 0;
+  {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    if (cudaMemPool_t pool = live_pool()) cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held);
+  }
+  if (held > kPoolKeep) cudaStreamSynchronize(st);
 }
 
 namespace {
@@ -547,6 +562,7 @@ double* Workspace::get(size_t n, size_t& cap) {
       for (auto& b : free_) release(b.p);
       free_.clear();
       ++generation;
+      if (pool_) cudaStreamSynchronize(stream);  // until then the pool may count them as in use
       scratch_trim();
       check_cuda(allocate(&p, n), "cudaMalloc");
     }

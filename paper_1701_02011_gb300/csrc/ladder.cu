@@ -513,7 +513,8 @@ extern "C" int dsrg_df_ladder(int n, int naux, int p0, int np, int nh, const dou
   long long bp = ladder_batch_rows(np, 1LL << 27);  // at most 1 GiB of scratch
   if (bp < 1) bp = 1;
   try {
-    Workspace ws(st, scratch_pool());
+    CallWorkspace call(st);
+    Workspace& ws = *call.ws;
     bool done = false;
     try {
       done = ladder_core_general(B, n, naux, p0, np, nh, t, L, 1LL << 27, ws);

@@ -1553,7 +1553,8 @@ extern "C" int dsrg_split_gemm(long long M, long long N, long long K, const doub
   if (!A || !B || !C) return set_error(DSRG_ERR_ARG, "split gemm: NULL pointer");
   cudaStream_t st = (cudaStream_t)stream;
   try {
-    Workspace ws(st, scratch_pool());
+    CallWorkspace call(st);
+    Workspace& ws = *call.ws;
     const WorkspaceBlock flag(ws, 1);
     ws.oz_status = reinterpret_cast<int*>(flag.p);
     check_cuda(cudaMemsetAsync(ws.oz_status, 0, sizeof(int), st), "status reset");

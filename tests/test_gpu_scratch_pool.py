@@ -24,6 +24,19 @@ def _free(torch):
     return torch.cuda.mem_get_info()[0]
 
 
+def test_a_large_call_leaves_at_most_a_gib(lib):
+    import torch
+    n = 9216  # 8 slices: 1.4 GB of digits per operand
+    A = torch.ones((1, n), dtype=torch.float64, device="cuda").expand(n, n)
+    C = torch.zeros((n, n), dtype=torch.float64, device="cuda")
+    lib.dsrg_split_gemm(A[:256], A, C[:256], 1.0, 8)
+    torch.cuda.synchronize()
+    before = _free(torch)
+    lib.dsrg_split_gemm(A, A, C, 1.0, 8)
+    assert before - _free(torch) <= GIB + (64 << 20)
+    assert bool((C[256:] == n).all()) and bool((C[:256] == 2 * n).all())
+
+
 def test_out_of_memory_gives_back_what_was_taken(lib):
     import torch
     M, K = 16384, 8192  # 2.1 GB of digits per operand, 3 GiB left free
