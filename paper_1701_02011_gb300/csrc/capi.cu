@@ -249,8 +249,21 @@ void check_status(dsrg::Handle& h) {
 void eager_energy(dsrg::Handle& h, bool pt3, dsrg_energies* out) {
   h.drop_graph();  // the handle's tensors move to new buffers
   double e2 = 0, e3a = 0, e3b = 0;
-  reset_status(h);
-  dsrg::run_energy(h, pt3, &e2, &e3a, &e3b);
+  for (bool again = false;; again = true) {
+    h.ladder_whole = false;
+    try {
+      reset_status(h);
+      dsrg::run_energy(h, pt3, &e2, &e3a, &e3b);
+      break;
+    } catch (const dsrg::Error& e) {
+      // out of memory with the ladder's matrix held whole: once more in
+      // batches, now and from here on
+      if (e.code != DSRG_ERR_OOM || !h.ladder_whole || again) throw;
+      h.lean = true;
+      h.ladder_claim.drop();
+      h.ws.recover();
+    }
+  }
   check_status(h);
   h.warm = true;
   h.ws.prof_collect();
@@ -301,12 +314,62 @@ static int run(dsrg_handle* hd, bool pt3, dsrg_energies* out) {
   if (!hd || !hd->h) return fail(DSRG_ERR_STATE, "NULL handle");
   if (!out) return fail(DSRG_ERR_ARG, "out is NULL");
   try {
+    hd->h->batch = false;
     eager_energy(*hd->h, pt3, out);
   } catch (const std::exception& e) {
     return fail(classify(e), e.what());
   }
   return DSRG_OK;
 }
+
+namespace {
+void run_batch(dsrg_handle* const* hs, int n, dsrg_energies* out) {
+  // graphs: captured once per handle (after one eager energy), replayed after
+  for (int i = 0; i < n; ++i) {
+    dsrg::Handle& h = *hs[i]->h;
+    h.batch = true;
+    if (h.graph && h.graph_gen != h.ws.generation) h.drop_graph();
+    if (!h.graph) {
+      if (!h.warm) eager_energy(h, true, &out[i]);
+      capture_energy(h);
+    }
+  }
+  // every handle's energy in flight at once, each on its own stream
+  for (int i = 0; i < n; ++i) {
+    dsrg::Handle& h = *hs[i]->h;
+    dsrg::check_cuda(cudaGraphLaunch(h.graph, h.stream), "cudaGraphLaunch");
+  }
+  for (int i = 0; i < n; ++i) {
+    dsrg::Handle& h = *hs[i]->h;
+    double e2 = 0, e3a = 0, e3b = 0;
+    dsrg::finish_energy(h, &e2, &e3a, &e3b);
+    check_status(h);
+    out[i].e2 = e2;
+    out[i].e3a = e3a;
+    out[i].e3b = e3b;
+    out[i].e3 = e3a + e3b;
+  }
+}
+
+// After a batch ran out of memory: every handle drops its graph and its
+// cached blocks and computes its ladder in batches of rows from here on.
+// False if that changes nothing: no handle held the matrix of its ladder.
+bool make_lean(dsrg_handle* const* hs, int n) {
+  bool any = false;
+  for (int i = 0; i < n; ++i) any = any || (hs[i]->h->ladder_whole && !hs[i]->h->lean);
+  if (!any) return false;
+  for (int i = 0; i < n; ++i) {
+    dsrg::Handle& h = *hs[i]->h;
+    cudaStreamSynchronize(h.stream);  // another handle's graph may be in flight
+    h.drop_graph();
+    h.warm = false;
+    h.lean = true;
+    h.ladder_claim.drop();
+    h.ws.recover();
+  }
+  return true;
+}
+}  // namespace
 
 int dsrg_pt3_batch(dsrg_handle* const* hs, int n, dsrg_energies* out) {
   g_last_error.clear();
@@ -319,29 +382,11 @@ int dsrg_pt3_batch(dsrg_handle* const* hs, int n, dsrg_energies* out) {
       if (hs[j] == hs[i]) return fail(DSRG_ERR_ARG, "a handle appears twice in the batch");
   }
   try {
-    // graphs: captured once per handle (after one eager energy), replayed after
-    for (int i = 0; i < n; ++i) {
-      dsrg::Handle& h = *hs[i]->h;
-      if (h.graph && h.graph_gen != h.ws.generation) h.drop_graph();
-      if (!h.graph) {
-        if (!h.warm) eager_energy(h, true, &out[i]);
-        capture_energy(h);
-      }
-    }
-    // every handle's energy in flight at once, each on its own stream
-    for (int i = 0; i < n; ++i) {
-      dsrg::Handle& h = *hs[i]->h;
-      dsrg::check_cuda(cudaGraphLaunch(h.graph, h.stream), "cudaGraphLaunch");
-    }
-    for (int i = 0; i < n; ++i) {
-      dsrg::Handle& h = *hs[i]->h;
-      double e2 = 0, e3a = 0, e3b = 0;
-      dsrg::finish_energy(h, &e2, &e3a, &e3b);
-      check_status(h);
-      out[i].e2 = e2;
-      out[i].e3a = e3a;
-      out[i].e3b = e3b;
-      out[i].e3 = e3a + e3b;
+    try {
+      run_batch(hs, n, out);
+    } catch (const dsrg::Error& e) {
+      if (e.code != DSRG_ERR_OOM || !make_lean(hs, n)) throw;
+      run_batch(hs, n, out);
     }
   } catch (const std::exception& e) {
     return fail(classify(e), e.what());
@@ -364,6 +409,7 @@ int dsrg_relaxed(dsrg_handle* hd, int n_alpha, int n_beta, dsrg_relaxed_energies
   } flag{h};
   try {
     h.relax = true;
+    h.batch = false;
     dsrg_energies e{};
     eager_energy(h, true, &e);
     h.relax = false;

@@ -310,17 +310,37 @@ void df_ladder(Handle& h, const Tensor& T2, Tensor& C2, double coef) {
   double* L = bl.p;
   // batches of rows within a budget (DSRG_LADDER_BUDGET_MB, default 1024 MB);
   // the first-order alpha-beta amplitudes have t[r,s,i,j] = t[s,r,j,i], so the
-  // pair-symmetric forms apply: with (pr|qs) over pairs held whole where that
-  // takes at most an eighth of the device (p <= 364 on 284 GB) or the stated
-  // budget, else in batches
-  double budget_mb = 1024.0, whole = h.device_bytes / 8.0;
+  // pair-symmetric forms apply: with (pr|qs) over pairs (2 p^4 bytes) held
+  // whole, or in batches, which take about twice as long.  Whole where the
+  // matrix is at most a 32nd of the device (8.9 of 284 GB: p <= 258) or as
+  // large as five of the energy's [P,P,H,H] tensors, and at most an eighth of
+  // the device (p <= 364); or where it is within the stated budget.  The rule
+  // looks at sizes only, so that a handle's energies agree to the last bit
+  // whatever else is on the device; an energy that runs out of memory is
+  // computed again in batches (h.lean).
+  double budget_mb = 1024.0;
+  const double five = 240.0 * (double)p * p * hh * hh, least = h.device_bytes / 32.0, most = h.device_bytes / 8.0;
+  double whole = five > least ? five < most ? five : most : least;
   if (const char* env = getenv("DSRG_LADDER_BUDGET_MB")) {
     budget_mb = atof(env);
     whole = budget_mb * 1048576.0;
   }
+  if (h.lean) whole = -1.0;
   long long maxd = (long long)(budget_mb * 131072.0);
   const long long tst[4] = {tv.st[0], tv.st[1], tv.st[2], tv.st[3]};
-  if (!ladder_core_pairs(h.B, h.n, h.naux, h.nc, p, hh, t, tst, L, maxd, whole, h.ws)) {
+  const double pairs = 0.5 * p * (p + 1.0);
+  h.ladder_whole = 8.0 * pairs * pairs <= whole;
+  bool done = false;
+  if (h.ladder_whole) {
+    // the matrix and its rows are scratch of this call, from the pool that all
+    // handles share, unless a graph will refer to them or they are so small
+    // that asking for them each time would show
+    const bool shared = !h.batch && 8.0 * pairs * pairs > 64e6;
+    Workspace scratch(h.ws.stream, shared ? scratch_pool() : nullptr, &h.ws);
+    if (shared) h.ladder_claim.raise((unsigned long long)(8.0 * pairs * pairs));
+    done = ladder_core_pairs(h.B, h.n, h.naux, h.nc, p, hh, t, tst, L, maxd, whole, h.ws, shared ? scratch : h.ws);
+  }
+  if (!done) {
     check_cuda(cudaMemsetAsync(L, 0, nL * sizeof(double), h.ws.stream), "memset");
     const long long p3 = (long long)p * p * p;
     if (maxd < p3) maxd = p3;  // one row p with every q >= p0 (the first batch)

@@ -46,6 +46,11 @@ struct Handle {
   cudaGraphExec_t graph = nullptr;
   unsigned long long graph_gen = 0;
   bool warm = false;  // one eager energy has filled the workspace cache
+  // the energy's ladder (df_ladder): the last energy held (pr|qs) whole; it
+  // may not (device memory ran out with it); the energy is one of a batch,
+  // whose graph needs the matrix for as long as it lives
+  bool ladder_whole = false, lean = false, batch = false;
+  ScratchClaim ladder_claim;  // so that the pool keeps the matrix for the next energy
   void drop_graph() {
     if (graph) cudaGraphExecDestroy(graph);
     graph = nullptr;

@@ -11,6 +11,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <set>
 #include <stdexcept>
 
 namespace dsrg {
@@ -72,6 +73,10 @@ std::mutex g_pool_mu;
 cudaMemPool_t g_pool[64] = {};
 unsigned long long g_pool_ctx[64] = {};
 constexpr unsigned long long kPoolKeep = 1ULL << 30;  // bytes kept between calls
+std::multiset<unsigned long long> g_claims[64];
+
+// bytes the pool of device dev keeps; g_pool_mu is held
+unsigned long long pool_keep(int dev) { return kPoolKeep + (g_claims[dev].empty() ? 0 : *g_claims[dev].rbegin()); }
 
 // the current device's pool, nullptr if there is none (a pool dies with its
 // context, by cudaDeviceReset); g_pool_mu is held
@@ -105,7 +110,7 @@ cudaMemPool_t scratch_pool() {
   props.location.type = cudaMemLocationTypeDevice;
   props.location.id = dev;
   cudaMemPool_t pool = nullptr;
-  unsigned long long keep = kPoolKeep;
+  unsigned long long keep = pool_keep(dev);
   if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
@@ -116,13 +121,45 @@ cudaMemPool_t scratch_pool() {
   return pool;
 }
 
+void ScratchClaim::raise(unsigned long long bytes) {
+  int dev = 0;
+  if (bytes <= bytes_ || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
+  drop();
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  g_claims[dev].insert(bytes);
+  dev_ = dev;
+  bytes_ = bytes;
+  unsigned long long keep = pool_keep(dev);
+  if (cudaMemPool_t pool = live_pool()) cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+}
+
+void ScratchClaim::drop() {
+  if (dev_ < 0) return;
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  g_claims[dev_].erase(g_claims[dev_].find(bytes_));
+  unsigned long long keep = pool_keep(dev_);
+  int dev = 0;
+  // on another device the pool adjusts itself at a later claim or trim
+  if (cudaGetDevice(&dev) == cudaSuccess && dev == dev_)
+    if (cudaMemPool_t pool = live_pool()) {
+      cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+      cudaMemPoolTrimTo(pool, keep);
+    }
+  cudaGetLastError();
+  dev_ = -1;
+  bytes_ = 0;
+}
+
 void scratch_settle(cudaStream_t st) {
-  unsigned long long held = 0;
+  unsigned long long held = 0, keep = kPoolKeep;
   {
     std::lock_guard<std::mutex> lock(g_pool_mu);
-    if (cudaMemPool_t pool = live_pool()) cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held);
+    if (cudaMemPool_t pool = live_pool()) {
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held);
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    }
   }
-  if (held > kPoolKeep) cudaStreamSynchronize(st);
+  if (held > keep) cudaStreamSynchronize(st);
 }
 
 namespace {
@@ -557,23 +594,47 @@ double* Workspace::get(size_t n, size_t& cap) {
     free_.erase(free_.begin() + bi);
   } else {
     if (allocate(&p, n) != cudaSuccess) {
-      // drop cached blocks, here and in the scratch pool, and retry once
+      // drop cached blocks, here and in the scratch pool, and retry once.  Not
+      // while the stream is being captured: blocks put back since then are
+      // operands of the nodes captured so far.
       cudaGetLastError();
-      for (auto& b : free_) release(b.p);
-      free_.clear();
-      ++generation;
-      if (pool_) cudaStreamSynchronize(stream);  // until then the pool may count them as in use
+      cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+      if (cudaStreamIsCapturing(stream, &cs) != cudaSuccess) cudaGetLastError();
+      if (cs == cudaStreamCaptureStatusNone) {
+        for (auto& b : free_) release(b.p);
+        free_.clear();
+        ++generation;
+        cudaStreamSynchronize(stream);  // until then the pool may count what was freed as in use
+      }
       scratch_trim();
       check_cuda(allocate(&p, n), "cudaMalloc");
     }
   }
-  in_use_ += got * sizeof(double);
+  account((long long)got);
+  cap = got;
+  return p;
+}
+
+void Workspace::account(long long n) {
+  if (counted_) counted_->account(n);
+  in_use_ += n * (long long)sizeof(double);
   if (in_use_ > peak_) {
     peak_ = in_use_;
     peak_tag_ = tag;
   }
-  cap = got;
-  return p;
+}
+
+void Workspace::recover() {
+  cudaStreamSynchronize(stream);
+  for (auto& r : recs) {
+    ev_pool.push_back(r.a);
+    ev_pool.push_back(r.b);
+  }
+  recs.clear();
+  retire_arena();
+  for (auto& b : free_) release(b.p);
+  free_.clear();
+  ++generation;
 }
 
 double* Workspace::get_zeroed(size_t n, int& arena) {
@@ -622,7 +683,7 @@ void Workspace::retire_arena() {
 
 void Workspace::put(double* p, size_t cap) {
   if (!p) return;
-  in_use_ -= cap * sizeof(double);
+  account(-(long long)cap);
   free_.push_back({p, cap});
 }
 

@@ -90,7 +90,9 @@ class Workspace {
  public:
   // pool: blocks come from this stream-ordered pool and go back to it (the
   // entry points that own no handle), else from cudaMalloc
-  explicit Workspace(cudaStream_t st, cudaMemPool_t pool = nullptr) : stream(st), pool_(pool) {}
+  // counted: workspace whose bytes_in_use and peak_bytes count this one's blocks
+  explicit Workspace(cudaStream_t st, cudaMemPool_t pool = nullptr, Workspace* counted = nullptr)
+      : stream(st), pool_(pool), counted_(counted) {}
   ~Workspace();
   double* get(size_t n, size_t& cap);
   void put(double* p, size_t cap);
@@ -107,6 +109,9 @@ class Workspace {
   double* get_zeroed(size_t n, int& arena);
   void arena_put(int arena);
   void retire_arena();
+  // After a call that ran out of memory: waits for the stream, forgets the
+  // timings begun and frees every cached block.  No graph may refer to them.
+  void recover();
   size_t bytes_in_use() const { return in_use_; }
   size_t peak_bytes() const { return peak_; }
   cudaStream_t stream;
@@ -148,8 +153,10 @@ class Workspace {
  private:
   cudaError_t allocate(double** p, size_t n);
   void release(double* p);
+  void account(long long n);
   struct Blk { double* p; size_t n; };
   cudaMemPool_t pool_ = nullptr;
+  Workspace* counted_ = nullptr;
   std::vector<Blk> free_;
   struct Arena { double* p = nullptr; size_t cap = 0, used = 0; int live = 0; };
   std::vector<Arena> arenas_;
@@ -260,6 +267,23 @@ void check_cuda(cudaError_t e, const char* what);
 // when an allocation of this library fails; the driver orders reuse across
 // streams and threads.  nullptr (plain cudaMalloc) where no pool can be had.
 cudaMemPool_t scratch_pool();
+// What a handle asks the pool to keep beyond that while the handle lives: the
+// largest claim on a device, not their sum (given back like the rest when an
+// allocation fails).  Without it the 7.6 GB of (pr|qs) of 248 particles were
+// mapped anew for every energy: 9 of 720 ms.
+class ScratchClaim {
+ public:
+  ScratchClaim() = default;
+  ~ScratchClaim() { drop(); }
+  ScratchClaim(const ScratchClaim&) = delete;
+  ScratchClaim& operator=(const ScratchClaim&) = delete;
+  void raise(unsigned long long bytes);  // for the current device
+  void drop();
+
+ private:
+  int dev_ = -1;
+  unsigned long long bytes_ = 0;
+};
 // One more synchronisation of st if the pool holds more than it keeps.
 void scratch_settle(cudaStream_t st);
 // Workspace of a call without a handle, on that pool.  Calls that took less

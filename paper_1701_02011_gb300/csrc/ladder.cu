@@ -355,16 +355,16 @@ constexpr long long kMaxRows = 65535;  // gridDim.y
 // max_doubles bounds a batch of G+- rows, m_bytes the matrix; false (nothing
 // done) where the matrix does not fit.
 bool ladder_core_pairs(const double* B, long long n, int naux, int p0, int np, int nh, const double* t,
-                       const long long* tst, double* L, long long max_doubles, double m_bytes, Workspace& ws) {
+                       const long long* tst, double* L, long long max_doubles, double m_bytes, Workspace& ws,
+                       Workspace& mws) {
   if (np <= 0 || nh <= 0) return true;
   const long long pairs = pair_index(np, 0);
   if ((double)pairs * (double)pairs * 8.0 > m_bytes || pairs >= (1LL << 31)) return false;
   cudaStream_t st = ws.stream;
-  const char* outer = ws.tag;
-  ws.tag = "ladder-build";
-  WorkspaceBlock M(ws, (size_t)(pairs * pairs));
+  ProfTag tag_(ws, "ladder-build");
+  WorkspaceBlock M(mws, (size_t)(pairs * pairs));
   {
-    WorkspaceBlock Bp(ws, (size_t)(naux * pairs));
+    WorkspaceBlock Bp(mws, (size_t)(naux * pairs));
     int r = ws.begin(K_AXPY, 0.0, 16.0 * (double)naux * (double)pairs);
     k_ladder_b<<<dim3(blocks_for(pairs, 256, 1024), blocks_for(naux, 1, 64)), 256, 0, st>>>(B, n, p0, np, naux, Bp.p);
     ws.end(r);
@@ -390,7 +390,7 @@ bool ladder_core_pairs(const double* B, long long n, int naux, int p0, int np, i
   tp.sym = 1;
   tp.cp = pair_index(nh, 0);
   tp.cm = tp.cp - nh;
-  WorkspaceBlock plus(ws, (size_t)(pairs * tp.cp)), minus(ws, (size_t)(pairs * tp.cm));
+  WorkspaceBlock plus(mws, (size_t)(pairs * tp.cp)), minus(mws, (size_t)(pairs * tp.cm));
   tp.plus = plus.p;
   tp.minus = minus.p;
   pair_amplitudes(ws, tp);
@@ -398,8 +398,8 @@ bool ladder_core_pairs(const double* B, long long n, int naux, int p0, int np, i
   if (rows > 128) rows = rows / 128 * 128;
   rows = rows < 1 ? 1 : rows > kMaxRows ? kMaxRows : rows;
   if (rows > pairs) rows = pairs;
-  WorkspaceBlock gp(ws, (size_t)(rows * pairs)), gm(ws, (size_t)(rows * pairs)), lp(ws, (size_t)(rows * tp.cp)),
-      lm(ws, (size_t)(rows * tp.cm));
+  WorkspaceBlock gp(mws, (size_t)(rows * pairs)), gm(mws, (size_t)(rows * pairs)), lp(mws, (size_t)(rows * tp.cp)),
+      lm(mws, (size_t)(rows * tp.cm));
   for (long long r0 = 0; r0 < pairs; r0 += rows) {
     const long long nr = r0 + rows < pairs ? rows : pairs - r0;
     const int r = ws.begin(K_AXPY, 0.0, 32.0 * (double)nr * (double)pairs);
@@ -408,7 +408,6 @@ bool ladder_core_pairs(const double* B, long long n, int naux, int p0, int np, i
     pair_contract(ws, tp, gp.p, gm.p, lp.p, lm.p, r0, nr, L);
   }
   check_cuda(cudaGetLastError(), "ladder launch");
-  ws.tag = outer;
   return true;
 }
 

@@ -22,10 +22,11 @@ void ladder_core_sym(const double* B, long long n, int naux, int p0, int np, int
                      Workspace* ws);
 // The same sums in pair form (see ladder.cu); false, and nothing done, where
 // the memory named does not suffice.  _pairs: B symmetric in its last two
-// indices and t as for ladder_core_sym; _general: any B and t (contiguous).
-// L is overwritten.
+// indices and t as for ladder_core_sym (its blocks come from mws);
+// _general: any B and t (contiguous).  L is overwritten.
 bool ladder_core_pairs(const double* B, long long n, int naux, int p0, int np, int nh, const double* t,
-                       const long long* tst, double* L, long long max_doubles, double m_bytes, Workspace& ws);
+                       const long long* tst, double* L, long long max_doubles, double m_bytes, Workspace& ws,
+                       Workspace& mws);
 bool ladder_core_general(const double* B, long long n, int naux, int p0, int np, int nh, const double* t, double* L,
                          long long max_doubles, Workspace& ws);
 // Largest batch of p rows whose (pr|qs) fits in max_doubles (0 if none).
