@@ -331,7 +331,15 @@ void run_batch(dsrg_handle* const* hs, int n, dsrg_energies* out) {
     if (h.graph && h.graph_gen != h.ws.generation) h.drop_graph();
     if (!h.graph) {
       if (!h.warm) eager_energy(h, true, &out[i]);
-      capture_energy(h);
+      try {
+        capture_energy(h);
+      } catch (const dsrg::Error& e) {
+        // once more without the blocks cached by earlier calls: a capture may
+        // not free them itself (Workspace::get)
+        if (e.code != DSRG_ERR_OOM) throw;
+        h.ws.recover();
+        capture_energy(h);
+      }
     }
   }
   // every handle's energy in flight at once, each on its own stream

@@ -34,10 +34,13 @@ def _free():
 
 
 class Batched:
-    """(pr|qs) in batches within 1 GiB"""
+    """(pr|qs) in batches within 1 GiB (or as much as is said)"""
+
+    def __init__(self, mb=1024):
+        self.mb = mb
 
     def __enter__(self):
-        os.environ["DSRG_LADDER_BUDGET_MB"] = "1024"
+        os.environ["DSRG_LADDER_BUDGET_MB"] = str(self.mb)
 
     def __exit__(self, *a):
         os.environ.pop("DSRG_LADDER_BUDGET_MB", None)
@@ -117,3 +120,22 @@ def test_idle_handles_keep_one_matrix_between_them(lib):
             h.close()
         assert before - _free() <= GIB + (64 << 20)
     assert used[1] <= used[0] + 3230 * 10 ** 6 + GIB + (256 << 20)
+
+
+def test_capture_without_the_blocks_of_earlier_calls(lib):
+    """An energy in batches of 4 GiB leaves a block that batches of 1 GiB do not
+    use; with half a GiB free the capture fits only without it."""
+    inst = _instance(216)  # 218 particles: the matrix would take 4.5 GB
+    with Batched():
+        h = lib.Dsrg(inst)
+        e = h.pt3()
+        h.close()
+    with Batched(4096):
+        h = lib.Dsrg(inst)
+        h.pt3()
+    try:
+        with Filled(GIB // 2), Batched():
+            assert lib.dsrg_pt3_batch([h]) == [e]
+            assert lib.dsrg_pt3_batch([h]) == [e]
+    finally:
+        h.close()
