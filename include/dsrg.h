@@ -259,10 +259,13 @@ long long dsrg_peak_bytes(const dsrg_handle *h);
  * current GPU; stream may be NULL (legacy default stream).  With t the
  * alpha-beta block of the spin-free first-order amplitudes this is the
  * spatial ladder from which the energy driver assembles all spin blocks.
- * The (pr|qs) rows are formed in batches in scratch of at most 1 GiB (and up
- * to 256 MiB of partial sums) from the library's stream-ordered memory pool,
- * given back before return (the pool keeps at most 1 GiB per device between
- * calls); the call synchronises `stream`.  Errors: DSRG_ERR_ARG (sizes, p0 + np > n, NULL
+ * Neither B nor t need any symmetry, and every element of L is the sum of its
+ * own products: a small L[p][q] beside a large L[q][p] has an error of its own
+ * size.  The (pr|qs) rows are formed in batches in scratch of at most 1 GiB
+ * (or one row, np^3 doubles, if that is more; less where less is free) from
+ * the library's stream-ordered memory pool, given back before return (the pool
+ * keeps at most 1 GiB per device between calls); the call synchronises
+ * `stream`.  Errors: DSRG_ERR_ARG (sizes, p0 + np > n, NULL
  * pointers), DSRG_ERR_OOM (scratch), DSRG_ERR_CUDA.
  */
 int dsrg_df_ladder(int n, int naux, int p0, int np, int nh, const double *B, const double *t, double *L,

@@ -345,7 +345,7 @@ void df_ladder(Handle& h, const Tensor& T2, Tensor& C2, double coef) {
     const long long p3 = (long long)p * p * p;
     if (maxd < p3) maxd = p3;  // one row p with every q >= p0 (the first batch)
     WorkspaceBlock G(h.ws, (size_t)maxd);
-    ladder_core_sym(h.B, h.n, h.naux, h.nc, p, hh, t, tst, L, G.p, maxd, h.ws.stream, &h.ws);
+    ladder_core_half(h.B, h.n, h.naux, h.nc, p, hh, t, tst, true, L, G.p, maxd, p, h.ws.stream, &h.ws);
   }
   // scatter into the spin blocks of C2 [2p][2p][2h][2h]
   const View& c = C2.v;

@@ -61,14 +61,16 @@ void ladder_core(const double* B, long long n, int naux, int p0, int np, int nh,
   }
 }
 
-// Pair-symmetric variant where the pair form below does not fit: with t[r,s,i,j] = t[s,r,j,i] (the alpha-beta block
-// of a spin-free T2) and (pr|qs) = (qs|pr), L[q,p,i,j] = L[p,q,j,i], so a
-// batch of rows p in [e0, e1) builds and contracts (pr|qs) only for
-// q >= e0 and writes the rows q >= e1 of the mirror image by a transposed
-// copy.  About half of the build and contraction work of ladder_core.
-void ladder_core_sym(const double* B, long long n, int naux, int p0, int np, int nh, const double* t,
-                     const long long* tst, double* L, double* G, long long max_doubles, cudaStream_t st,
-                     Workspace* ws) {
+// By (pr|qs) = (qs|pr), a batch of rows p in [e0, e1) builds (pr|qs) only for
+// q >= e0, half of the build of ladder_core.  It contracts them with t[r,s] into
+// the rows L[p, q >= e0] and, for q >= e1, into L[q,p] = sum_{r,s} (pr|qs) t[s,r];
+// with t[r,s,i,j] = t[s,r,j,i] (t_sym: the alpha-beta block of a spin-free T2)
+// L[q,p,i,j] = L[p,q,j,i] instead, by a transposed copy.  Either way every
+// element of L is the plain sum of its own products.  most_rows bounds a
+// batch: the rows p, q within it are built twice.
+void ladder_core_half(const double* B, long long n, int naux, int p0, int np, int nh, const double* t,
+                      const long long* tst, bool t_sym, double* L, double* G, long long max_doubles, long long most_rows,
+                      cudaStream_t st, Workspace* ws) {
   if (np <= 0 || nh <= 0) return;
   const long long p2 = (long long)np * np, h2 = (long long)nh * nh;
   if (max_doubles < np * p2) throw std::runtime_error("ladder: scratch below one row of (pr|qs)");
@@ -76,6 +78,7 @@ void ladder_core_sym(const double* B, long long n, int naux, int p0, int np, int
   while (e0 < np) {
     const long long nf = np - e0;  // q in [e0, np)
     long long nb = max_doubles / (nf * p2);
+    if (nb > most_rows) nb = most_rows;
     if (nb < 1) nb = 1;
     if (nb > nf) nb = nf;
     const long long e1 = e0 + nb;
@@ -104,29 +107,32 @@ void ladder_core_sym(const double* B, long long n, int naux, int p0, int np, int
       else launch_gemm(g, st, 1);
     }
     if (ws) ws->tag = "ladder-contract";
-    {  // L[e, q, i, j] += sum_{r,s} G[e, q - e0, r, s] t[r, s, i, j]
+    // L[e, q, i, j] (swap: L[q, e, i, j]) += sum_{r,s} G[e, q - e0, r, s] t[r, s, i, j] (t[s, r, i, j]), q in [q0, np)
+    auto contract = [&](long long q0, bool swap) {
       GemmArgs g{};
-      g.A = G;
+      g.A = G + (q0 - e0) * p2;
       g.B = t;
-      g.C = L + (e0 * np + e0) * h2;
+      g.C = L + (swap ? q0 * np + e0 : e0 * np + q0) * h2;
       g.alpha = 1.0;
       g.nM = 2;
-      g.eM[0] = (int)nb; g.aM[0] = nf * p2; g.cM[0] = np * h2;
-      g.eM[1] = (int)nf; g.aM[1] = p2;      g.cM[1] = h2;
+      g.eM[0] = (int)nb;        g.aM[0] = nf * p2; g.cM[0] = swap ? h2 : np * h2;
+      g.eM[1] = (int)(np - q0); g.aM[1] = p2;      g.cM[1] = swap ? np * h2 : h2;
       g.nK = 2;
-      g.eK[0] = np; g.aK[0] = np; g.bK[0] = tst[0];
-      g.eK[1] = np; g.aK[1] = 1;  g.bK[1] = tst[1];
+      g.eK[0] = np; g.aK[0] = np; g.bK[0] = tst[swap ? 1 : 0];
+      g.eK[1] = np; g.aK[1] = 1;  g.bK[1] = tst[swap ? 0 : 1];
       g.nN = 2;
       g.eN[0] = nh; g.bN[0] = tst[2]; g.cN[0] = nh;
       g.eN[1] = nh; g.bN[1] = tst[3]; g.cN[1] = 1;
-      g.M = nb * nf;
+      g.M = nb * (np - q0);
       g.N = h2;
       g.K = p2;
       g.nbatch = 1;
       if (ws) run_gemm(*ws, g, K_LADDER_CONTRACT);
       else launch_gemm(g, st, 2);
-    }
-    if (e1 < np) {  // L[q, e, i, j] = L[e, q, j, i] for e in [e0, e1), q in [e1, np)
+    };
+    contract(e0, false);
+    if (e1 < np && !t_sym) contract(e1, true);
+    if (e1 < np && t_sym) {  // L[q, e, i, j] = L[e, q, j, i] for e in [e0, e1), q in [e1, np)
       NdArgs a{};
       a.nd = 4;
       a.e[0] = (int)nb;       a.sa[0] = np * h2; a.sb[0] = h2;
@@ -147,19 +153,20 @@ void ladder_core_sym(const double* B, long long n, int naux, int p0, int np, int
 // ---------------------------------------------------------------------------
 // pair form
 // ---------------------------------------------------------------------------
-// With t+-[rs] = (t[r,s] +- t[s,r]) / 2 and G+-[pq,rs] = (pr|qs) +- (ps|qr),
+// For B symmetric in its last two indices and t[r,s,i,j] = t[s,r,j,i] (a spin-free
+// T2).  With t+-[rs] = (t[r,s] +- t[s,r]) / 2 and G+-[pq,rs] = (pr|qs) +- (ps|qr),
 // r >= s, p >= q (the sum once for r = s),
-//   L[p,q] = S + D,  L[q,p] = S - D,  S = sum_{r >= s} G+ t+,  D = sum_{r > s} G- t-:
-// two contractions of a quarter of the full one's size.  If t[r,s,i,j] =
-// t[s,r,j,i] as well (a spin-free T2), t+- is symmetric or antisymmetric in
-// i, j and only i >= j is needed: an eighth each.  If B is symmetric in its
-// last two indices (pr|qs) is one symmetric matrix over pairs (p >= r),
-// (q >= s), an eighth of the full build.
+//   L[p,q] = S + D,  L[q,p] = S - D,  S = sum_{r >= s} G+ t+,  D = sum_{r > s} G- t-.
+// t+- is symmetric or antisymmetric in i, j, so only i >= j is needed: two
+// contractions of an eighth of the full one's size each; (pr|qs) is one
+// symmetric matrix over pairs (p >= r), (q >= s), an eighth of the full build.
+// An L[p,q] much smaller than L[q,p] has an error of the size of the latter's: right
+// for an energy, which sums over both, not for a caller's own t and L
+// (dsrg_df_ladder takes ladder_core_rows).
 // Bound: the FP64 (or tensor) pipe of the two products.  np = 106, nh = 16, 400
-// auxiliary functions, FP64: general 140 -> 85 ms; symmetric (the energy) build
-// 81 -> 12.6 ms, contraction 58 -> 17 ms, G+- rows 0.27 ms, mirror 0.06 ms.
-// np = 248, nh = 28, split: build and contraction 130 -> 60 ms, of which the
-// G+- rows 8.3 ms.
+// auxiliary functions, FP64: build 81 -> 12.6 ms, contraction 58 -> 17 ms, G+- rows
+// 0.27 ms, mirror 0.06 ms.  np = 248, nh = 28, split: build and contraction 130 ->
+// 60 ms, of which the G+- rows 8.3 ms.
 namespace {
 __host__ __device__ inline long long pair_index(long long a, long long b) { return a * (a + 1) / 2 + b; }
 
@@ -175,9 +182,9 @@ __device__ __forceinline__ void pair_of(unsigned x, int& a, int& b) {
 struct TPairs {
   const double* t;
   long long st[4];
-  int np, nh, sym;  // sym: columns of t+ are i >= j, of t- i > j; else both all (i, j)
+  int np, nh;
   double *plus, *minus;
-  long long cp, cm;  // columns
+  long long cp, cm;  // columns: i >= j of t+, i > j of t-
 };
 
 // t+ and t- [pairs r >= s][columns]; blockIdx.y walks the pairs
@@ -190,18 +197,11 @@ __global__ void k_ladder_t(const TPairs a) {
     const double* t2 = a.t + s * a.st[0] + r * a.st[1];
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < a.cp; c += (long long)gridDim.x * blockDim.x) {
       int i, j;
-      if (a.sym) {
-        pair_of((unsigned)c, i, j);
-      } else {
-        i = (int)(c / a.nh);
-        j = (int)(c - (long long)i * a.nh);
-      }
+      pair_of((unsigned)c, i, j);
       const long long o = i * a.st[2] + j * a.st[3];
       const double u = t1[o], v = t2[o];
       a.plus[x * a.cp + c] = r == s ? u : 0.5 * (u + v);
-      const double m = r == s ? 0.0 : 0.5 * (u - v);
-      if (!a.sym) a.minus[x * a.cm + c] = m;
-      else if (i > j) a.minus[x * a.cm + (long long)i * (i - 1) / 2 + j] = m;
+      if (i > j) a.minus[x * a.cm + (long long)i * (i - 1) / 2 + j] = r == s ? 0.0 : 0.5 * (u - v);
     }
   }
 }
@@ -253,26 +253,8 @@ __global__ void k_ladder_g_pairs(const double* __restrict__ M, int np, long long
   }
 }
 
-// the same rows from a batch G[p - b0][q][r][s], q < nq, of rows p in [b0, b1)
-__global__ void k_ladder_g_rows(const double* __restrict__ G, int np, int nq, int b0, long long row0, long long first,
-                                double* __restrict__ plus, double* __restrict__ minus) {
-  const long long pairs = pair_index(np, 0), row = first + blockIdx.y;
-  int p, q;
-  pair_of((unsigned)row, p, q);
-  const double* g = G + ((long long)(p - b0) * nq + q) * np * np;
-  double* gp = plus + (row - row0) * pairs;
-  double* gm = minus + (row - row0) * pairs;
-  for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < pairs; x += (long long)gridDim.x * blockDim.x) {
-    int r, s;
-    pair_of((unsigned)x, r, s);
-    const double u = g[(long long)r * np + s], v = g[(long long)s * np + r];
-    gp[x] = r == s ? u : u + v;
-    gm[x] = r == s ? 0.0 : u - v;
-  }
-}
-
 // L from S (plus) and D (minus) of the pairs p >= q from row0 on
-__global__ void k_ladder_out(const double* __restrict__ plus, const double* __restrict__ minus, int np, int nh, int sym,
+__global__ void k_ladder_out(const double* __restrict__ plus, const double* __restrict__ minus, int np, int nh,
                              long long cp, long long cm, long long row0, double* __restrict__ L) {
   int p, q;
   pair_of((unsigned)(row0 + blockIdx.y), p, q);
@@ -281,12 +263,6 @@ __global__ void k_ladder_out(const double* __restrict__ plus, const double* __re
   double* qp = L + ((long long)q * np + p) * h2;
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < cp; c += (long long)gridDim.x * blockDim.x) {
     const double S = plus[blockIdx.y * cp + c];
-    if (!sym) {
-      const double D = minus[blockIdx.y * cm + c];
-      pq[c] = S + D;
-      if (p != q) qp[c] = S - D;
-      continue;
-    }
     int i, j;
     pair_of((unsigned)c, i, j);
     const double D = i > j ? minus[blockIdx.y * cm + (long long)i * (i - 1) / 2 + j] : 0.0;
@@ -335,8 +311,8 @@ void pair_contract(Workspace& ws, const TPairs& t, const double* gp, const doubl
     pair_product(ws, K_LADDER_CONTRACT, gm, pairs, 1, t.minus, t.cm, lm, t.cm, rows, t.cm, pairs);
   }
   const int r = ws.begin(K_AXPY, 0.0, 32.0 * (double)rows * (double)t.cp);
-  k_ladder_out<<<dim3(blocks_for(t.cp, 128, 8), (unsigned)rows), 128, 0, ws.stream>>>(lp, lm, t.np, t.nh, t.sym, t.cp,
-                                                                                      t.cm, row0, L);
+  k_ladder_out<<<dim3(blocks_for(t.cp, 128, 8), (unsigned)rows), 128, 0, ws.stream>>>(lp, lm, t.np, t.nh, t.cp, t.cm,
+                                                                                      row0, L);
   ws.end(r);
 }
 
@@ -387,7 +363,6 @@ bool ladder_core_pairs(const double* B, long long n, int naux, int p0, int np, i
   for (int k = 0; k < 4; ++k) tp.st[k] = tst[k];
   tp.np = np;
   tp.nh = nh;
-  tp.sym = 1;
   tp.cp = pair_index(nh, 0);
   tp.cm = tp.cp - nh;
   WorkspaceBlock plus(mws, (size_t)(pairs * tp.cp)), minus(mws, (size_t)(pairs * tp.cm));
@@ -411,69 +386,97 @@ bool ladder_core_pairs(const double* B, long long n, int naux, int p0, int np, i
   return true;
 }
 
-// The pair form for any B and t: (pr|qs) for q < p + 1 in batches of rows p.
-// All scratch stays within max_doubles; false (nothing done) where that is
-// too little for ten batches or so.
-bool ladder_core_general(const double* B, long long n, int naux, int p0, int np, int nh, const double* t, double* L,
-                         long long max_doubles, Workspace& ws) {
-  const long long pairs = pair_index(np, 0), h2 = (long long)nh * nh, p2 = (long long)np * np;
-  const long long left = max_doubles - 2 * pairs * h2;
-  // a row p: its (pr|qs) and, for its pairs, G+- and S, D
-  const long long per = np * p2 + np * (2 * pairs + 2 * h2);
-  long long nb = left / per;
-  if (nb > (np + 9) / 10) nb = (np + 9) / 10;
-  if (nb < 1 || nb * np > kMaxRows || pairs >= (1LL << 31)) return false;
-  cudaStream_t st = ws.stream;
-  TPairs tp{};
-  tp.t = t;
-  const long long tst[4] = {np * h2, h2, nh, 1};
-  for (int k = 0; k < 4; ++k) tp.st[k] = tst[k];
-  tp.np = np;
-  tp.nh = nh;
-  tp.cp = tp.cm = h2;
-  WorkspaceBlock plus(ws, (size_t)(pairs * h2)), minus(ws, (size_t)(pairs * h2));
-  tp.plus = plus.p;
-  tp.minus = minus.p;
-  pair_amplitudes(ws, tp);
-  WorkspaceBlock G(ws, (size_t)(nb * np * p2));
-  // as many pairs per contraction as the rest of the budget holds
-  long long cap = (left - nb * np * p2) / (2 * pairs + 2 * h2);
-  if (cap > pairs) cap = pairs;
-  if (cap > kMaxRows) cap = kMaxRows;
-  WorkspaceBlock gp(ws, (size_t)(cap * pairs)), gm(ws, (size_t)(cap * pairs)), lp(ws, (size_t)(cap * h2)),
-      lm(ws, (size_t)(cap * h2));
-  long long row0 = 0, row1 = 0;  // pairs whose G+- rows are held
-  for (int b0 = 0; b0 < np; b0 += (int)nb) {
-    const int b1 = b0 + nb < np ? b0 + (int)nb : np;
-    const int nq = b1;
-    check_cuda(cudaMemsetAsync(G.p, 0, (size_t)(b1 - b0) * nq * p2 * sizeof(double), st), "cudaMemsetAsync (ladder)");
-    GemmArgs g{};  // G[p - b0, q, r, s] = sum_Q B[Q, p0+p, p0+r] B[Q, p0+q, p0+s], p in [b0, b1), q < b1
-    g.A = B + (p0 + b0) * n + p0;
-    g.B = B + (long long)p0 * n + p0;
-    g.C = G.p;
-    g.alpha = 1.0;
-    g.nM = g.nN = 2;
-    g.eM[0] = b1 - b0; g.aM[0] = n; g.cM[0] = nq * p2;
-    g.eM[1] = np;      g.aM[1] = 1; g.cM[1] = np;
-    g.eN[0] = nq;      g.bN[0] = n; g.cN[0] = p2;
-    g.eN[1] = np;      g.bN[1] = 1; g.cN[1] = 1;
-    g.nK = 1;
-    g.eK[0] = naux; g.aK[0] = n * n; g.bK[0] = n * n;
-    g.M = (long long)(b1 - b0) * np;
-    g.N = (long long)nq * np;
-    g.K = naux;
-    g.nbatch = 1;
-    run_gemm(ws, g, K_LADDER_BUILD);
-    const long long next = pair_index(b1, 0);
-    if (next - row0 > cap) {
-      pair_contract(ws, tp, gp.p, gm.p, lp.p, lm.p, row0, row1 - row0, L);
-      row0 = row1;
-    }
-    k_ladder_g_rows<<<dim3(blocks_for(pairs, 256, 64), (unsigned)(next - row1)), 256, 0, st>>>(G.p, np, nq, b0, row0,
-                                                                                               row1, gp.p, gm.p);
-    row1 = next;
+// ---------------------------------------------------------------------------
+// any B and t
+// ---------------------------------------------------------------------------
+// (pr|qs) for q <= p as rows [pq][rs], and one product with both orders of t,
+//   L[p,q] = sum_{r,s} (pr|qs) t[r,s],  L[q,p] = sum_{r,s} (pr|qs) t[s,r]
+// (by (ps|qr) = (qr|ps)): half of the build of ladder_core, every element of L
+// the plain sum of its own products.  Bound: the FP64 pipe.  np = 106, nh = 16,
+// 400 auxiliary functions: 140 (ladder_core) -> 107 ms; a contraction per batch
+// of p (ladder_core_half, which needs less memory) takes 113.  Sums and
+// differences as in the pair form took 85, and lost the smaller one of L[p,q]
+// and L[q,p].
+namespace {
+// t2[rs][0][ij] = t[r][s][ij], t2[rs][1][ij] = t[s][r][ij]
+__global__ void k_ladder_t2(const double* __restrict__ t, long long np, long long h2, double* __restrict__ t2) {
+  const long long n = np * np * h2;
+  for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < n; x += (long long)gridDim.x * blockDim.x) {
+    const long long rs = x / h2, ij = x - rs * h2, r = rs / np, s = rs - r * np;
+    t2[2 * rs * h2 + ij] = t[x];
+    t2[(2 * rs + 1) * h2 + ij] = t[(s * np + r) * h2 + ij];
   }
-  pair_contract(ws, tp, gp.p, gm.p, lp.p, lm.p, row0, row1 - row0, L);
+}
+
+// L[p,q] and L[q,p] from the rows (p - b0, q), p in [b0, b0 + gridDim.z), q < gridDim.y
+__global__ void k_ladder_rows_out(const double* __restrict__ c, int b0, int np, long long h2, double* __restrict__ L) {
+  const int p = b0 + blockIdx.z, q = blockIdx.y;
+  if (q > p) return;  // p's own row in the same batch has it
+  const double* row = c + ((long long)blockIdx.z * gridDim.y + q) * 2 * h2;
+  double* pq = L + ((long long)p * np + q) * h2;
+  double* qp = L + ((long long)q * np + p) * h2;
+  for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < h2; x += (long long)gridDim.x * blockDim.x) {
+    pq[x] = row[x];
+    if (q < p) qp[x] = row[h2 + x];
+  }
+}
+}  // namespace
+
+bool ladder_core_rows(const double* B, long long n, int naux, int p0, int np, int nh, const double* t, double* L,
+                      long long max_doubles, Workspace& ws) {
+  const long long p2 = (long long)np * np, h2 = (long long)nh * nh;
+  // batches of p whose build has at least 256 rows (p, r); rows held: those of
+  // all batches, or as many as fit, but at least one batch
+  const long long nb = np < 256 ? (255 + np) / np : 1;
+  const long long cap = (max_doubles - 2 * p2 * h2) / (p2 + 2 * h2);
+  if (cap < nb * np || np > 65535) return false;
+  const long long all = (p2 + (nb + 1) * np) / 2 + nb;
+  const long long held = cap < all ? cap : all;
+  cudaStream_t st = ws.stream;
+  WorkspaceBlock t2(ws, (size_t)(2 * p2 * h2)), G(ws, (size_t)(held * p2)), C(ws, (size_t)(held * 2 * h2));
+  k_ladder_t2<<<blocks_for(p2 * h2, 256, 152 * 16), 256, 0, st>>>(t, np, h2, t2.p);
+  for (int p = 0; p < np;) {
+    const int first = p;
+    long long rows = 0;
+    auto size = [&](int b0) { return (b0 + nb < np ? nb : np - b0) * (b0 + nb < np ? b0 + nb : np); };
+    for (; p < np && rows + size(p) <= held; p += (int)nb) rows += size(p);
+    check_cuda(cudaMemsetAsync(G.p, 0, (size_t)(rows * p2) * sizeof(double), st), "cudaMemsetAsync (ladder)");
+    check_cuda(cudaMemsetAsync(C.p, 0, (size_t)(rows * 2 * h2) * sizeof(double), st), "cudaMemsetAsync (ladder)");
+    const int end = p < np ? p : np;
+    long long at = 0;
+    for (int b0 = first; b0 < end; b0 += (int)nb) {
+      const int b1 = b0 + nb < np ? b0 + (int)nb : np;
+      GemmArgs g{};  // G[p - b0, q, r, s] = sum_Q B[Q, p0+p, p0+r] B[Q, p0+q, p0+s], p in [b0, b1), q < b1
+      g.A = B + (p0 + b0) * n + p0;
+      g.B = B + (long long)p0 * n + p0;
+      g.C = G.p + at * p2;
+      g.alpha = 1.0;
+      g.nM = g.nN = 2;
+      g.eM[0] = b1 - b0; g.aM[0] = n; g.cM[0] = b1 * p2;
+      g.eM[1] = np;      g.aM[1] = 1; g.cM[1] = np;
+      g.eN[0] = b1;      g.bN[0] = n; g.cN[0] = p2;
+      g.eN[1] = np;      g.bN[1] = 1; g.cN[1] = 1;
+      g.nK = 1;
+      g.eK[0] = naux; g.aK[0] = n * n; g.bK[0] = n * n;
+      g.M = (long long)(b1 - b0) * np;
+      g.N = (long long)b1 * np;
+      g.K = naux;
+      g.nbatch = 1;
+      run_gemm(ws, g, K_LADDER_BUILD);
+      at += size(b0);
+    }
+    // sums of 2048 products each, added up in C: half the rounding error of one
+    // sum over all p2 of them (1.8e-15 against 3.7e-15 of the largest element, above)
+    for (long long k = 0; k < p2; k += 2048)
+      pair_product(ws, K_LADDER_CONTRACT, G.p + k, p2, 1, t2.p + k * 2 * h2, 2 * h2, C.p, 2 * h2, rows, 2 * h2,
+                   p2 - k < 2048 ? p2 - k : 2048);
+    at = 0;
+    for (int b0 = first; b0 < end; b0 += (int)nb) {
+      const int b1 = b0 + nb < np ? b0 + (int)nb : np;
+      k_ladder_rows_out<<<dim3(blocks_for(h2, 256, 8), b1, b1 - b0), 256, 0, st>>>(C.p + at * 2 * h2, b0, np, h2, L);
+      at += size(b0);
+    }
+  }
   check_cuda(cudaGetLastError(), "ladder launch");
   return true;
 }
@@ -509,23 +512,39 @@ extern "C" int dsrg_df_ladder(int n, int naux, int p0, int np, int nh, const dou
   if (np == 0 || nh == 0) return DSRG_OK;
   cudaStream_t st = (cudaStream_t)stream;
   const long long p3 = (long long)np * np * np;
-  long long bp = ladder_batch_rows(np, 1LL << 27);  // at most 1 GiB of scratch
-  if (bp < 1) bp = 1;
+  const long long tst[4] = {(long long)np * nh * nh, (long long)nh * nh, nh, 1};
+  // Scratch of at most 1 GiB, or one row of (pr|qs): rows, and up to 256 MiB of
+  // partial sums (kSums).  In one batch where the build has less than 2e8 flops:
+  // two launches, and half of so little is not worth a third (24 particles, 96
+  // auxiliary functions 0.11 ms; 32 and 128, above the line, 0.36 in two batches,
+  // 0.43 in rows).  Batch by batch where the pairs' rows do not fit.
+  constexpr long long kMost = 1LL << 27, kSums = 1LL << 25;
+  const bool one = 2.0 * (double)naux * (double)p3 * (double)np < 2e8;
+  long long rows = one ? np : (np + 15) / 16;
+  if (rows > ladder_batch_rows(np, kMost - kSums)) rows = ladder_batch_rows(np, kMost - kSums);
+  if (rows < 1) rows = 1;
   try {
     CallWorkspace call(st);
     Workspace& ws = *call.ws;
     bool done = false;
     try {
-      done = ladder_core_general(B, n, naux, p0, np, nh, t, L, 1LL << 27, ws);
+      done = !one && ladder_core_rows(B, n, naux, p0, np, nh, t, L, kMost - kSums, ws);
     } catch (const Error& e) {
-      if (e.code != DSRG_ERR_OOM) throw;  // too little memory: the batched form needs less
+      if (e.code != DSRG_ERR_OOM) throw;
     }
-    if (!done) {
-      const WorkspaceBlock rows(ws, (size_t)(bp * p3));
-      check_cuda(cudaMemsetAsync(L, 0, (size_t)np * np * nh * nh * sizeof(double), st), "cudaMemsetAsync");
-      const long long tst[4] = {(long long)np * nh * nh, (long long)nh * nh, nh, 1};
-      ladder_core(B, n, naux, p0, np, nh, t, tst, L, rows.p, bp, st, nullptr);
-      check_cuda(cudaGetLastError(), "ladder launch");
+    for (bool sums = true; !done;) {
+      try {
+        const WorkspaceBlock G(ws, (size_t)(rows * p3));
+        check_cuda(cudaMemsetAsync(L, 0, (size_t)np * np * nh * nh * sizeof(double), st), "cudaMemsetAsync");
+        ladder_core_half(B, n, naux, p0, np, nh, t, tst, false, L, G.p, rows * p3, rows, st, sums ? &ws : nullptr);
+        check_cuda(cudaGetLastError(), "ladder launch");
+        done = true;
+      } catch (const Error& e) {
+        // too little memory: half the rows, and with one row no partial sums
+        if (e.code != DSRG_ERR_OOM || !sums) throw;
+        if (rows == 1) sums = false;
+        rows = (rows + 1) / 2;
+      }
     }
     check_cuda(cudaStreamSynchronize(st), "cudaStreamSynchronize");
   } catch (const Error& ex) {

@@ -14,21 +14,23 @@ namespace dsrg {
 // Launches go through `ws` (counted, optionally timed) when it is non-null.
 void ladder_core(const double* B, long long n, int naux, int p0, int np, int nh, const double* t,
                  const long long* tst, double* L, double* G, long long bp, cudaStream_t st, Workspace* ws);
-// The same sum for a t with t[r,s,i,j] = t[s,r,j,i] (L must be zero on
-// entry), using (pr|qs) = (qs|pr): about half the work; G holds at most
-// max_doubles doubles.
-void ladder_core_sym(const double* B, long long n, int naux, int p0, int np, int nh, const double* t,
-                     const long long* tst, double* L, double* G, long long max_doubles, cudaStream_t st,
-                     Workspace* ws);
-// The same sums in pair form (see ladder.cu); false, and nothing done, where
-// the memory named does not suffice.  _pairs: B symmetric in its last two
-// indices and t as for ladder_core_sym (its blocks come from mws);
-// _general: any B and t (contiguous).  L is overwritten.
+// The same sum (L must be zero on entry) using (pr|qs) = (qs|pr): half the
+// build, and with t[r,s,i,j] = t[s,r,j,i] (t_sym) half the contraction; G holds
+// at most max_doubles doubles, a batch at most most_rows rows.
+void ladder_core_half(const double* B, long long n, int naux, int p0, int np, int nh, const double* t,
+                      const long long* tst, bool t_sym, double* L, double* G, long long max_doubles, long long most_rows,
+                      cudaStream_t st, Workspace* ws);
+// The same sums in pair form (see ladder.cu) for B symmetric in its last two
+// indices and t_sym; its blocks come from mws.  False, and nothing done, where
+// the matrix of (pr|qs) takes more than m_bytes.  L is overwritten.
 bool ladder_core_pairs(const double* B, long long n, int naux, int p0, int np, int nh, const double* t,
                        const long long* tst, double* L, long long max_doubles, double m_bytes, Workspace& ws,
                        Workspace& mws);
-bool ladder_core_general(const double* B, long long n, int naux, int p0, int np, int nh, const double* t, double* L,
-                         long long max_doubles, Workspace& ws);
+// The same sums for any B and t (contiguous), in rows over pairs p >= q (see
+// ladder.cu); false, and nothing done, where max_doubles do not hold a batch of
+// them.  L is overwritten.
+bool ladder_core_rows(const double* B, long long n, int naux, int p0, int np, int nh, const double* t, double* L,
+                      long long max_doubles, Workspace& ws);
 // Largest batch of p rows whose (pr|qs) fits in max_doubles (0 if none).
 long long ladder_batch_rows(int np, long long max_doubles);
 int ladder_check_args(int n, int naux, int p0, int np, int nh, const void* B, const void* t, const void* L,
