@@ -178,10 +178,10 @@ struct OzArgs {
   int S, MT, NT, KT;
   long long M, N;
   double alpha;
-  // alpha = +-2^alpha_exp (its effect is on sign and exponent) unless alpha_mul;
-  // split-k partials carry no alpha
+  // alpha = +-2^alpha_exp (its effect is on sign and exponent) unless alpha_fma
+  // or alpha_zero; split-k partials carry no alpha
   int alpha_exp;
-  bool alpha_neg, alpha_mul;
+  bool alpha_neg, alpha_fma, alpha_zero;
   double* C;
   // C offsets: row m -> decoded with (nM, eM, cM), column n -> (nN, eN, cN)
   int nM, nN;
@@ -608,6 +608,7 @@ __global__ void __launch_bounds__(OZ_CTA_THREADS, 1) k_ozaki_mma(const OzArgs a)
       table_sync();  // this tile's tables are written, the last one's may be overwritten
       if (!ok) continue;
       double* const out = a.splits > 1 ? a.part : a.C;
+      const long long keep = a.alpha_zero ? 0LL : ~0LL;  // alpha = 0 adds zeros
       // element u of a lane in a group of OZ_EPC columns: along the columns of
       // rows 4 u + lane / 8, or along the rows of column u
       auto place = [&](int c0, int u) -> long long {
@@ -665,13 +666,33 @@ __global__ void __launch_bounds__(OZ_CTA_THREADS, 1) k_ozaki_mma(const OzArgs a)
                                                              em + colE[tb][c0 + q], a.alpha_neg);
           }
           __syncwarp();
+          if (a.alpha_fma) {
+            // alpha t + C rounded once, as where alpha is a power of two, by
+            // loads a few elements ahead (61504 x 784 x 64, 7 slices: 687 us, one
+            // by one 1003; a reduction in L2, 485, would round alpha t first)
+            constexpr int AHEAD = 4;
 #pragma unroll
-          for (int u = 0; u < OZ_EPC; ++u) {
-            const long long o = place(c0, u);
-            const double t = sp[u * sstep];
-            if (o >= 0) {
-              if (a.splits > 1) out[o] = t;
-              else red_add(out + o, a.alpha_mul ? a.alpha * t : t);
+            for (int u0 = 0; u0 < OZ_EPC; u0 += AHEAD) {
+              long long o[AHEAD];
+              double c[AHEAD];
+#pragma unroll
+              for (int u = 0; u < AHEAD; ++u) {
+                o[u] = place(c0, u0 + u);
+                c[u] = o[u] >= 0 ? a.C[o[u]] : 0.0;
+              }
+#pragma unroll
+              for (int u = 0; u < AHEAD; ++u)
+                if (o[u] >= 0) a.C[o[u]] = fma(a.alpha, sp[(u0 + u) * sstep], c[u]);
+            }
+          } else {
+#pragma unroll
+            for (int u = 0; u < OZ_EPC; ++u) {
+              const long long o = place(c0, u);
+              const double t = sp[u * sstep];
+              if (o >= 0) {
+                if (a.splits > 1) out[o] = t;
+                else red_add(out + o, __longlong_as_double(__double_as_longlong(t) & keep));
+              }
             }
           }
           __syncwarp();
@@ -1406,7 +1427,8 @@ void ozaki_run(Workspace& ws, const GemmArgs& g0, int S, int kind, const OzChoic
     int e = 0;
     const double f = std::frexp(g0.alpha, &e);  // +-0.5 for a power of two
     const bool pow2 = std::fabs(f) == 0.5 && e > -500 && e < 500;
-    a.alpha_mul = !pow2 && splits <= 1;
+    a.alpha_zero = g0.alpha == 0.0 && splits <= 1;  // the tuner's: timed as the power of two it stands for
+    a.alpha_fma = !pow2 && !a.alpha_zero && splits <= 1;
     a.alpha_exp = pow2 && splits <= 1 ? e - 1 : 0;
     a.alpha_neg = pow2 && splits <= 1 && f < 0.0;
   }
