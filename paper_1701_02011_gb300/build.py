@@ -2,6 +2,7 @@
 from __future__ import annotations
 
 import os
+import re
 import shutil
 import subprocess
 import sys
@@ -24,6 +25,19 @@ def nvcc() -> str:
     raise RuntimeError("nvcc not found")
 
 
+def check_registers(source: str, log: str) -> None:
+    """The split kernel's warpgroups move registers between them (setmaxnreg)
+    within the total that the block is launched with, so every instantiation
+    has to be compiled to exactly the count that the source states."""
+    want = int(re.search(r"constexpr int OZ_REGS = (\d+)", source).group(1))
+    used = re.findall(r"Compiling entry function '(\S*k_ozaki_mma\S*)'.*?Used (\d+) registers", log, re.S)
+    if not used:
+        raise RuntimeError("ptxas reported no registers for k_ozaki_mma")
+    bad = [f"{name}: {n}" for name, n in used if int(n) != want]
+    if bad:
+        raise RuntimeError(f"k_ozaki_mma needs {want} registers a thread, compiled to " + ", ".join(bad))
+
+
 def _newer(target, deps):
     if not os.path.exists(target):
         return False
@@ -43,12 +57,20 @@ def build(force: bool = False, verbose: bool = False, extra_flags=None) -> str:
         o = os.path.join(BUILD, src.replace(".cu", ".o"))
         if not force and _newer(o, [s] + headers):
             return o
-        cmd = [cc] + ARCH + flags + ["-c", s, "-o", o]
+        ptxas = ["-Xptxas", "-v"] if src == "ozaki.cu" else []
+        cmd = [cc] + ARCH + flags + ptxas + ["-c", s, "-o", o]
         if verbose:
             print(" ".join(cmd), flush=True)
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed for {src}:\n{r.stdout}\n{r.stderr}")
+        if ptxas:
+            try:
+                with open(s) as f:
+                    check_registers(f.read(), r.stdout + r.stderr)
+            except RuntimeError:
+                os.remove(o)
+                raise
         if verbose and r.stderr:
             print(r.stderr, file=sys.stderr)
         return o
