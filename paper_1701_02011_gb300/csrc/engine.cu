@@ -163,6 +163,12 @@ void scratch_settle(cudaStream_t st) {
 }
 
 namespace {
+// Revision of the kernels that tuning chooses between, part of a stored
+// decision's key: raised when a change moves which tile or path is the faster
+// one, so that files of earlier kernels are timed anew.  (Revision 1, whose
+// lines carry none: the split kernel with one CTA per tile.)
+constexpr int kTuneRevision = 2;
+
 std::string gpu_key() {
   int dev = 0;
   check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
@@ -172,7 +178,7 @@ std::string gpu_key() {
   for (char& c : name)
     if (c == ' ' || c == '\t') c = '_';
   return name + "/sm" + std::to_string(p.multiProcessorCount) + "/cc" + std::to_string(p.major) +
-         std::to_string(p.minor);
+         std::to_string(p.minor) + "/r" + std::to_string(kTuneRevision);
 }
 
 std::mutex g_tc_mu;

@@ -310,7 +310,8 @@ unsigned long long current_context_id();
 // Persistent record of tuning decisions (file named by DSRG_TUNE_CACHE; no
 // file: decisions live for the process only).  A decision is a few integers
 // stored under (kind, GPU, M, N, K, slices); the GPU is identified by its
-// name, SM count and compute capability.  lookup fills `vals` and returns
+// name, SM count and compute capability, followed by the revision of the
+// kernels (kTuneRevision).  lookup fills `vals` and returns
 // true when the file holds the key; store appends a line.
 bool tune_cache_lookup(const char* kind, long long M, long long N, long long K, int slices, int nvals, int* vals);
 void tune_cache_store(const char* kind, long long M, long long N, long long K, int slices, int nvals,
