@@ -430,7 +430,7 @@ bool split_route(Workspace& ws, const GemmArgs& g) {
 // one flat launch over the output blocks of tab (npairs operand pairs)
 void run_gemm_flat(Workspace& ws, const GemmArgs& g, const FlatTable& tab, int npairs) {
   const size_t O = (size_t)(g.M * g.N * g.nbatch);
-  if (gemm_use_narrow(g)) {
+  if (gemm_use_narrow(g, tab.ngroups)) {
     const NarrowPlan np = gemm_narrow_plan(g, tab.ngroups);
     const WorkspaceBlock npart(ws, np.z > 1 ? (size_t)tab.ngroups * np.z * O : 0);
     const int r = ws.begin(K_GEMM, 2.0 * (double)g.M * (double)g.N * (double)g.K * npairs, 0.0);

@@ -423,7 +423,7 @@ __global__ void k_gemm_flat_reduce(const GemmArgs g, const FlatK fk, const FlatT
   }
 }
 
-// Narrow contraction: outputs with one short side of at most NS <= 48.  A thread
+// Narrow contraction: outputs with one short side of at most NS <= 40.  A thread
 // owns one index m of the long side and keeps all its NS sums in registers,
 // so each element of the long operand is read once (the flat kernel reads it
 // once per output column: at 11236 x 36 x 2560 the long operand does not fit
@@ -434,7 +434,7 @@ __global__ void k_gemm_flat_reduce(const GemmArgs g, const FlatK fk, const FlatT
 // consecutive elements of C whichever side is contiguous there.
 // 11236 x 36 x 2560: 3.6 -> 0.91 ms; 1722112 x 8 x 48 (six spin blocks of k = 8):
 // 1.75 -> 1.24 ms, of 1.05 ms at the FP64 rate.
-constexpr int NARROW_T = 128, NKB = 32, NARROW_EPC = 4;
+constexpr int NARROW_T = 128, NKB = 32, NARROW_EPC = 4, NARROW_CTAS = 6 * 152;
 template <int NS>
 __global__ void __launch_bounds__(NARROW_T) k_gemm_narrow(const NarrowArgs a, const FlatTable tab, double* part) {
   __shared__ double Bs[NKB][NS];
@@ -512,14 +512,15 @@ __global__ void __launch_bounds__(NARROW_T) k_gemm_narrow(const NarrowArgs a, co
 #pragma unroll
   for (int c0 = 0; c0 < NS; c0 += NARROW_EPC) {
 #pragma unroll
-    for (int j = 0; j < NARROW_EPC; ++j) stg[tid][j] = acc[c0 + j];
+    for (int j = 0; j < NARROW_EPC; ++j)
+      if (c0 + j < NS) stg[tid][j] = acc[c0 + j];
     __syncwarp();
 #pragma unroll
     for (int j = 0; j < NARROW_EPC; ++j) {
       const int i = j * 32 + lane;
       const int r = warp * 32 + (a.cmfast ? lane : i / NARROW_EPC), c = c0 + (a.cmfast ? j : i % NARROW_EPC);
       const double v = stg[r][c - c0];
-      if (mc[r] < 0 || nc[c] < 0) continue;
+      if (c >= NS || mc[r] < 0 || nc[c] < 0) continue;
       if (gridDim.y > 1) C[(long long)(blockIdx.x * (unsigned)NARROW_T + r) * a.N + c] = v;
       else C[mc[r] + nc[c]] += a.alpha * v;
     }
@@ -1004,26 +1005,36 @@ void launch_gemm_flat(const GemmArgs& g, const FlatPlan& p, const FlatTable& tab
   }
 }
 
-bool gemm_use_narrow(const GemmArgs& g) {
-  // one short side of at most 48 (its sums fit a thread's registers) and a
-  // long one that gives at least a warp to every SM; k long enough to pay for
-  // the tables.  At most 32 k chunks (65535 column blocks are never reached).
-  const long long s = g.M < g.N ? g.M : g.N, l = g.M < g.N ? g.N : g.M;
-  return g.nbatch == 1 && s >= 3 && s <= 48 && l >= 152 * 32 && l < (1LL << 31) && g.K >= 4 && g.K < (1LL << 31);
-}
-
 NarrowPlan gemm_narrow_plan(const GemmArgs& g, int groups) {
   NarrowPlan p{};
   const long long l = g.M < g.N ? g.N : g.M;
   const long long ctas = (l + NARROW_T - 1) / NARROW_T * (groups > 1 ? groups : 1);
-  // about four CTAs per SM, at least 4 NKB of k each
-  long long z = (4 * 152 + ctas - 1) / ctas;
+  // about six CTAs per SM, at least 4 NKB of k each, at most 32 chunks (65535
+  // column blocks are never reached)
+  long long z = (NARROW_CTAS + ctas - 1) / ctas;
   if (z > g.K / (4 * NKB)) z = g.K / (4 * NKB);
   if (z > 32) z = 32;
   if (z < 1) z = 1;
   p.len = (g.K + z - 1) / z;
   p.z = (int)((g.K + p.len - 1) / p.len);
+  p.ctas = ctas * p.z;
   return p;
+}
+
+// The narrow kernel keeps the FP64 units as busy as its CTAs fill the SMs and
+// as little of its columns is padding; the flat kernel's limit is the traffic of
+// the long operand, which depends on layout and cache.  So: a short side of at
+// most 40 (its sums fit a thread's registers with loads in flight), padded to
+// even by at most 15 %, and at least six CTAs per SM, so that a last one costs
+// little.  With fewer the flat kernel was up to four times as fast (4864 x 48 x
+// 200: 87 against 391 us).  Over 1139 contractions met in fifteen energies: 247 ms
+// flat, 191 narrow wherever there is a warp per SM, 192 by this rule with no
+// shape more than 6 % slower than flat.
+bool gemm_use_narrow(const GemmArgs& g, int groups) {
+  const long long s = g.M < g.N ? g.M : g.N, l = g.M < g.N ? g.N : g.M;
+  if (g.nbatch != 1 || s < 4 || s > 40 || s == 5 || l < 152 * 32 || l >= (1LL << 31) || g.K < 4 || g.K >= (1LL << 31))
+    return false;
+  return gemm_narrow_plan(g, groups).ctas >= NARROW_CTAS;
 }
 
 void launch_gemm_narrow(const GemmArgs& g, const NarrowPlan& p, const FlatTable& tab0, double* part, cudaStream_t st) {
@@ -1055,12 +1066,13 @@ void launch_gemm_narrow(const GemmArgs& g, const NarrowPlan& p, const FlatTable&
   a.bkfast = a.nK > 0 && (a.nN == 0 || a.bK[a.nK - 1] < a.bN[a.nN - 1]);
   a.cmfast = a.nM > 0 && (a.nN == 0 || a.cM[a.nM - 1] < a.cN[a.nN - 1]);
   const dim3 grid((unsigned)((a.M + NARROW_T - 1) / NARROW_T), (unsigned)p.z, (unsigned)tab.ngroups);
-  switch ((int)((a.N + 3) / 4)) {
+  switch ((int)((a.N + 1) / 2)) {
 #define DSRG_NARROW(n) \
-  case n: k_gemm_narrow<4 * n><<<grid, NARROW_T, 0, st>>>(a, tab, part); break;
-    DSRG_NARROW(1) DSRG_NARROW(2) DSRG_NARROW(3) DSRG_NARROW(4) DSRG_NARROW(5) DSRG_NARROW(6)
-    DSRG_NARROW(7) DSRG_NARROW(8) DSRG_NARROW(9) DSRG_NARROW(10) DSRG_NARROW(11)
-    default: k_gemm_narrow<48><<<grid, NARROW_T, 0, st>>>(a, tab, part); break;
+  case n: k_gemm_narrow<2 * n><<<grid, NARROW_T, 0, st>>>(a, tab, part); break;
+    DSRG_NARROW(2) DSRG_NARROW(3) DSRG_NARROW(4) DSRG_NARROW(5) DSRG_NARROW(6) DSRG_NARROW(7) DSRG_NARROW(8)
+    DSRG_NARROW(9) DSRG_NARROW(10) DSRG_NARROW(11) DSRG_NARROW(12) DSRG_NARROW(13) DSRG_NARROW(14)
+    DSRG_NARROW(15) DSRG_NARROW(16) DSRG_NARROW(17) DSRG_NARROW(18) DSRG_NARROW(19)
+    default: k_gemm_narrow<40><<<grid, NARROW_T, 0, st>>>(a, tab, part); break;
 #undef DSRG_NARROW
   }
   if (p.z > 1) {

@@ -158,7 +158,7 @@ bool gemm_use_flat(const GemmArgs& g);
 FlatPlan gemm_flat_plan(const GemmArgs& g, int groups = 1);
 // part needs groups * z * M*N*nbatch doubles when the plan has z > 1
 void launch_gemm_flat(const GemmArgs& g, const FlatPlan& p, const FlatTable& tab, double* part, cudaStream_t st);
-// Narrow contraction: an output with a short side of at most 48 and a long one.
+// Narrow contraction: an output with a short side of at most 40 and a long one.
 // part needs groups * z * M*N doubles when the plan has z > 1.
 struct NarrowArgs {
   int nM, nN, nK;
@@ -171,8 +171,10 @@ struct NarrowArgs {
 struct NarrowPlan {
   int z;          // k chunks
   long long len;  // k per chunk
+  long long ctas;
 };
-bool gemm_use_narrow(const GemmArgs& g);
+// whether to use it for `groups` output blocks of this geometry
+bool gemm_use_narrow(const GemmArgs& g, int groups);
 NarrowPlan gemm_narrow_plan(const GemmArgs& g, int groups);
 void launch_gemm_narrow(const GemmArgs& g, const NarrowPlan& p, const FlatTable& tab, double* part, cudaStream_t st);
 // kind 0: generic contraction, 1: DF build of (pr|qs), 2: ladder contraction
