@@ -19,13 +19,6 @@
 namespace {
 
 constexpr int CH_MAX_CTAS = 152 * 4;
-// Threads per CTA.  Every correction is one rounded product and one rounded
-// sum, and an SM retires two FP64 operations a clock, so a step lasts as long
-// as the SM with the most rows: up to N = 152 x 96 each SM gets one CTA of 96
-// rows (with 256 threads at N = 13456 the factorisation used 53 of the 152
-// SMs, 40 us a vector on average; now 24 us, 22 us with chained launches).
-// Larger N fill the chip with 256.
-constexpr long long CH_SMALL_N = 152LL * 96;
 constexpr int CH_Q = 512;  // earlier vectors whose pivot entries are held at a time
 
 struct ChState {
@@ -200,6 +193,57 @@ inline int ch_grid(long long N, int threads) {
   return (int)g;
 }
 
+// f with the CTA size as a constant
+template <class F>
+void ch_dispatch(int threads, F&& f) {
+  switch (threads) {
+    case 96: f(std::integral_constant<int, 96>{}); break;
+    case 128: f(std::integral_constant<int, 128>{}); break;
+    case 160: f(std::integral_constant<int, 160>{}); break;
+    case 192: f(std::integral_constant<int, 192>{}); break;
+    case 224: f(std::integral_constant<int, 224>{}); break;
+    default: f(std::integral_constant<int, 256>{}); break;
+  }
+}
+
+// How a size is launched.  Every correction is one rounded product and one
+// rounded sum, and an SM retires two FP64 operations a clock, so a step lasts as
+// long as the SM with the most rows: of the CTA sizes whose CTAs are all
+// resident, the one that gives the fullest SM the fewest.  The launches are chained
+// unless the next step's CTAs, which take their places while this one's still
+// hold theirs, would not all find one: those that come later pile up on a few
+// SMs.  Microseconds a vector, 200 vectors (100 and 60 at the ends):
+//   N = 14592 13.4 (152 CTAs of 96; 57 of 256 took 20.6), 20000 20.3 (125 of 160;
+//   chained 256: 25.2), 38900 25.5 (304 of 128), 39000 30.0 (407 of 96, plain;
+//   chained 39.8, 153 of 256 chained 41.4), 60000 38.4 (268 of 224), 100000 29.1
+//   (1042 of 96, plain; 391 of 256 38.0).
+struct ChPlan {
+  int threads, grid;
+  bool chained;
+};
+ChPlan ch_plan(long long N) {
+  ChPlan best{96, ch_grid(N, 96), false};  // where no size has all its CTAs resident (N > 77824)
+  long long least = -1;
+  for (int t = 256; t >= 96; t -= 32) {
+    int fit = 1;  // CTAs resident on an SM
+    ch_dispatch(t, [&](auto c) {
+      constexpr int T = decltype(c)::value;
+      static const int n = [] {
+        int v = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_chol_step<T>, T, 0) != cudaSuccess) cudaGetLastError();
+        return v < 1 ? 1 : v;
+      }();
+      fit = n;
+    });
+    const long long ctas = (N + t - 1) / t, wave = 152LL * fit;
+    const long long rows = (ctas + 151) / 152 * t;
+    if (ctas > wave || (least >= 0 && rows > least)) continue;
+    least = rows;
+    best = ChPlan{t, ch_grid(N, t), fit <= 2 || 2 * ctas <= wave};
+  }
+  return best;
+}
+
 }  // namespace
 
 extern "C" int dsrg_cholesky(long long N, const double* V, double tau, int max_vecs, double* B, int* nvecs,
@@ -211,8 +255,8 @@ extern "C" int dsrg_cholesky(long long N, const double* V, double tau, int max_v
   if (!V || !B) return set_error(DSRG_ERR_ARG, "cholesky: V and B must be device pointers");
   if (N > (1LL << 40) / N) return set_error(DSRG_ERR_ARG, "cholesky: N too large");
   cudaStream_t st = (cudaStream_t)stream;
-  const bool small = N <= CH_SMALL_N;
-  const int grid = ch_grid(N, small ? 96 : 256);
+  const ChPlan plan = ch_plan(N);
+  const int threads = plan.threads, grid = plan.grid;
   // scratch: D [N], per-CTA maxima, pivots [max_vecs], state
   const size_t bytes = (size_t)N * 8 + (size_t)grid * 16 + (size_t)max_vecs * 8 + sizeof(ChState) + 64;
   try {
@@ -225,13 +269,21 @@ extern "C" int dsrg_cholesky(long long N, const double* V, double tau, int max_v
     long long* piv = pi + grid;
     ChState* cs = reinterpret_cast<ChState*>(piv + max_vecs);
     check_cuda(cudaMemsetAsync(cs, 0, sizeof(ChState), st), "cudaMemsetAsync (cholesky)");
-    (small ? k_chol_init<96> : k_chol_init<256>)<<<grid, small ? 96 : 256, 0, st>>>(V, N, D, pv, pi, cs, tau, max_vecs, piv);
+    void (*step)(const double*, long long, double*, double*, double*, long long*, ChState*, double, int, long long*) = nullptr;
+    ch_dispatch(threads, [&](auto t) {
+      constexpr int T = decltype(t)::value;
+      k_chol_init<T><<<grid, T, 0, st>>>(V, N, D, pv, pi, cs, tau, max_vecs, piv);
+      step = k_chol_step<T>;
+    });
     check_cuda(cudaGetLastError(), "cholesky launch");
     ChState h{};
     for (int q = 0; q < max_vecs; ++q) {
-      check_cuda(launch_chained(small ? k_chol_step<96> : k_chol_step<256>, grid, small ? 96 : 256, st, V, N, B, D, pv, pi,
-                                cs, tau, max_vecs, piv),
-                 "cholesky launch");
+      if (plan.chained) {
+        check_cuda(launch_chained(step, grid, threads, st, V, N, B, D, pv, pi, cs, tau, max_vecs, piv), "cholesky launch");
+      } else {
+        step<<<grid, threads, 0, st>>>(V, N, B, D, pv, pi, cs, tau, max_vecs, piv);
+        check_cuda(cudaGetLastError(), "cholesky launch");
+      }
       // every 32 vectors: stop launching once the factorisation has stopped
       if ((q & 31) == 31 || q == max_vecs - 1) {
         check_cuda(cudaMemcpyAsync(&h, cs, sizeof h, cudaMemcpyDeviceToHost, st), "cudaMemcpyAsync (cholesky)");
