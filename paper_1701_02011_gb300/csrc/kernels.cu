@@ -676,11 +676,12 @@ __device__ __forceinline__ void dot_tree(double* sh_s, double* sh_c) {
 }
 
 // The terms go into a running sum s and a correction c with four FP64
-// operations a term: with t = fma(a, b, s), fma(a, b, s - t) is what the sum
-// and the product lost, exactly where |s| >= |a b| and to a rounding of t
-// elsewhere (a plain product would lose as much on every term).  The FP64
-// pipe bounds this kernel (two operations a clock and SM), not memory; with
-// a rounded product and Neumaier's branch it took six.
+// operations a term: with t = fma(a, b, s), c collects fma(a, b, s - t), what the
+// sum and the product lost.  That is exact where s - t is (a double for most
+// terms smaller than s); where a term exceeds s or cancels most of it, s - t
+// is rounded, by at most 2^-53 |a b|, which is what a rounded product loses on
+// every term.  The FP64 pipe bounds this kernel (two operations a clock and SM),
+// not memory; with a rounded product and Neumaier's branch it took six.
 template <bool FAST, int V>
 __global__ void __launch_bounds__(DOT_THREADS) k_dot_blocks(const NdArgs g, const DotBlocks p, double* partial,
                                                            unsigned* ticket, double alpha, double* out) {

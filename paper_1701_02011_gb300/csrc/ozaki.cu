@@ -28,7 +28,11 @@ constexpr int OZ_GROUP = 8;
 constexpr int OZ_THREADS = 256;  // 8 warps: lane quadrant (warp % 4) x column half (warp / 4)
 constexpr int OZ_CTA_THREADS = OZ_THREADS + 128;  // and a warpgroup with one warp for the bulk copies and one for the MMAs
 // registers per thread: the block is launched with 384 x 168 (a quarter of
-// them on each sub-partition) and the warpgroups take 208 + 208 + 88 = 3 x 168
+// them on each sub-partition) and the warpgroups take 208 + 208 + 88 = 3 x 168.
+// The build checks that every instantiation has 168.  Where a summing thread
+// holds 64-bit sums for 32 columns the compiler still spills a little: 40 to 72
+// bytes at 6 to 8 slices with 64 columns, 24 at 3 and 8 at 5; with 32 columns
+// 28 at 8; none elsewhere.
 constexpr int OZ_REGS = 168, OZ_REGS_SUM = 208, OZ_REGS_ISSUE = 88;
 static_assert(2 * OZ_REGS_SUM + OZ_REGS_ISSUE == 3 * OZ_REGS, "register split");
 constexpr int OZ_TILE_ELEMS = OZ_BM * OZ_BK;  // A stage tile of one slice: 2048 bf16 = 4 KiB
@@ -210,10 +214,10 @@ __device__ __forceinline__ long long c_offset(long long lin, int nd, const int* 
   return o;
 }
 
-// barrier 1 over the 8 warps of the tile; whether every thread's pred was true
 // barrier 2: the tile's warps and the two that write its tables.  Every one
 // of them passes it once per tile, whatever happened before.
 __device__ __forceinline__ void table_sync() { asm volatile("bar.sync 2, %0;" ::"n"(OZ_THREADS + 64) : "memory"); }
+// barrier 1 over the 8 warps of the tile; whether every thread's pred was true
 __device__ __forceinline__ bool tile_sync_and(bool pred) {
   uint32_t r;
   asm volatile(
@@ -1080,7 +1084,7 @@ __global__ void __launch_bounds__(PACK_T) k_ozaki_digits(const PackPass pp) {
 // lanes, each group loaded once), or where the rows are the contiguous
 // direction and many, one thread per row, which reads it twice.  The window
 // rule gets the bound that holds for any digits (one window, and the quick
-// sums for k up to 128 at 8 slices).  Every padded row is written, so nothing
+// sums for k up to 112 at 8 slices).  Every padded row is written, so nothing
 // is cleared beforehand: one launch in place of three.
 constexpr int PACK_SHORT = 256, PACK_ROWS = 4096;
 template <int S>
