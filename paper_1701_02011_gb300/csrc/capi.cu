@@ -188,11 +188,10 @@ int dsrg_init(const dsrg_inputs* in, const dsrg_options* opts, dsrg_handle** out
     if (h->na > 0)
       for (int k = 0; k < 9; ++k) h->blk[k] = h->own(pow_na(h->na, rank[k]));
     h->ws.cap_results = 1 << 16;
-    dsrg::check_cuda(cudaMalloc(&h->ws.results, h->ws.cap_results * sizeof(double)), "cudaMalloc (results)");
+    h->ws.results = (double*)dsrg::device_alloc(h->ws.cap_results * sizeof(double), "cudaMalloc (results)");
     h->ws.dot_scratch_len = 2 * 152 * 16;
     // dot partials, then the dot's ticket and the split kernels' status flag
-    dsrg::check_cuda(cudaMalloc(&h->ws.dot_scratch, (h->ws.dot_scratch_len + 4) * sizeof(double)),
-                     "cudaMalloc (scratch)");
+    h->ws.dot_scratch = (double*)dsrg::device_alloc((h->ws.dot_scratch_len + 4) * sizeof(double), "cudaMalloc (scratch)");
     h->ws.dot_ticket = reinterpret_cast<unsigned*>(h->ws.dot_scratch + h->ws.dot_scratch_len);
     h->ws.oz_status = reinterpret_cast<int*>(h->ws.dot_scratch + h->ws.dot_scratch_len + 2);
     dsrg::check_cuda(cudaMemsetAsync(h->ws.dot_ticket, 0, 4 * sizeof(double), st), "cudaMemsetAsync (ticket)");

@@ -74,6 +74,11 @@ cudaMemPool_t g_pool[64] = {};
 unsigned long long g_pool_ctx[64] = {};
 constexpr unsigned long long kPoolKeep = 1ULL << 30;  // bytes kept between calls
 std::multiset<unsigned long long> g_claims[64];
+// ends of the latest small calls of a device (CallWorkspace), on whatever
+// streams; one is reused after this many calls
+constexpr int kMarks = 16;
+cudaEvent_t g_marks[64][kMarks] = {};
+unsigned g_mark[64] = {};
 
 // bytes the pool of device dev keeps; g_pool_mu is held
 unsigned long long pool_keep(int dev) { return kPoolKeep + (g_claims[dev].empty() ? 0 : *g_claims[dev].rbegin()); }
@@ -88,8 +93,14 @@ cudaMemPool_t live_pool() {
 
 // gives the memory that the current device's pool keeps back to the driver
 void scratch_trim() {
+  int dev = 0;
   std::lock_guard<std::mutex> lock(g_pool_mu);
-  if (cudaMemPool_t pool = live_pool()) cudaMemPoolTrimTo(pool, 0);
+  if (cudaMemPool_t pool = live_pool()) {
+    cudaGetDevice(&dev);
+    for (cudaEvent_t e : g_marks[dev])
+      if (e) cudaEventSynchronize(e);
+    cudaMemPoolTrimTo(pool, 0);
+  }
   cudaGetLastError();
 }
 }  // namespace
@@ -118,6 +129,7 @@ cudaMemPool_t scratch_pool() {
   if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) cudaGetLastError();
   g_pool[dev] = pool;
   g_pool_ctx[dev] = ctx;
+  for (cudaEvent_t& e : g_marks[dev]) e = nullptr;  // those of an earlier context died with it
   return pool;
 }
 
@@ -150,16 +162,28 @@ void ScratchClaim::drop() {
   bytes_ = 0;
 }
 
-void scratch_settle(cudaStream_t st) {
-  unsigned long long held = 0, keep = kPoolKeep;
-  {
-    std::lock_guard<std::mutex> lock(g_pool_mu);
-    if (cudaMemPool_t pool = live_pool()) {
-      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held);
-      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-    }
+CallWorkspace::~CallWorkspace() {
+  const bool small = ws->peak_bytes() < ((size_t)8 << 20);
+  ws.reset();
+  if (!small) {
+    cudaStreamSynchronize(st);
+    return;
   }
-  if (held > keep) cudaStreamSynchronize(st);
+  int dev = 0;
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  if (!live_pool() || cudaGetDevice(&dev) != cudaSuccess) return;
+  cudaEvent_t& e = g_marks[dev][g_mark[dev]++ % kMarks];
+  if ((!e && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) || cudaEventRecord(e, st) != cudaSuccess)
+    cudaGetLastError();
+}
+
+void* device_alloc(size_t bytes, const char* what) {
+  void* p = nullptr;
+  if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+  cudaGetLastError();
+  scratch_trim();
+  check_cuda(cudaMalloc(&p, bytes), what);
+  return p;
 }
 
 namespace {
@@ -610,7 +634,7 @@ double* Workspace::get(size_t n, size_t& cap) {
         for (auto& b : free_) release(b.p);
         free_.clear();
         ++generation;
-        cudaStreamSynchronize(stream);  // until then the pool may count what was freed as in use
+        cudaStreamSynchronize(stream);  // until then the pool counts what was freed as in use
       }
       scratch_trim();
       check_cuda(allocate(&p, n), "cudaMalloc");

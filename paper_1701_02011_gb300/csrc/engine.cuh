@@ -263,7 +263,7 @@ void check_cuda(cudaError_t e, const char* what);
 // that own no handle.  Such a call allocates, runs and synchronises, so with
 // cudaMalloc and cudaFree a small product spent 300 of 380 us on its scratch.
 // The pool keeps at most 1 GiB between calls (what is above that goes back at
-// the first synchronisation after the frees: scratch_settle) and gives that back
+// the first synchronisation after the frees: CallWorkspace) and gives that back
 // when an allocation of this library fails; the driver orders reuse across
 // streams and threads.  nullptr (plain cudaMalloc) where no pool can be had.
 cudaMemPool_t scratch_pool();
@@ -284,23 +284,21 @@ class ScratchClaim {
   int dev_ = -1;
   unsigned long long bytes_ = 0;
 };
-// One more synchronisation of st if the pool holds more than it keeps.
-void scratch_settle(cudaStream_t st);
-// Workspace of a call without a handle, on that pool.  Calls that took less
-// than 8 MiB do not ask what the pool holds (128 of them at once stay within
-// what it keeps; the synchronisation would take 3 of a small product's 70 us).
+// Workspace of a call without a handle, on that pool.  The pool can only give
+// back what the host has seen to be free, so a call ends with a synchronisation
+// after its frees (which also brings the pool down to what it keeps), or, below
+// 8 MiB, with an event that is waited for when the memory is wanted: the
+// synchronisation would take 3 of a small product's 70 us.
 struct CallWorkspace {
   const cudaStream_t st;
   std::optional<Workspace> ws;
   explicit CallWorkspace(cudaStream_t s) : st(s) { ws.emplace(s, scratch_pool()); }
-  ~CallWorkspace() {
-    const bool ask = ws->peak_bytes() >= ((size_t)8 << 20);
-    ws.reset();
-    if (ask) scratch_settle(st);
-  }
+  ~CallWorkspace();
   CallWorkspace(const CallWorkspace&) = delete;
   CallWorkspace& operator=(const CallWorkspace&) = delete;
 };
+// cudaMalloc that has the pool give back what it keeps before it fails
+void* device_alloc(size_t bytes, const char* what);
 // bytes of the current device's memory, asked once per device: the runtime
 // takes 0.3 to 0.5 ms to list a device's properties
 double device_memory();

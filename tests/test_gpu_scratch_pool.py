@@ -64,3 +64,29 @@ def test_out_of_memory_gives_back_what_was_taken(lib):
     finally:
         del fill
         torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("small_call_after", [False, True])
+def test_a_handle_gets_what_the_pool_keeps(lib, small_call_after):
+    """0.5 GB of scratch per operand stay in the pool, 0.2 GB are free, and a
+    handle's inputs take 0.42 GB; nothing synchronises in between."""
+    import numpy as np
+    import synth
+    import torch
+    inst = synth.make_instance(1, 2, 2, 717, 4, 0.5, seed=1)
+    inst["naux"], inst["B"] = 100, np.zeros((100, 720, 720))
+    dev = {k: torch.from_numpy(np.ascontiguousarray(v)).cuda() if isinstance(v, np.ndarray) else v for k, v in inst.items()}
+    n = 5600
+    A = torch.ones((1, n), dtype=torch.float64, device="cuda").expand(n, n)
+    C = torch.zeros((n, n), dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    lib.dsrg_split_gemm(A, A, C, 1.0, 8)
+    if small_call_after:
+        lib.dsrg_split_gemm(A[:64, :64], A[:64, :64], C[:64, :64], 1.0, 6)
+    fill = torch.empty(_free(torch) - (200 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        lib.Dsrg(dev).close()
+    finally:
+        del fill
+        torch.cuda.empty_cache()
