@@ -393,7 +393,7 @@ bool ladder_core_pairs(const double* B, long long n, int naux, int p0, int np, i
 //   L[p,q] = sum_{r,s} (pr|qs) t[r,s],  L[q,p] = sum_{r,s} (pr|qs) t[s,r]
 // (by (ps|qr) = (qr|ps)): half of the build of ladder_core, every element of L
 // the plain sum of its own products.  Bound: the FP64 pipe.  np = 106, nh = 16,
-// 400 auxiliary functions: 140 (ladder_core) -> 107 ms; a contraction per batch
+// 400 auxiliary functions: 140 (ladder_core) -> 103 ms; a contraction per batch
 // of p (ladder_core_half, which needs less memory) takes 113.  Sums and
 // differences as in the pair form took 85, and lost the smaller one of L[p,q]
 // and L[q,p].
@@ -419,6 +419,43 @@ __global__ void k_ladder_rows_out(const double* __restrict__ c, int b0, int np, 
     pq[x] = row[x];
     if (q < p) qp[x] = row[h2 + x];
   }
+}
+
+// C [M][N] = A [M][K] B [K][N] in sums of at most 1024 products each, as partial
+// tiles of one launch within kSums doubles: a third of the rounding error of one
+// sum over all K, and with 2400 tiles or more (of 128 products at least) hardly
+// a part-filled last wave.
+constexpr long long kSums = 1LL << 25;
+void rows_contract(Workspace& ws, const double* A, const double* B, double* C, long long M, long long N, long long K) {
+  int bm, bn;
+  gemm_tile(M, N, 2, &bm, &bn);
+  const long long tiles = ((M + bm - 1) / bm) * ((N + bn - 1) / bn);
+  long long z = (2400 + tiles - 1) / tiles;
+  if (z > K / 128) z = K / 128;
+  if (z < (K + 1023) / 1024) z = (K + 1023) / 1024;
+  if (z > kSums / (M * N)) z = kSums / (M * N);
+  if (z < 2) {
+    pair_product(ws, K_LADDER_CONTRACT, A, K, 1, B, N, C, N, M, N, K);
+    return;
+  }
+  GemmArgs g{};
+  g.A = A;
+  g.B = B;
+  g.C = C;
+  g.alpha = 1.0;
+  g.nM = g.nN = g.nK = 1;
+  g.eM[0] = (int)M; g.aM[0] = K; g.cM[0] = N;
+  g.eN[0] = (int)N; g.bN[0] = 1; g.cN[0] = 1;
+  g.eK[0] = (int)K; g.aK[0] = 1; g.bK[0] = N;
+  g.M = M;
+  g.N = N;
+  g.K = K;
+  g.nbatch = 1;
+  g.kper = ((K + z - 1) / z + 15) / 16 * 16;
+  g.splits = (int)((K + g.kper - 1) / g.kper);
+  const WorkspaceBlock part(ws, (size_t)(g.splits * M * N));
+  g.part = part.p;
+  launch_gemm(g, ws.stream, 2);
 }
 }  // namespace
 
@@ -465,11 +502,7 @@ bool ladder_core_rows(const double* B, long long n, int naux, int p0, int np, in
       run_gemm(ws, g, K_LADDER_BUILD);
       at += size(b0);
     }
-    // sums of 2048 products each, added up in C: half the rounding error of one
-    // sum over all p2 of them (1.8e-15 against 3.7e-15 of the largest element, above)
-    for (long long k = 0; k < p2; k += 2048)
-      pair_product(ws, K_LADDER_CONTRACT, G.p + k, p2, 1, t2.p + k * 2 * h2, 2 * h2, C.p, 2 * h2, rows, 2 * h2,
-                   p2 - k < 2048 ? p2 - k : 2048);
+    rows_contract(ws, G.p, t2.p, C.p, rows, 2 * h2, p2);
     at = 0;
     for (int b0 = first; b0 < end; b0 += (int)nb) {
       const int b1 = b0 + nb < np ? b0 + (int)nb : np;
@@ -518,7 +551,7 @@ extern "C" int dsrg_df_ladder(int n, int naux, int p0, int np, int nh, const dou
   // two launches, and half of so little is not worth a third (24 particles, 96
   // auxiliary functions 0.11 ms; 32 and 128, above the line, 0.36 in two batches,
   // 0.43 in rows).  Batch by batch where the pairs' rows do not fit.
-  constexpr long long kMost = 1LL << 27, kSums = 1LL << 25;
+  constexpr long long kMost = 1LL << 27;
   const bool one = 2.0 * (double)naux * (double)p3 * (double)np < 2e8;
   long long rows = one ? np : (np + 15) / 16;
   if (rows > ladder_batch_rows(np, kMost - kSums)) rows = ladder_batch_rows(np, kMost - kSums);
