@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <array>
+#include <atomic>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -79,6 +80,9 @@ std::multiset<unsigned long long> g_claims[64];
 constexpr int kMarks = 16;
 cudaEvent_t g_marks[64][kMarks] = {};
 unsigned g_mark[64] = {};
+// whether blocks of 8 MiB or more have been in a device's pool since it was
+// last emptied
+std::atomic<bool> g_large[64] = {};
 
 // bytes the pool of device dev keeps; g_pool_mu is held
 unsigned long long pool_keep(int dev) { return kPoolKeep + (g_claims[dev].empty() ? 0 : *g_claims[dev].rbegin()); }
@@ -99,6 +103,7 @@ void scratch_trim() {
     cudaGetDevice(&dev);
     for (cudaEvent_t e : g_marks[dev])
       if (e) cudaEventSynchronize(e);
+    g_large[dev] = false;
     cudaMemPoolTrimTo(pool, 0);
   }
   cudaGetLastError();
@@ -135,7 +140,9 @@ cudaMemPool_t scratch_pool() {
 
 void ScratchClaim::raise(unsigned long long bytes) {
   int dev = 0;
-  if (bytes <= bytes_ || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
+  g_large[dev] = true;
+  if (bytes <= bytes_) return;
   drop();
   std::lock_guard<std::mutex> lock(g_pool_mu);
   g_claims[dev].insert(bytes);
@@ -165,13 +172,16 @@ void ScratchClaim::drop() {
 CallWorkspace::~CallWorkspace() {
   const bool small = ws->peak_bytes() < ((size_t)8 << 20);
   ws.reset();
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
   if (!small) {
+    g_large[dev] = true;
     cudaStreamSynchronize(st);
     return;
   }
-  int dev = 0;
+  if (!g_large[dev]) return;
   std::lock_guard<std::mutex> lock(g_pool_mu);
-  if (!live_pool() || cudaGetDevice(&dev) != cudaSuccess) return;
+  if (!live_pool()) return;
   cudaEvent_t& e = g_marks[dev][g_mark[dev]++ % kMarks];
   if ((!e && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) || cudaEventRecord(e, st) != cudaSuccess)
     cudaGetLastError();

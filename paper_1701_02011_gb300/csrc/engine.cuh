@@ -287,8 +287,9 @@ class ScratchClaim {
 // Workspace of a call without a handle, on that pool.  The pool can only give
 // back what the host has seen to be free, so a call ends with a synchronisation
 // after its frees (which also brings the pool down to what it keeps), or, below
-// 8 MiB, with an event that is waited for when the memory is wanted: the
-// synchronisation would take 3 of a small product's 70 us.
+// 8 MiB, with an event that is waited for when the memory is wanted, if there is
+// anything large in the pool: the synchronisation would take 3 of a small
+// product's 70 us, the event takes 1.
 struct CallWorkspace {
   const cudaStream_t st;
   std::optional<Workspace> ws;
