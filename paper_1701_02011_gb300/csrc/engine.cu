@@ -75,8 +75,8 @@ cudaMemPool_t g_pool[64] = {};
 unsigned long long g_pool_ctx[64] = {};
 constexpr unsigned long long kPoolKeep = 1ULL << 30;  // bytes kept between calls
 std::multiset<unsigned long long> g_claims[64];
-// ends of the latest small calls of a device (CallWorkspace), on whatever
-// streams; one is reused after this many calls
+// ends of a device's latest calls on streams other than the legacy one
+// (CallWorkspace); one is reused after this many calls
 constexpr int kMarks = 16;
 cudaEvent_t g_marks[64][kMarks] = {};
 unsigned g_mark[64] = {};
@@ -101,6 +101,10 @@ void scratch_trim() {
   std::lock_guard<std::mutex> lock(g_pool_mu);
   if (cudaMemPool_t pool = live_pool()) {
     cudaGetDevice(&dev);
+    // (an error here: a blocking stream is being captured, which the
+    // synchronisation would spoil)
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(cudaStreamLegacy, &cs) == cudaSuccess) cudaStreamSynchronize(cudaStreamLegacy);
     for (cudaEvent_t e : g_marks[dev])
       if (e) cudaEventSynchronize(e);
     g_large[dev] = false;
@@ -174,17 +178,24 @@ CallWorkspace::~CallWorkspace() {
   ws.reset();
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
-  if (!small) {
-    g_large[dev] = true;
-    cudaStreamSynchronize(st);
-    return;
-  }
-  if (!g_large[dev]) return;
+  if (!small) g_large[dev] = true;
+  const bool legacy = st == nullptr || st == cudaStreamLegacy;
+  if (legacy ? small : !g_large[dev]) return;
   std::lock_guard<std::mutex> lock(g_pool_mu);
-  if (!live_pool()) return;
-  cudaEvent_t& e = g_marks[dev][g_mark[dev]++ % kMarks];
-  if ((!e && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) || cudaEventRecord(e, st) != cudaSuccess)
-    cudaGetLastError();
+  cudaMemPool_t pool = live_pool();
+  if (!pool) return;
+  unsigned long long held = 0, keep = ~0ULL;
+  if (!small) {
+    cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held);
+    cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+  }
+  if (held > keep) {
+    cudaStreamSynchronize(st);
+  } else if (!legacy) {
+    cudaEvent_t& e = g_marks[dev][g_mark[dev]++ % kMarks];
+    if ((!e && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) || cudaEventRecord(e, st) != cudaSuccess)
+      cudaGetLastError();
+  }
 }
 
 void* device_alloc(size_t bytes, const char* what) {

@@ -284,12 +284,13 @@ class ScratchClaim {
   int dev_ = -1;
   unsigned long long bytes_ = 0;
 };
-// Workspace of a call without a handle, on that pool.  The pool can only give
-// back what the host has seen to be free, so a call ends with a synchronisation
-// after its frees (which also brings the pool down to what it keeps), or, below
-// 8 MiB, with an event that is waited for when the memory is wanted, if there is
-// anything large in the pool: the synchronisation would take 3 of a small
-// product's 70 us, the event takes 1.
+// Workspace of a call without a handle, on that pool.  The call synchronises
+// once more after its frees if it took 8 MiB or more and the pool holds more than
+// it keeps.  The pool can only give back what the host has seen to be free: when
+// an allocation fails the legacy stream is synchronised, for calls on it, and
+// events that the calls on other streams leave at their end are waited for (while
+// the pool holds nothing large they leave none).  A synchronisation or an event
+// with every call would take 3 and 1 of a small product's 70 us.
 struct CallWorkspace {
   const cudaStream_t st;
   std::optional<Workspace> ws;

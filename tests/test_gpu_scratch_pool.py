@@ -67,7 +67,8 @@ def test_out_of_memory_gives_back_what_was_taken(lib):
 
 
 @pytest.mark.parametrize("small_call_after", [False, True])
-def test_a_handle_gets_what_the_pool_keeps(lib, small_call_after):
+@pytest.mark.parametrize("own_stream", [False, True])
+def test_a_handle_gets_what_the_pool_keeps(lib, own_stream, small_call_after):
     """0.5 GB of scratch per operand stay in the pool, 0.2 GB are free, and a
     handle's inputs take 0.42 GB; nothing synchronises in between."""
     import numpy as np
@@ -81,9 +82,10 @@ def test_a_handle_gets_what_the_pool_keeps(lib, small_call_after):
     C = torch.zeros((n, n), dtype=torch.float64, device="cuda")
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
-    lib.dsrg_split_gemm(A, A, C, 1.0, 8)
+    st = [torch.cuda.Stream().cuda_stream if own_stream else None for _ in range(2)]
+    lib.dsrg_split_gemm(A, A, C, 1.0, 8, st[0])
     if small_call_after:
-        lib.dsrg_split_gemm(A[:64, :64], A[:64, :64], C[:64, :64], 1.0, 6)
+        lib.dsrg_split_gemm(A[:64, :64], A[:64, :64], C[:64, :64], 1.0, 6, st[1])
     fill = torch.empty(_free(torch) - (200 << 20), dtype=torch.uint8, device="cuda")
     try:
         lib.Dsrg(dev).close()
